@@ -204,6 +204,7 @@ struct gs_frame {
   RowGeom* geom = nullptr;
   uint32_t* tcount = nullptr;
   uint32_t* vals = nullptr;
+  uint16_t* masks = nullptr;  // per instance, the 4 x 4 pixel blocks of its tile (see launch_ranges)
   int2* ranges = nullptr;
   uint32_t* order = nullptr;  // tiles by list length, longest first
   int32_t* last = nullptr;
@@ -308,9 +309,9 @@ gs_status build_lists(gs_scene* sc, gs_frame* f, const char* who, cudaStream_t s
   const int64_t K = Kh;
   if (K >= (int64_t(1) << 31)) return failed(fail(GS_ERR_CAPACITY, std::string(who) + ": more than 2^31 tile instances"));
   f->K = K;
-  uint32_t* keys = tmp.get<uint32_t>(K > 0 ? K : 1, st);
+  uint32_t* keys = f->buf.get<uint32_t>(K > 0 ? K : 1, st);
   uint32_t* vals = f->buf.get<uint32_t>(K > 0 ? K : 1, st);
-  uint32_t* keys2 = tmp.get<uint32_t>(K > 0 ? K : 1, st);
+  uint32_t* keys2 = f->buf.get<uint32_t>(K > 0 ? K : 1, st);
   uint32_t* vals2 = f->buf.get<uint32_t>(K > 0 ? K : 1, st);
   uint32_t* ktmp = tmp.get<uint32_t>(radix_tmp_words(K), st);
   if (!keys || !vals || !keys2 || !vals2 || !ktmp)
@@ -321,7 +322,10 @@ gs_status build_lists(gs_scene* sc, gs_frame* f, const char* who, cudaStream_t s
   GS_CKC(radix_sort_pairs(keys, vals, keys2, vals2, K, bits_for(ntiles), ktmp, &tk, &tv, st));
   f->vals = tv;
   f->buf.release(tv == vals ? vals2 : vals, st);
-  GS_CKC(launch_ranges(tk, K, f->ranges, ntiles, st));
+  // the key buffer that the sort left free holds the block masks
+  f->masks = reinterpret_cast<uint16_t*>(tk == keys ? keys2 : keys);
+  GS_CKC(launch_ranges(tk, tv, K, f->ranges, ntiles, f->geom, rf, cam, f->masks, st));
+  f->buf.release(tk, st);
   if (tile_order_supported(ntiles)) GS_CKC(launch_tile_order(f->ranges, ntiles, f->order, st));
   else f->order = nullptr;  // natural tile order (the buffer stays owned by f->buf)
 #undef GS_CKC
@@ -344,7 +348,7 @@ gs_status blend_forward(gs_scene* sc, gs_frame* f, float* out, int32_t* n_contri
   SegBufs sb;
   sb.lseg = split_lseg(ntiles, f->K, sms);
   if (sb.lseg == 0) {
-    e = launch_blend_fwd(cam, set, f->order, f->rec, f->geom, f->vals, f->ranges, out, n_contrib, f->last, f->med,
+    e = launch_blend_fwd(cam, set, f->order, f->rec, f->masks, f->vals, f->ranges, out, n_contrib, f->last, f->med,
                          f->counters, st);
     return e == cudaSuccess ? GS_OK : cuda_fail(e, "gs_render: blend");
   }
@@ -364,7 +368,7 @@ gs_status blend_forward(gs_scene* sc, gs_frame* f, float* out, int32_t* n_contri
     tmp.release_all(st);
     return fail(GS_ERR_OOM, "gs_render: device allocation failed (segments)");
   }
-  e = launch_blend_fwd_split(cam, set, f->order, f->rec, f->geom, f->vals, f->ranges, out, n_contrib, f->last,
+  e = launch_blend_fwd_split(cam, set, f->order, f->rec, f->masks, f->vals, f->ranges, out, n_contrib, f->last,
                              f->med, f->counters, sb, st);
   tmp.release_all(st);
   return e == cudaSuccess ? GS_OK : cuda_fail(e, "gs_render: blend");
@@ -521,7 +525,7 @@ gs_status gs_contribution(gs_scene* sc, const gs_camera* c, float gamma, float w
   s = build_lists(sc, f, "gs_contribution", st);
   if (s == GS_OK) {
     const bool zero_cand = !view_sum || !view_count;
-    e = launch_contribution(f->cam, to_dev(sc->settings), gamma, weight, f->order, f->rec, f->geom, f->vals,
+    e = launch_contribution(f->cam, to_dev(sc->settings), gamma, weight, f->order, f->rec, f->masks, f->vals,
                             f->ranges, f->cand, f->ncand, n, zero_cand, csum, ccnt, contrib, st);
     if (e != cudaSuccess) s = cuda_fail(e, "gs_contribution");
   }
@@ -654,7 +658,7 @@ gs_status gs_backward(gs_scene* sc, gs_frame* f, const float* const* adj_sets,
   if (e == cudaSuccess) e = cudaMemsetAsync(f->counters + 2, 0, 3 * sizeof(unsigned long long), st);
   const SetDev set = to_dev(sc->settings);
   if (e == cudaSuccess)
-    e = launch_blend_bwd(f->cam, set, f->order, f->rec, f->geom, f->vals, f->ranges, f->out, f->last, f->med, adj,
+    e = launch_blend_bwd(f->cam, set, f->order, f->rec, f->masks, f->vals, f->ranges, f->out, f->last, f->med, adj,
                          grec, screen_grads, n, f->K, f->counters, st);
   if (e == cudaSuccess) e = launch_preprocess_bwd(sc->P, f->cam, f->cand, f->ncand, f->tcount, grec, *grads, st);
   sc->al.put(grec, sizeof(float) * kGradRec * (size_t)(n > 0 ? n : 1), st);

@@ -1,24 +1,32 @@
 // Per-pixel compositing (forward) and its adjoint (reverse replay).
 //
 // Forward (Eq. 1, Sec. 3.1, with the 2DGS surfel model and the low-pass
-// filter of Sec. 3.2): one CTA of 128 threads per 16 x 16 tile; each warp
-// covers an 8 x 8 block of pixels and each thread two pixels of one column,
-// four rows apart, so that an entry read from shared memory serves two
-// pixels and the two per-pixel dependency chains interleave.  The tile's
+// filter of Sec. 3.2): one CTA of 128 threads per 16 x 16 tile; each lane
+// group of eight covers a 4 x 4 block of pixels and each thread two pixels of
+// one column, two rows apart, so that an entry read from shared memory serves
+// two pixels and the two per-pixel dependency chains interleave.  The tile's
 // depth-sorted surfel list is staged through shared memory in batches of
-// 256 entries; while staging, each entry's footprint is tested against the
-// tile's four warp blocks (a conservative cover from the stored footprint
-// shape) and warps skip entries that cannot touch them.  Each pixel
-// intersects its ray with the surfel plane (rho_obj), takes the
-// screen-space filter (rho_scr) where smaller, and composites front to back
-// until the transmittance would drop below T_min.
+// 256 entries; each group walks the entries whose footprint can touch its
+// block (the block masks that launch_ranges made, turned into one index list
+// per group and batch), so the four groups of a warp evaluate four entries
+// side by side.  Each pixel intersects its ray with the surfel plane
+// (rho_obj), takes the screen-space filter (rho_scr) where smaller, and
+// composites front to back until the transmittance would drop below T_min.
 //
 // Backward: the same tiles replay each pixel's list back to front from the
 // final transmittance, T_before = T_after / (1 - alpha), with suffix sums
 // for d L / d alpha.  A thread adds the gradients of its two pixels, the
-// warp reduces them with a reduce-scatter of shuffles (one reduction per 64
-// pixels), the tile sums them in shared memory, and they reach global
-// memory once per (surfel, tile).
+// group reduces them with a reduce-scatter of shuffles (one reduction per
+// four entries and 16 pixels each), the tile sums them in shared memory, and
+// they reach global memory once per (surfel, tile).
+//
+// Both are bound by instruction issue, so the time is (group, entry) steps
+// times instructions per step.  With one list per warp (8 x 8 pixels) only 10
+// (4M-surfel orbit view) to 18 (1M aerial view) of a step's 32 lanes blended
+// anything; 4 x 4 blocks cost a warp the longest of its four lists instead of
+// their union: forward 501 -> 335 us and backward 1160 -> 980 us on a
+// 1M-surfel 1600 x 900 view, 1148 -> 690 us (forward) on a 4M-surfel 1080p
+// view, and 9.6 -> 7.4 ms for the four backwards of a 4M-surfel training step.
 #include <math.h>
 
 #include "gs2d_internal.cuh"
@@ -46,15 +54,16 @@ __device__ __forceinline__ float ex2_approx(float x) {
 constexpr float kNegHalfLog2e = -0.72134752044448170f;  // -log2(e) / 2
 
 // Pixels of thread t within its tile: warp w covers columns 8 (w & 1) .. +7
-// and rows 8 (w >> 1) .. +7; lane l takes column l & 7 and rows l >> 3 and
-// (l >> 3) + 4 of that block.
-__device__ __forceinline__ int local_x(int t) { return (((t >> 5) & 1) << 3) | (t & 7); }
-__device__ __forceinline__ int local_y(int t) { return ((t >> 6) << 3) | ((t >> 3) & 3); }
+// and rows 8 (w >> 1) .. +7, its lane group g = (l >> 3) the 4 x 4 block at
+// column 4 (g & 1), row 4 (g >> 1) of those, and lane l column l & 3 and rows
+// (l >> 2) & 1 and that + kRowStep of the group's block.
+constexpr int kRowStep = 2;  // rows between a thread's two pixels
+__device__ __forceinline__ int local_x(int t) { return (((t >> 5) & 1) << 3) | (((t >> 3) & 1) << 2) | (t & 3); }
+__device__ __forceinline__ int local_y(int t) { return ((t >> 6) << 3) | (((t >> 4) & 1) << 2) | ((t >> 2) & 1); }
 
 // Staged entry: s0 = (c.x, c.y relative to the tile origin, e.x, e.y),
 // s1 = Jh, s2 = (p_z, opacity, r, g), s3 = (b, n.x, n.y, n.z), s4 = Jl,
-// s5 = (nu0h, nv0h, nu0l, nv0l); wmask bit w set when the footprint may
-// reach warp w's pixel block.
+// s5 = (nu0h, nv0h, nu0l, nv0l).
 //
 // Tile-relative ray-splat coordinates.  For a pixel at offset (lx, ly) from
 // the tile origin o, Ji d = Ji (o - c) + Ji (lx, ly) = n0 + Ji (lx, ly).  Held
@@ -76,13 +85,9 @@ __device__ __forceinline__ int local_y(int t) { return ((t >> 6) << 3) | ((t >> 
 // FP32 rounding of the result itself, whatever the conditioning of Ji.
 struct Staged {
   float4 s0, s1, s2, s3, s4, s5;
-  uint32_t wmask;
 };
 
-
-__device__ __forceinline__ Staged stage_entry(const float4* __restrict__ rec,
-                                              const RowGeom* __restrict__ geom, uint32_t s,
-                                              int tx0, int ty0, int H, float rf) {
+__device__ __forceinline__ Staged stage_entry(const float4* __restrict__ rec, uint32_t s, int tx0, int ty0) {
   const float4* R = rec + (size_t)s * kRecF4;
   const float4 r0 = R[0], r1 = R[1], r2 = R[2], r3 = R[3], r4 = R[4], r5 = R[5], r6 = R[6];
   Staged e;
@@ -106,36 +111,44 @@ __device__ __forceinline__ Staged stage_entry(const float4* __restrict__ rec,
   const float lv = __fmaf_rn(r5.z, dox, __fmaf_rn(r5.w, doy, r6.y));
   const float qu = __fmul_rn(rintf(__fmul_rn(lu, ug)), dg), qv = __fmul_rn(rintf(__fmul_rn(lv, ug)), dg);
   e.s5 = make_float4(__fadd_rn(hu, qu), __fadd_rn(hv, qv), __fsub_rn(lu, qu), __fsub_rn(lv, qv));
-  const RowGeom g = geom[s];
-  uint32_t m = 0u;
-#pragma unroll
-  for (int b = 0; b < 2; ++b) {
-    const int ja = ty0 + 8 * b;
-    if (ja >= H) break;
-    int ilo, ihi;
-    if (!band_pixels(g, ja, min(ja + 7, H - 1), rf, &ilo, &ihi)) continue;
-    if (ilo <= tx0 + 7 && ihi >= tx0) m |= 1u << (2 * b);
-    if (ilo <= tx0 + 15 && ihi >= tx0 + 8) m |= 1u << (2 * b + 1);
-  }
-  e.wmask = m;
   return e;
 }
 
-// Per warp, the batch's entries whose footprint may reach the warp's pixel
-// block, as kBatch / 32 bit words (ballots of the staged masks); the loops
-// below visit only their set bits, so entries that miss the block cost
-// nothing (long lists, where most entries miss a given block).
-constexpr int kWords = kBatch / 32;
-template <int NW = kWords>
-__device__ __forceinline__ void warp_entry_bits(const uint32_t* sm, int nb, int warp, int lane,
-                                                uint32_t* wb) {
+// Per lane group of eight, the batch's entries whose footprint may reach the
+// group's 4 x 4 pixel block, as a list of indices into the batch: the four
+// groups of a warp walk their own lists side by side, so an entry costs a
+// group nothing where it misses the group's block.
+// sm holds the entries' block masks (bit 4 w + g); entry e is listed for a
+// group only below the group's limit.  Returns the length of the caller's
+// group's list.
+template <int NB>
+__device__ __forceinline__ int group_lists(const uint16_t* sm, int nb, int warp, int lane, uint8_t (*list)[NB],
+                                           int limit = NB) {
+  const uint32_t lt = (1u << lane) - 1u;
+  int base[4] = {0, 0, 0, 0}, lim[4];
 #pragma unroll
-  for (int j = 0; j < NW; ++j) {
+  for (int g = 0; g < 4; ++g) lim[g] = min(__shfl_sync(0xffffffffu, limit, 8 * g), nb);
+#pragma unroll
+  for (int j = 0; j < NB / 32; ++j) {
     const int e = 32 * j + lane;
-    const uint32_t w = __ballot_sync(0xffffffffu, e < nb && ((sm[e] >> warp) & 1u));
-    if (lane == 0) wb[j] = w;
+    const uint32_t m = e < nb ? (uint32_t)sm[e] >> (4 * warp) : 0u;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const bool in = ((m >> g) & 1u) && e < lim[g];
+      const uint32_t b = __ballot_sync(0xffffffffu, in);
+      if (in) list[g][base[g] + __popc(b & lt)] = (uint8_t)e;
+      base[g] += __popc(b);
+    }
   }
   __syncwarp();
+  const int g = lane >> 3;
+  return g == 0 ? base[0] : (g == 1 ? base[1] : (g == 2 ? base[2] : base[3]));
+}
+
+// The longest of the four groups' lists.
+__device__ __forceinline__ int warp_longest(int n) {
+  n = max(n, __shfl_xor_sync(0xffffffffu, n, 8));
+  return max(n, __shfl_xor_sync(0xffffffffu, n, 16));
 }
 
 struct Pair {
@@ -170,19 +183,19 @@ __device__ __forceinline__ void finish_pair(float lx, float ly, float4 s0, float
   q.hit = (q.rho <= set.rho_max) && (q.alpha >= set.alpha_min);
 }
 
-// One entry against a thread's two pixels, (lx, ly) and (lx, ly + 4) from
-// the tile origin: the exact grid sums nu0h + Jh (lx, ly) (row B adds 4 Jh
-// exactly), plus the small low-part corrections (see Staged).
+// One entry against a thread's two pixels, (lx, ly) and (lx, ly + kRowStep)
+// from the tile origin: the exact grid sums nu0h + Jh (lx, ly) (row B adds
+// kRowStep Jh exactly), plus the small low-part corrections (see Staged).
 __device__ __forceinline__ void eval_two(float lx, float ly, float4 s0, float4 jh, float4 jl, float4 n0,
                                          float opac, const SetDev& set, Pair& qa, Pair& qb) {
   const float suA = __fmaf_rn(jh.x, lx, __fmaf_rn(jh.y, ly, n0.x));
   const float svA = __fmaf_rn(jh.z, lx, __fmaf_rn(jh.w, ly, n0.y));
   const float cuA = __fmaf_rn(jl.x, lx, __fmaf_rn(jl.y, ly, n0.z));
   const float cvA = __fmaf_rn(jl.z, lx, __fmaf_rn(jl.w, ly, n0.w));
-  const float suB = __fmaf_rn(jh.y, 4.f, suA), svB = __fmaf_rn(jh.w, 4.f, svA);
-  const float cuB = __fmaf_rn(jl.y, 4.f, cuA), cvB = __fmaf_rn(jl.w, 4.f, cvA);
+  const float suB = __fmaf_rn(jh.y, (float)kRowStep, suA), svB = __fmaf_rn(jh.w, (float)kRowStep, svA);
+  const float cuB = __fmaf_rn(jl.y, (float)kRowStep, cuA), cvB = __fmaf_rn(jl.w, (float)kRowStep, cvA);
   finish_pair(lx, ly, s0, __fadd_rn(suA, cuA), __fadd_rn(svA, cvA), opac, set, qa);
-  finish_pair(lx, __fadd_rn(ly, 4.f), s0, __fadd_rn(suB, cuB), __fadd_rn(svB, cvB), opac, set, qb);
+  finish_pair(lx, __fadd_rn(ly, (float)kRowStep), s0, __fadd_rn(suB, cuB), __fadd_rn(svB, cvB), opac, set, qb);
 }
 
 // ---------------------------------------------------------------------------
@@ -270,21 +283,40 @@ __device__ __forceinline__ void fwd_store(const FwdPix& p, const CamDev& cam, co
 // Shared-memory staging area of one CTA.
 struct FwdSmem {
   float4 s0[kBatch], s1[kBatch], s2[kBatch], s3[kBatch], s4[kBatch], s5[kBatch];
-  uint32_t sm[kBatch];
-  uint32_t wbits[kThreads / 32][kWords];
+  uint16_t sm[kBatch];
+  uint8_t list[kThreads / 32][4][kBatch];
   unsigned long long tot[2];
 };
 
+// Stage nb entries of a tile's list from position base on (the entries that
+// reach no pixel block of the tile leave their slot as it is: no list has it).
+__device__ __forceinline__ void stage_batch(FwdSmem& sh, const float4* __restrict__ rec,
+                                            const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals,
+                                            int base, int nb, int tx0, int ty0) {
+  for (int t = threadIdx.x; t < nb; t += kThreads) {
+    const uint16_t m = masks[base + t];
+    sh.sm[t] = m;
+    if (m == 0u) continue;
+    const Staged e = stage_entry(rec, vals[base + t], tx0, ty0);
+    sh.s0[t] = e.s0;
+    sh.s1[t] = e.s1;
+    sh.s2[t] = e.s2;
+    sh.s3[t] = e.s3;
+    sh.s4[t] = e.s4;
+    sh.s5[t] = e.s5;
+  }
+}
+
 // Forward blend of tile (bx, by) of one view by the whole CTA.
 __device__ __forceinline__ void blend_fwd_tile(
-    FwdSmem& sh, const CamDev& cam, const SetDev& set, float rf, const float4* __restrict__ rec,
-    const RowGeom* __restrict__ geom, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
+    FwdSmem& sh, const CamDev& cam, const SetDev& set, const float4* __restrict__ rec,
+    const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
     float* __restrict__ out, int32_t* __restrict__ n_contrib, int32_t* __restrict__ last,
     int32_t* __restrict__ med, unsigned long long* __restrict__ counters, int bx, int by, int lseg = 0) {
   const int tile = by * cam.tiles_x + bx;
   const int tx0 = bx * kTile, ty0 = by * kTile;
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
-  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + 4;
+  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
   const int warp = threadIdx.x >> 5;
   const float lx = (float)lxi + 0.5f, lyA = (float)lyi + 0.5f;
   const int2 rg = ranges[tile];
@@ -295,32 +327,18 @@ __device__ __forceinline__ void blend_fwd_tile(
   fwd_init(b, px < cam.W && pyB < cam.H);
   for (int b0 = 0; b0 < len; b0 += kBatch) {
     if (__syncthreads_count(a.done && b.done) == kThreads) break;
-    for (int t = threadIdx.x; t < kBatch; t += kThreads) {
-      if (b0 + t < len) {
-        const Staged e = stage_entry(rec, geom, vals[rg.x + b0 + t], tx0, ty0, cam.H, rf);
-        sh.s0[t] = e.s0;
-        sh.s1[t] = e.s1;
-        sh.s2[t] = e.s2;
-        sh.s3[t] = e.s3;
-        sh.s4[t] = e.s4;
-        sh.s5[t] = e.s5;
-        sh.sm[t] = e.wmask;
-      }
-    }
-    __syncthreads();
     const int nb = min(kBatch, len - b0);
-    warp_entry_bits(sh.sm, nb, warp, threadIdx.x & 31, sh.wbits[warp]);
-    for (int j = 0; j < kWords && !(a.done && b.done); ++j) {
-      uint32_t bits = sh.wbits[warp][j];
-      while (bits != 0u && !(a.done && b.done)) {
-        const int k = 32 * j + __ffs(bits) - 1;
-        bits &= bits - 1u;
-        const float4 e0 = sh.s0[k], e1 = sh.s1[k], e2 = sh.s2[k], e3 = sh.s3[k];
-        Pair qa, qb;
-        eval_two(lx, lyA, e0, e1, sh.s4[k], sh.s5[k], e2.y, set, qa, qb);
-        fwd_step(a, qa, e2, e3, b0 + k, set);
-        fwd_step(b, qb, e2, e3, b0 + k, set);
-      }
+    stage_batch(sh, rec, masks, vals, rg.x + b0, nb, tx0, ty0);
+    __syncthreads();
+    const int glen = group_lists<kBatch>(sh.sm, nb, warp, threadIdx.x & 31, sh.list[warp]);
+    const uint8_t* list = sh.list[warp][(threadIdx.x & 31) >> 3];
+    for (int i = 0; i < glen && !(a.done && b.done); ++i) {
+      const int k = list[i];
+      const float4 e0 = sh.s0[k], e1 = sh.s1[k], e2 = sh.s2[k], e3 = sh.s3[k];
+      Pair qa, qb;
+      eval_two(lx, lyA, e0, e1, sh.s4[k], sh.s5[k], e2.y, set, qa, qb);
+      fwd_step(a, qa, e2, e3, b0 + k, set);
+      fwd_step(b, qb, e2, e3, b0 + k, set);
     }
   }
   fwd_store(a, cam, set, px, pyA, out, n_contrib, last, med);
@@ -350,13 +368,13 @@ __device__ __forceinline__ void blend_fwd_tile(
 
 // One CTA per tile; block b takes tile order[b] (longest lists first).
 __global__ void __launch_bounds__(kThreads, 5) blend_fwd_kernel(
-    CamDev cam, SetDev set, float rf, const uint32_t* __restrict__ order, const float4* __restrict__ rec,
-    const RowGeom* __restrict__ geom, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
+    CamDev cam, SetDev set, const uint32_t* __restrict__ order, const float4* __restrict__ rec,
+    const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
     float* __restrict__ out, int32_t* __restrict__ n_contrib, int32_t* __restrict__ last,
     int32_t* __restrict__ med, unsigned long long* __restrict__ counters, int lseg) {
   __shared__ FwdSmem sh;
   const int t = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
-  blend_fwd_tile(sh, cam, set, rf, rec, geom, vals, ranges, out, n_contrib, last, med, counters,
+  blend_fwd_tile(sh, cam, set, rec, masks, vals, ranges, out, n_contrib, last, med, counters,
                  t % cam.tiles_x, t / cam.tiles_x, lseg);
 }
 
@@ -399,26 +417,8 @@ __device__ __forceinline__ bool seg_of(const uint32_t* seg_tile, const uint32_t*
   return true;
 }
 
-// Stage entries [b0, b0 + nb) of the tile's list (shared by the segment kernels).
-__device__ __forceinline__ void stage_batch(FwdSmem& sh, const float4* __restrict__ rec,
-                                            const RowGeom* __restrict__ geom, const uint32_t* __restrict__ vals,
-                                            int base, int nb, int tx0, int ty0, int H, float rf) {
-  for (int t = threadIdx.x; t < kBatch; t += kThreads) {
-    if (t < nb) {
-      const Staged e = stage_entry(rec, geom, vals[base + t], tx0, ty0, H, rf);
-      sh.s0[t] = e.s0;
-      sh.s1[t] = e.s1;
-      sh.s2[t] = e.s2;
-      sh.s3[t] = e.s3;
-      sh.s4[t] = e.s4;
-      sh.s5[t] = e.s5;
-      sh.sm[t] = e.wmask;
-    }
-  }
-}
-
 __global__ void __launch_bounds__(kThreads) seg_trans_kernel(
-    CamDev cam, SetDev set, float rf, const float4* __restrict__ rec, const RowGeom* __restrict__ geom,
+    CamDev cam, SetDev set, const float4* __restrict__ rec, const uint16_t* __restrict__ masks,
     const uint32_t* __restrict__ vals, const int2* __restrict__ ranges, int lseg,
     const uint32_t* __restrict__ seg_tile, const uint32_t* __restrict__ seg_idx, const uint32_t* __restrict__ nseg,
     float* __restrict__ trans) {
@@ -435,20 +435,17 @@ __global__ void __launch_bounds__(kThreads) seg_trans_kernel(
   for (int b0 = e0; b0 < e1; b0 += kBatch) {
     const int nb = min(kBatch, e1 - b0);
     __syncthreads();
-    stage_batch(sh, rec, geom, vals, rg.x + b0, nb, tx0, ty0, cam.H, rf);
+    stage_batch(sh, rec, masks, vals, rg.x + b0, nb, tx0, ty0);
     __syncthreads();
-    warp_entry_bits(sh.sm, nb, warp, threadIdx.x & 31, sh.wbits[warp]);
-    for (int j = 0; j < kWords; ++j) {
-      uint32_t bits = sh.wbits[warp][j];
-      while (bits != 0u) {
-        const int k = 32 * j + __ffs(bits) - 1;
-        bits &= bits - 1u;
-        const float4 f0 = sh.s0[k], f1 = sh.s1[k], f2 = sh.s2[k];
-        Pair qa, qb;
-        eval_two(lx, lyA, f0, f1, sh.s4[k], sh.s5[k], f2.y, set, qa, qb);
-        TA = qa.hit ? TA * (1.f - qa.alpha) : TA;
-        TB = qb.hit ? TB * (1.f - qb.alpha) : TB;
-      }
+    const int glen = group_lists<kBatch>(sh.sm, nb, warp, threadIdx.x & 31, sh.list[warp]);
+    const uint8_t* list = sh.list[warp][(threadIdx.x & 31) >> 3];
+    for (int i = 0; i < glen; ++i) {
+      const int k = list[i];
+      const float4 f0 = sh.s0[k], f1 = sh.s1[k], f2 = sh.s2[k];
+      Pair qa, qb;
+      eval_two(lx, lyA, f0, f1, sh.s4[k], sh.s5[k], f2.y, set, qa, qb);
+      TA = qa.hit ? TA * (1.f - qa.alpha) : TA;
+      TB = qb.hit ? TB * (1.f - qb.alpha) : TB;
     }
   }
   trans[(size_t)blockIdx.x * kTilePix + threadIdx.x] = TA;
@@ -465,7 +462,7 @@ __device__ __forceinline__ void seg_store(const FwdPix& p, bool inside, SegPart*
 }
 
 __global__ void __launch_bounds__(kThreads) seg_blend_kernel(
-    CamDev cam, SetDev set, float rf, const float4* __restrict__ rec, const RowGeom* __restrict__ geom,
+    CamDev cam, SetDev set, const float4* __restrict__ rec, const uint16_t* __restrict__ masks,
     const uint32_t* __restrict__ vals, const int2* __restrict__ ranges, int lseg,
     const uint32_t* __restrict__ seg_tile, const uint32_t* __restrict__ seg_idx, const uint32_t* __restrict__ nseg,
     const float* __restrict__ trans, SegPart* __restrict__ part, unsigned long long* __restrict__ counters) {
@@ -474,7 +471,7 @@ __global__ void __launch_bounds__(kThreads) seg_blend_kernel(
   if (!seg_of(seg_tile, seg_idx, nseg, blockIdx.x, &tile, &s)) return;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
-  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + 4;
+  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
   const int warp = threadIdx.x >> 5;
   const float lx = (float)lxi + 0.5f, lyA = (float)lyi + 0.5f;
   const int2 rg = ranges[tile];
@@ -495,20 +492,17 @@ __global__ void __launch_bounds__(kThreads) seg_blend_kernel(
   for (int b0 = e0; b0 < e1; b0 += kBatch) {
     if (__syncthreads_count(a.done && b.done) == kThreads) break;
     const int nb = min(kBatch, e1 - b0);
-    stage_batch(sh, rec, geom, vals, rg.x + b0, nb, tx0, ty0, cam.H, rf);
+    stage_batch(sh, rec, masks, vals, rg.x + b0, nb, tx0, ty0);
     __syncthreads();
-    warp_entry_bits(sh.sm, nb, warp, threadIdx.x & 31, sh.wbits[warp]);
-    for (int j = 0; j < kWords && !(a.done && b.done); ++j) {
-      uint32_t bits = sh.wbits[warp][j];
-      while (bits != 0u && !(a.done && b.done)) {
-        const int k = 32 * j + __ffs(bits) - 1;
-        bits &= bits - 1u;
-        const float4 f0 = sh.s0[k], f1 = sh.s1[k], f2 = sh.s2[k], f3 = sh.s3[k];
-        Pair qa, qb;
-        eval_two(lx, lyA, f0, f1, sh.s4[k], sh.s5[k], f2.y, set, qa, qb);
-        fwd_step<true>(a, qa, f2, f3, b0 + k, set);
-        fwd_step<true>(b, qb, f2, f3, b0 + k, set);
-      }
+    const int glen = group_lists<kBatch>(sh.sm, nb, warp, threadIdx.x & 31, sh.list[warp]);
+    const uint8_t* list = sh.list[warp][(threadIdx.x & 31) >> 3];
+    for (int i = 0; i < glen && !(a.done && b.done); ++i) {
+      const int k = list[i];
+      const float4 f0 = sh.s0[k], f1 = sh.s1[k], f2 = sh.s2[k], f3 = sh.s3[k];
+      Pair qa, qb;
+      eval_two(lx, lyA, f0, f1, sh.s4[k], sh.s5[k], f2.y, set, qa, qb);
+      fwd_step<true>(a, qa, f2, f3, b0 + k, set);
+      fwd_step<true>(b, qb, f2, f3, b0 + k, set);
     }
   }
   SegPart* pp = part + (size_t)blockIdx.x * kTilePix;
@@ -570,7 +564,7 @@ __global__ void __launch_bounds__(kThreads) seg_merge_kernel(
   if (!seg_of(seg_tile, seg_idx, nseg, blockIdx.x, &tile, &s) || s != 0) return;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
-  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + 4;
+  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
   const int2 rg = ranges[tile];
   const float zref = rec[(size_t)vals[rg.x] * kRecF4 + 2].z;
   const int ns = (int)segcnt[tile];
@@ -616,7 +610,7 @@ __global__ void __launch_bounds__(kThreads) blend_fwd_batched_kernel(BlendBatch 
     while (j + 1 < batch.njobs && batch.job[j + 1].tile_begin <= t) ++j;
     const BlendJob& jb = batch.job[j];
     const int local = t - jb.tile_begin;
-    blend_fwd_tile(sh, jb.cam, jb.set, jb.rf, jb.rec, jb.geom, jb.vals, jb.ranges, jb.out, jb.n_contrib,
+    blend_fwd_tile(sh, jb.cam, jb.set, jb.rec, jb.masks, jb.vals, jb.ranges, jb.out, jb.n_contrib,
                    nullptr, nullptr, batch.work, local % jb.cam.tiles_x, local / jb.cam.tiles_x);
   }
 }
@@ -655,11 +649,13 @@ struct Layout {
   static constexpr int kN = kRec + 2 * kMaxSets;  // 18 or 21
 };
 
-// Balanced reduce-scatter of N values over the warp: at each halving level
-// the lanes whose bit is clear keep the first ceil(N/2) values and the others
-// the rest, exchanging the halves they do not keep; N values need about
-// N + 5 shuffles.  Afterwards v[0] holds the warp sum of one slot, given by
-// rs_slot() for the lane (or nothing when rs_slot() returns -1).
+// Balanced reduce-scatter of N values over a lane group of eight: at each
+// halving level the lanes whose bit is clear keep the first ceil(N/2) values
+// and the others the rest, exchanging the halves they do not keep (17
+// shuffles for 18 values, and the warp's four groups reduce four entries at
+// once).  Afterwards v[0 .. kRsMax) holds the group's sums of the slots
+// given by rs_slots() for the lane.
+constexpr int kGroup = 8;
 template <int O, int N>
 __device__ __forceinline__ void rs_level(float* v, int lane) {
   constexpr int L = (N + 1) / 2, H = N - L;
@@ -674,10 +670,13 @@ __device__ __forceinline__ void rs_level(float* v, int lane) {
   if constexpr (O > 1) rs_level<O / 2, L>(v, lane);
 }
 
+constexpr int rs_max(int n) { return ((n + 1) / 2 + 1) / 2 / 2 + ((((n + 1) / 2 + 1) / 2) & 1); }
+
+// The lane's slots after the reduce-scatter: *n of them from the returned one.
 template <int N>
-__device__ __forceinline__ int rs_slot(int lane) {
+__device__ __forceinline__ int rs_slots(int lane, int* count) {
   int n = N, real = N, slot = 0;
-  for (int o = 16; o >= 1; o >>= 1) {
+  for (int o = kGroup / 2; o >= 1; o >>= 1) {
     const int L = (n + 1) / 2;
     if (lane & o) {
       slot += L;
@@ -687,7 +686,8 @@ __device__ __forceinline__ int rs_slot(int lane) {
     }
     n = L;
   }
-  return real > 0 ? slot : -1;
+  *count = real;
+  return slot;
 }
 
 // Per-pixel state of the reverse replay: transmittance, suffix sums S of
@@ -847,21 +847,23 @@ __device__ __forceinline__ void bwd_pair(BwdPix& p, const Pair& q, float4 e0, fl
 template <int kAcc, int kBB>
 struct BwdSmem {
   float4 s0[kBB], s1[kBB], s2[kBB], s3[kBB], s4[kBB], s5[kBB];
-  uint32_t sm[kBB];
+  uint16_t sm[kBB];
   uint32_t sid[kBB];
   float acc[kBB][kAcc];
-  uint32_t wbits[kThreads / 32][kBB / 32];
+  uint8_t list[kThreads / 32][4][kBB];
   int smax;
 };
 
-// Reverse replay of entry kk (list position k) for a thread's two pixels:
-// the pair's gradients, reduced over the warp into the entry's accumulator.
+// Reverse replay of entry kk of the batch (list position k) for a thread's two
+// pixels, each lane group its own entry: the pairs' gradients, reduced over
+// the group into the entry's accumulator.  active is false for the lanes of a
+// group whose list is used up.
 template <bool kLoss, int kN, int kAcc, int kBB>
-__device__ __forceinline__ void bwd_entry(BwdSmem<kAcc, kBB>& sh, int kk, int k, float lx, float ly, BwdPix& a,
-                                          BwdPix& b, int nsets, const SetDev& set, int lane, int myslot,
-                                          unsigned& wentries, unsigned& wlanes) {
+__device__ __forceinline__ void bwd_entry(BwdSmem<kAcc, kBB>& sh, bool active, int kk, int k, float lx, float ly,
+                                          BwdPix& a, BwdPix& b, int nsets, const SetDev& set, int lane, int myslot,
+                                          int nslots, unsigned& wentries, unsigned& wlanes) {
   const float4 e0 = sh.s0[kk], jh = sh.s1[kk], e2 = sh.s2[kk];
-  const bool liveA = k < a.last, liveB = k < b.last;
+  const bool liveA = active && k < a.last, liveB = active && k < b.last;
   Pair qa, qb;
   const float4 jl = sh.s4[kk];
   eval_two(lx, ly, e0, jh, jl, sh.s5[kk], e2.y, set, qa, qb);
@@ -878,26 +880,14 @@ __device__ __forceinline__ void bwd_entry(BwdSmem<kAcc, kBB>& sh, int kk, int k,
   const float4 e3 = sh.s3[kk];
   // Ji = Jh + Jl (FP32) for the chain rule
   const float4 e1 = make_float4(jh.x + jl.x, jh.y + jl.y, jh.z + jl.z, jh.w + jl.w);
-  // a pixel row with no hit in the whole warp needs no gradient pass (a
-  // masked pair leaves the pixel's state and the sums unchanged)
-  const bool anyA = __any_sync(0xffffffffu, qa.hit), anyB = __any_sync(0xffffffffu, qb.hit);
-  if (anyA && anyB) {
-    bwd_pair<kLoss>(a, qa, e0, e1, e2, e3, k, nsets, set, v);
-    bwd_pair<kLoss>(b, qb, e0, e1, e2, e3, k, nsets, set, v);
-  } else if (anyA) {
-    bwd_pair<kLoss>(a, qa, e0, e1, e2, e3, k, nsets, set, v);
-  } else {
-    bwd_pair<kLoss>(b, qb, e0, e1, e2, e3, k, nsets, set, v);
-  }
-  if (__popc(ballot) == 1) {
-    if (contrib) {
+  bwd_pair<kLoss>(a, qa, e0, e1, e2, e3, k, nsets, set, v);
+  bwd_pair<kLoss>(b, qb, e0, e1, e2, e3, k, nsets, set, v);
+  rs_level<kGroup / 2, kN>(v, lane);
+  if ((ballot >> (lane & 24)) & 0xffu) {
+    constexpr int kM = rs_max(kN);
 #pragma unroll
-      for (int i = 0; i < kN; ++i)
-        if (v[i] != 0.f) atomicAdd(&sh.acc[kk][i], v[i]);
-    }
-  } else {
-    rs_level<16, kN>(v, lane);
-    if (myslot >= 0 && v[0] != 0.f) atomicAdd(&sh.acc[kk][myslot], v[0]);
+    for (int i = 0; i < kM; ++i)
+      if (i < nslots && v[i] != 0.f) atomicAdd(&sh.acc[kk][myslot + i], v[i]);
   }
 }
 
@@ -905,27 +895,28 @@ __device__ __forceinline__ void bwd_entry(BwdSmem<kAcc, kBB>& sh, int kk, int k,
 // registers; 4: up to 128, for dense lists of small footprints).
 template <bool kLoss, int kMinCtas>
 __global__ void __launch_bounds__(kThreads, kMinCtas) blend_bwd_kernel(
-    CamDev cam, SetDev set, float rf, const uint32_t* __restrict__ order, const float4* __restrict__ rec,
-    const RowGeom* __restrict__ geom, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
+    CamDev cam, SetDev set, const uint32_t* __restrict__ order, const float4* __restrict__ rec,
+    const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
     const float* __restrict__ out, const int32_t* __restrict__ last, const int32_t* __restrict__ med,
     AdjDev adj, float* __restrict__ grec, float* __restrict__ screen, int n,
     unsigned long long* __restrict__ counters) {
   using LY = Layout<kLoss>;
   constexpr int kN = LY::kN;
   constexpr int kAcc = kN | 1;  // odd row stride: the flush's column reads are conflict-free
-  constexpr int kBatchB = batch_b(kMinCtas), kWordsB = kBatchB / 32;
+  constexpr int kBatchB = batch_b(kMinCtas);
   __shared__ BwdSmem<kAcc, kBatchB> sh;
   const int tile = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
-  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + 4;
+  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
   const int warp = threadIdx.x >> 5;
   const float lx = (float)lxi + 0.5f, lyA = (float)lyi + 0.5f;
   const int2 rg = ranges[tile];
   const size_t HW = (size_t)cam.W * cam.H;
   const int lane = threadIdx.x & 31;
   const int nsets = adj.n_sets;
-  const int myslot = rs_slot<kN>(lane);
+  int nslots;
+  const int myslot = rs_slots<kN>(lane, &nslots);
   const bool inA = px < cam.W && pyA < cam.H, inB = px < cam.W && pyB < cam.H;
   BwdPix a, b;
   bwd_init<kLoss>(a, inA, inA ? (size_t)pyA * cam.W + px : 0, HW, out, last, med, adj, set);
@@ -935,11 +926,11 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) blend_bwd_kernel(
   atomicMax(&sh.smax, max(a.last, b.last));
   __syncthreads();
   const int maxlast = sh.smax;
-  // the warp's own last blended position: entries behind it are dead for all
-  // of its pixels and are not visited
-  int wlast = max(a.last, b.last);
+  // the lane group's own last blended position: entries behind it are dead for
+  // all of its pixels and are not visited
+  int glast = max(a.last, b.last);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) wlast = max(wlast, __shfl_xor_sync(0xffffffffu, wlast, o));
+  for (int o = kGroup / 2; o > 0; o >>= 1) glast = max(glast, __shfl_xor_sync(0xffffffffu, glast, o));
   unsigned replayed = 0, wentries = 0, wlanes = 0;
 
   for (int bend = maxlast; bend > 0; bend -= kBatchB) {
@@ -947,47 +938,39 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) blend_bwd_kernel(
     const int nb = bend - b0;
     __syncthreads();
     for (int t = threadIdx.x; t < nb; t += kThreads) {
+      // every entry, also one that reaches no block: a group whose list is
+      // used up evaluates entry 0 with its pairs masked
       const uint32_t s = vals[rg.x + b0 + t];
       sh.sid[t] = s;
-      const Staged e = stage_entry(rec, geom, s, tx0, ty0, cam.H, rf);
+      sh.sm[t] = masks[rg.x + b0 + t];
+      const Staged e = stage_entry(rec, s, tx0, ty0);
       sh.s0[t] = e.s0;
       sh.s1[t] = e.s1;
       sh.s2[t] = e.s2;
       sh.s3[t] = e.s3;
       sh.s4[t] = e.s4;
       sh.s5[t] = e.s5;
-      sh.sm[t] = e.wmask;
     }
     for (int i = threadIdx.x; i < nb * kAcc; i += kThreads) (&sh.acc[0][0])[i] = 0.f;
     __syncthreads();
-    warp_entry_bits<kWordsB>(sh.sm, nb, warp, lane, sh.wbits[warp]);
-    if (lane == 0) {
-#pragma unroll
-      for (int j = 0; j < kWordsB; ++j) {
-        const int lw = wlast - b0 - 32 * j;
-        sh.wbits[warp][j] &= lw >= 32 ? 0xffffffffu : (lw > 0 ? (1u << lw) - 1u : 0u);
-      }
-    }
-    __syncwarp();
+    const int glen = group_lists<kBatchB>(sh.sm, nb, warp, lane, sh.list[warp], max(glast - b0, 0));
+    const uint8_t* list = sh.list[warp][lane >> 3];
     if (counters) {
-      // the batch's entries before each pixel's last blended one that the
-      // warp visits (performance counter)
-#pragma unroll
-      for (int j = 0; j < kWordsB; ++j) {
-        const uint32_t bits = sh.wbits[warp][j];
-        const int la = a.last - b0 - 32 * j, lb = b.last - b0 - 32 * j;
-        replayed += (unsigned)__popc(la >= 32 ? bits : (la > 0 ? bits & ((1u << la) - 1u) : 0u));
-        replayed += (unsigned)__popc(lb >= 32 ? bits : (lb > 0 ? bits & ((1u << lb) - 1u) : 0u));
+      // the batch's entries before each pixel's last blended one that its
+      // group visits (performance counter)
+      for (int i = 0; i < glen; ++i) {
+        const int k = b0 + list[i];
+        replayed += (k < a.last ? 1u : 0u) + (k < b.last ? 1u : 0u);
       }
     }
-    for (int j = kWordsB - 1; j >= 0; --j) {
-      uint32_t bits = sh.wbits[warp][j];
-      while (bits != 0u) {  // back to front: highest set bit first
-        const int hb = 31 - __clz(bits);
-        bits &= ~(1u << hb);
-        bwd_entry<kLoss, kN, kAcc, kBatchB>(sh, 32 * j + hb, b0 + 32 * j + hb, lx, lyA, a, b, nsets, set, lane, myslot,
-                                   wentries, wlanes);
-      }
+    // back to front, the groups side by side: a group whose list is used up
+    // takes part in the warp's votes and shuffles without a pair
+    const int longest = warp_longest(glen);
+    for (int i = 1; i <= longest; ++i) {
+      const bool active = i <= glen;
+      const int kk = active ? list[glen - i] : 0;
+      bwd_entry<kLoss, kN, kAcc, kBatchB>(sh, active, kk, b0 + kk, lx, lyA, a, b, nsets, set, lane, myslot, nslots,
+                                          wentries, wlanes);
     }
     __syncthreads();
     // flush this batch: one (surfel, tile) gradient record per entry, the
@@ -1058,18 +1041,19 @@ __device__ __forceinline__ float contrib_step(float& T, bool& stopped, const Pai
 }
 
 __global__ void __launch_bounds__(kThreads) blend_contrib_kernel(
-    CamDev cam, SetDev set, float rf, float gamma, const uint32_t* __restrict__ order,
-    const float4* __restrict__ rec, const RowGeom* __restrict__ geom, const uint32_t* __restrict__ vals,
+    CamDev cam, SetDev set, float gamma, const uint32_t* __restrict__ order,
+    const float4* __restrict__ rec, const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals,
     const int2* __restrict__ ranges, float* __restrict__ csum, uint32_t* __restrict__ ccnt) {
   __shared__ float4 s0[kBatch], s1[kBatch], s2[kBatch], s4[kBatch], s5[kBatch];
-  __shared__ uint32_t sm[kBatch], sid[kBatch];
+  __shared__ uint32_t sid[kBatch];
+  __shared__ uint16_t sm[kBatch];
   __shared__ float asum[kBatch];
   __shared__ uint32_t acnt[kBatch];
-  __shared__ uint32_t wbits[kThreads / 32][kWords];
+  __shared__ uint8_t lists[kThreads / 32][4][kBatch];
   const int tile = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
-  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + 4;
+  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float lx = (float)lxi + 0.5f, lyA = (float)lyi + 0.5f;
   const bool inA = px < cam.W && pyA < cam.H, inB = px < cam.W && pyB < cam.H;
@@ -1080,42 +1064,42 @@ __global__ void __launch_bounds__(kThreads) blend_contrib_kernel(
   for (int b0 = 0; b0 < len; b0 += kBatch) {
     const int nb = min(kBatch, len - b0);
     __syncthreads();
-    for (int t = threadIdx.x; t < kBatch; t += kThreads) {
-      if (t < nb) {
-        const uint32_t sidx = vals[rg.x + b0 + t];
-        const Staged e = stage_entry(rec, geom, sidx, tx0, ty0, cam.H, rf);
-        s0[t] = e.s0;
-        s1[t] = e.s1;
-        s2[t] = e.s2;
-        s4[t] = e.s4;
-        s5[t] = e.s5;
-        sm[t] = e.wmask;
-        sid[t] = sidx;
-        asum[t] = 0.f;
-        acnt[t] = 0u;
-      }
+    for (int t = threadIdx.x; t < nb; t += kThreads) {
+      const uint32_t sidx = vals[rg.x + b0 + t];
+      const uint16_t m = masks[rg.x + b0 + t];
+      sm[t] = m;
+      sid[t] = sidx;
+      asum[t] = 0.f;
+      acnt[t] = 0u;
+      if (m == 0u) continue;
+      const Staged e = stage_entry(rec, sidx, tx0, ty0);
+      s0[t] = e.s0;
+      s1[t] = e.s1;
+      s2[t] = e.s2;
+      s4[t] = e.s4;
+      s5[t] = e.s5;
     }
     __syncthreads();
-    warp_entry_bits(sm, nb, warp, lane, wbits[warp]);
-    for (int j = 0; j < kWords; ++j) {
-      uint32_t bits = wbits[warp][j];
-      while (bits != 0u) {
-        const int k = 32 * j + __ffs(bits) - 1;
-        bits &= bits - 1u;
-        const float4 e0 = s0[k], e1 = s1[k], e2 = s2[k];
-        Pair qa, qb;
-        eval_two(lx, lyA, e0, e1, s4[k], s5[k], e2.y, set, qa, qb);
-        const unsigned ba = __ballot_sync(0xffffffffu, inA && qa.rho <= set.rho_max);
-        const unsigned bb = __ballot_sync(0xffffffffu, inB && qb.rho <= set.rho_max);
-        const uint32_t cnt = (uint32_t)(__popc(ba) + __popc(bb));
-        float c = contrib_step(TA, stA, qa, set, gamma) + contrib_step(TB, stB, qb, set, gamma);
-        if (cnt == 0u) continue;
-  #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (lane == 0) {
-          atomicAdd(&acnt[k], cnt);
-          if (c != 0.f) atomicAdd(&asum[k], c);
-        }
+    const int glen = group_lists<kBatch>(sm, nb, warp, lane, lists[warp]);
+    const uint8_t* list = lists[warp][lane >> 3];
+    const int longest = warp_longest(glen);
+    for (int i = 0; i < longest; ++i) {
+      const bool active = i < glen;
+      const int k = active ? list[i] : 0;
+      const float4 e0 = s0[k], e1 = s1[k], e2 = s2[k];
+      Pair qa, qb;
+      eval_two(lx, lyA, e0, e1, s4[k], s5[k], e2.y, set, qa, qb);
+      const unsigned ba = __ballot_sync(0xffffffffu, active && inA && qa.rho <= set.rho_max);
+      const unsigned bb = __ballot_sync(0xffffffffu, active && inB && qb.rho <= set.rho_max);
+      if ((ba | bb) == 0u) continue;
+      const int sft = lane & 24;
+      const uint32_t cnt = (uint32_t)(__popc((ba >> sft) & 0xffu) + __popc((bb >> sft) & 0xffu));
+      float c = active ? contrib_step(TA, stA, qa, set, gamma) + contrib_step(TB, stB, qb, set, gamma) : 0.f;
+#pragma unroll
+      for (int o = kGroup / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      if ((lane & 7) == 0 && cnt != 0u) {
+        atomicAdd(&acnt[k], cnt);
+        if (c != 0.f) atomicAdd(&asum[k], c);
       }
     }
     __syncthreads();
@@ -1131,13 +1115,12 @@ __global__ void __launch_bounds__(kThreads) blend_contrib_kernel(
 }  // namespace
 
 cudaError_t launch_blend_fwd(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
-                             const RowGeom* geom, const uint32_t* vals, const int2* ranges, float* out,
+                             const uint16_t* masks, const uint32_t* vals, const int2* ranges, float* out,
                              int32_t* n_contrib, int32_t* last, int32_t* med,
                              unsigned long long* counters, cudaStream_t st) {
   const unsigned grid = (unsigned)cam.tiles_x * (unsigned)cam.tiles_y;
-  const float rf = (float)sqrt((double)set.rho_max / (double)set.sinv);
   ProfScope ps(kProfBlendFwd, st);
-  blend_fwd_kernel<<<grid, kThreads, 0, st>>>(cam, set, rf, order, rec, geom, vals, ranges, out, n_contrib,
+  blend_fwd_kernel<<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, n_contrib,
                                               last, med, counters, 0);
   count_launch();
   return cudaGetLastError();
@@ -1146,11 +1129,10 @@ cudaError_t launch_blend_fwd(const CamDev& cam, const SetDev& set, const uint32_
 size_t seg_part_bytes() { return sizeof(SegPart); }
 
 cudaError_t launch_blend_fwd_split(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
-                                   const RowGeom* geom, const uint32_t* vals, const int2* ranges, float* out,
+                                   const uint16_t* masks, const uint32_t* vals, const int2* ranges, float* out,
                                    int32_t* n_contrib, int32_t* last, int32_t* med, unsigned long long* counters,
                                    const SegBufs& sb, cudaStream_t st) {
   const int ntiles = cam.tiles_x * cam.tiles_y;
-  const float rf = (float)sqrt((double)set.rho_max / (double)set.sinv);
   ProfScope ps(kProfBlendFwd, st);
   count_launch(2);
   seg_count_kernel<<<div_up(ntiles, 256), 256, 0, st>>>(ranges, ntiles, sb.lseg, sb.segcnt);
@@ -1160,11 +1142,11 @@ cudaError_t launch_blend_fwd_split(const CamDev& cam, const SetDev& set, const u
   // the whole tiles, then the segments (grids sized for the bound, the device
   // count decides)
   count_launch(4);
-  blend_fwd_kernel<<<(unsigned)ntiles, kThreads, 0, st>>>(cam, set, rf, order, rec, geom, vals, ranges, out,
+  blend_fwd_kernel<<<(unsigned)ntiles, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out,
                                                           n_contrib, last, med, counters, sb.lseg);
-  seg_trans_kernel<<<sb.nseg_max, kThreads, 0, st>>>(cam, set, rf, rec, geom, vals, ranges, sb.lseg, sb.seg_tile,
+  seg_trans_kernel<<<sb.nseg_max, kThreads, 0, st>>>(cam, set, rec, masks, vals, ranges, sb.lseg, sb.seg_tile,
                                                      sb.seg_idx, sb.nseg, sb.trans);
-  seg_blend_kernel<<<sb.nseg_max, kThreads, 0, st>>>(cam, set, rf, rec, geom, vals, ranges, sb.lseg, sb.seg_tile,
+  seg_blend_kernel<<<sb.nseg_max, kThreads, 0, st>>>(cam, set, rec, masks, vals, ranges, sb.lseg, sb.seg_tile,
                                                      sb.seg_idx, sb.nseg, sb.trans,
                                                      static_cast<SegPart*>(sb.part), counters);
   seg_merge_kernel<<<sb.nseg_max, kThreads, 0, st>>>(cam, set, rec, vals, ranges, sb.segcnt, sb.seg_tile,
@@ -1181,12 +1163,11 @@ cudaError_t launch_blend_fwd_batched(const BlendBatch& batch, int grid, cudaStre
 }
 
 cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
-                             const RowGeom* geom, const uint32_t* vals, const int2* ranges, const float* out,
+                             const uint16_t* masks, const uint32_t* vals, const int2* ranges, const float* out,
                              const int32_t* last, const int32_t* med, const AdjDev& adj,
                              float* grec, float* screen, int n, int64_t K, unsigned long long* counters,
                              cudaStream_t st) {
   const unsigned grid = (unsigned)cam.tiles_x * (unsigned)cam.tiles_y;
-  const float rf = (float)sqrt((double)set.rho_max / (double)set.sinv);
   // the training loss drives set 0 through colour and inverse depth only and
   // the other sets through colour: a leaner kernel for that layout
   bool loss_layout = (adj.mask[0] & ~(GS_MASK_RGB | (1u << GS_PLANE_INVDEPTH))) == 0u;
@@ -1196,7 +1177,7 @@ cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_
   const bool dense = K >= (int64_t)kDenseListLen * (int64_t)grid;
   ProfScope ps(kProfBlendBwd, st);
 #define GS_BWD(L, M)                                                                                           \
-  blend_bwd_kernel<L, M><<<grid, kThreads, 0, st>>>(cam, set, rf, order, rec, geom, vals, ranges, out, last, med, \
+  blend_bwd_kernel<L, M><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, last, med, \
                                                     adj, grec, screen, n, counters)
   if (loss_layout) {
     if (dense) GS_BWD(true, 4);
@@ -1211,12 +1192,11 @@ cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_
 }
 
 cudaError_t launch_blend_contrib(const CamDev& cam, const SetDev& set, float gamma, const uint32_t* order,
-                                 const float4* rec, const RowGeom* geom, const uint32_t* vals,
+                                 const float4* rec, const uint16_t* masks, const uint32_t* vals,
                                  const int2* ranges, float* csum, uint32_t* ccnt, cudaStream_t st) {
   const unsigned grid = (unsigned)cam.tiles_x * (unsigned)cam.tiles_y;
-  const float rf = (float)sqrt((double)set.rho_max / (double)set.sinv);
   ProfScope ps(kProfContrib, st);
-  blend_contrib_kernel<<<grid, kThreads, 0, st>>>(cam, set, rf, gamma, order, rec, geom, vals, ranges, csum,
+  blend_contrib_kernel<<<grid, kThreads, 0, st>>>(cam, set, gamma, order, rec, masks, vals, ranges, csum,
                                                   ccnt);
   count_launch();
   return cudaGetLastError();

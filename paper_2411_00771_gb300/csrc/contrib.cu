@@ -126,7 +126,7 @@ unsigned grid_for(int64_t n) {
 }  // namespace
 
 cudaError_t launch_contribution(const CamDev& cam, const SetDev& set, float gamma, float weight,
-                                const uint32_t* order, const float4* rec, const RowGeom* geom,
+                                const uint32_t* order, const float4* rec, const uint16_t* masks,
                                 const uint32_t* vals, const int2* ranges, const uint32_t* cand,
                                 const uint32_t* ncand, int64_t n, bool zero_cand, float* csum, uint32_t* ccnt,
                                 float* contrib, cudaStream_t st) {
@@ -138,7 +138,7 @@ cudaError_t launch_contribution(const CamDev& cam, const SetDev& set, float gamm
       contrib_zero_kernel<<<grid_for(n), kThreads, 0, st>>>(cand, ncand, csum, ccnt);
     }
   }
-  cudaError_t e = launch_blend_contrib(cam, set, gamma, order, rec, geom, vals, ranges, csum, ccnt, st);
+  cudaError_t e = launch_blend_contrib(cam, set, gamma, order, rec, masks, vals, ranges, csum, ccnt, st);
   if (e != cudaSuccess || !contrib) return e;
   ProfScope ps(kProfContrib, st);
   count_launch();

@@ -80,7 +80,7 @@ struct SetDev {
 // screen-filter disk is |d| <= rf.  [ilo, ihi] x [jlo, jhi] is the
 // pixel-centre index box of the whole footprint (FP64, clipped to the image).
 // Derived terms are computed in FP64 and rounded once.
-struct RowGeom {
+struct alignas(8) RowGeom {
   float cx_hi, cx_lo, cy_hi, cy_lo;
   float e0x, e0y, hy, t, slope, wsc;
   int ilo, ihi, jlo, jhi;
@@ -224,8 +224,12 @@ cudaError_t launch_gather_counts(const uint32_t* order, const uint32_t* tcount, 
 cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint32_t* counts,
                         const uint2* rect, const RowGeom* geom, float rf, int64_t n, int tiles_x,
                         uint32_t* keys, uint32_t* vals, cudaStream_t st, const uint32_t* n_dev = nullptr);
-cudaError_t launch_ranges(const uint32_t* keys, int64_t K, int2* ranges, int ntiles,
-                          cudaStream_t st);
+// Per-tile ranges of the sorted instances, and per instance the mask of the
+// tile's sixteen 4 x 4 pixel blocks that the footprint can reach: bit 4 w + g,
+// w = the 8 x 8 block's (column | row << 1), g = the 4 x 4 block's within it
+// (a superset, from the footprint's row rule on bands of four rows).
+cudaError_t launch_ranges(const uint32_t* keys, const uint32_t* vals, int64_t K, int2* ranges, int ntiles,
+                          const RowGeom* geom, float rf, const CamDev& cam, uint16_t* masks, cudaStream_t st);
 // Tile ids ordered by list length, longest first (launch order of the blends);
 // for images with more tiles than the ordering kernel holds, nothing is
 // written and the blends take the natural order (pass a null order).
@@ -233,7 +237,7 @@ bool tile_order_supported(int ntiles);
 cudaError_t launch_tile_order(const int2* ranges, int ntiles, uint32_t* order, cudaStream_t st);
 
 cudaError_t launch_blend_fwd(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
-                             const RowGeom* geom, const uint32_t* vals, const int2* ranges, float* out,
+                             const uint16_t* masks, const uint32_t* vals, const int2* ranges, float* out,
                              int32_t* n_contrib, int32_t* last, int32_t* med,
                              unsigned long long* counters, cudaStream_t st);
 
@@ -269,7 +273,7 @@ inline int split_lseg(int ntiles, int64_t K, int sms) {
 // 2 len / lseg, and the lengths sum to at most K.
 inline int64_t split_nseg_max(int64_t K, int lseg) { return (2 * K + lseg - 1) / lseg; }
 cudaError_t launch_blend_fwd_split(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
-                                   const RowGeom* geom, const uint32_t* vals, const int2* ranges, float* out,
+                                   const uint16_t* masks, const uint32_t* vals, const int2* ranges, float* out,
                                    int32_t* n_contrib, int32_t* last, int32_t* med, unsigned long long* counters,
                                    const SegBufs& sb, cudaStream_t st);
 
@@ -277,10 +281,9 @@ cudaError_t launch_blend_fwd_split(const CamDev& cam, const SetDev& set, const u
 struct BlendJob {
   CamDev cam;
   SetDev set;
-  float rf;
   int tile_begin;  // first work item of this view in the batch
   const float4* rec;
-  const RowGeom* geom;
+  const uint16_t* masks;
   const uint32_t* vals;
   const int2* ranges;
   float* out;
@@ -306,7 +309,7 @@ struct AdjDev {
 constexpr int kGradRec = 16;  // Ji(4) e(2) c(2) p_z(1) opacity(1) rgb(3) n(3)
 
 cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
-                             const RowGeom* geom, const uint32_t* vals, const int2* ranges, const float* out,
+                             const uint16_t* masks, const uint32_t* vals, const int2* ranges, const float* out,
                              const int32_t* last, const int32_t* med, const AdjDev& adj,
                              float* grec, float* screen, int n, int64_t K, unsigned long long* counters,
                              cudaStream_t st);
@@ -315,13 +318,13 @@ cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_
 // lists: per surfel the support count and the sum of alpha^gamma T^(1-gamma)
 // (csum, ccnt: [N], accumulated).
 cudaError_t launch_blend_contrib(const CamDev& cam, const SetDev& set, float gamma, const uint32_t* order,
-                                 const float4* rec, const RowGeom* geom, const uint32_t* vals,
+                                 const float4* rec, const uint16_t* masks, const uint32_t* vals,
                                  const int2* ranges, float* csum, uint32_t* ccnt, cudaStream_t st);
 // Zero the candidates' csum/ccnt (when zero_cand), run the contribution blend
 // and add weight * csum / ccnt to contrib[n] for the candidates (contrib may
 // be null).
 cudaError_t launch_contribution(const CamDev& cam, const SetDev& set, float gamma, float weight,
-                                const uint32_t* order, const float4* rec, const RowGeom* geom,
+                                const uint32_t* order, const float4* rec, const uint16_t* masks,
                                 const uint32_t* vals, const int2* ranges, const uint32_t* cand,
                                 const uint32_t* ncand, int64_t n, bool zero_cand, float* csum, uint32_t* ccnt,
                                 float* contrib, cudaStream_t st);

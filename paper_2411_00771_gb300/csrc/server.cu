@@ -91,6 +91,7 @@ struct Slot {
   uint32_t* sidx = nullptr;  // sorted surfel order (one of idx / idx2)
   uint32_t* ncand = nullptr; // device count of sorted candidates
   uint32_t* vals_final = nullptr;
+  uint16_t* masks = nullptr;  // block masks, in the key buffer that the sort left free
   size_t bytes() const {
     return rec.bytes + geom.bytes + rect.bytes + tcount.bytes + dkey.bytes + idx.bytes + dkey2.bytes +
            idx2.bytes + cnts.bytes + offs.bytes + cand.bytes + rtmp.bytes + keys.bytes + vals.bytes +
@@ -313,7 +314,9 @@ int stage_b(gs_server* s, Slot& sl, std::string* msg) {
   if (e == cudaSuccess)
     e = radix_sort_pairs((uint32_t*)sl.keys.p, (uint32_t*)sl.vals.p, (uint32_t*)sl.keys2.p,
                          (uint32_t*)sl.vals2.p, K, bits, (uint32_t*)sl.ktmp.p, &tk, &tv, st);
-  if (e == cudaSuccess) e = launch_ranges(tk, K, (int2*)sl.ranges.p, ntiles, st);
+  sl.masks = reinterpret_cast<uint16_t*>(tk == (uint32_t*)sl.keys.p ? sl.keys2.p : sl.keys.p);
+  if (e == cudaSuccess)
+    e = launch_ranges(tk, tv, K, (int2*)sl.ranges.p, ntiles, (const RowGeom*)sl.geom.p, sl.rf, sl.cam, sl.masks, st);
   if (e == cudaSuccess) e = cudaEventRecord(sl.ev_b, st);
   if (e != cudaSuccess) {
     *msg = std::string("stage B: ") + cudaGetErrorString(e);
@@ -361,8 +364,7 @@ bool launch_batch(gs_server* s, const std::vector<int>& ready, std::string* msg)
       sb.trans = (float*)sl.seg_trans.p;
       sb.part = sl.seg_part.p;
       const cudaError_t es = launch_blend_fwd_split(sl.cam, sl.set, nullptr, (const float4*)sl.rec.p,
-                                                    (const RowGeom*)sl.geom.p, sl.vals_final,
-                                                    (const int2*)sl.ranges.p, sl.t->req.out, sl.t->req.n_contrib,
+                                                    sl.masks, sl.vals_final, (const int2*)sl.ranges.p, sl.t->req.out, sl.t->req.n_contrib,
                                                     nullptr, nullptr, s->work, sb, s->blend_st);
       if (es != cudaSuccess) {
         *msg = std::string("blend: ") + cudaGetErrorString(es);
@@ -373,10 +375,9 @@ bool launch_batch(gs_server* s, const std::vector<int>& ready, std::string* msg)
     BlendJob& j = b.job[nj++];
     j.cam = sl.cam;
     j.set = sl.set;
-    j.rf = sl.rf;
     j.tile_begin = tiles;
     j.rec = (const float4*)sl.rec.p;
-    j.geom = (const RowGeom*)sl.geom.p;
+    j.masks = sl.masks;
     j.vals = sl.vals_final;
     j.ranges = (const int2*)sl.ranges.p;
     j.out = sl.t->req.out;

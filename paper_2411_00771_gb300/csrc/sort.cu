@@ -420,12 +420,34 @@ __global__ void __launch_bounds__(256) emit_kernel(const uint32_t* __restrict__ 
     emit_warp(r0 + lane, n, lane, order, offs, counts, rect, geom, rf, tiles_x, keys, vals);
 }
 
-__global__ void ranges_kernel(const uint32_t* __restrict__ keys, int64_t K, int2* __restrict__ ranges) {
+// One thread per sorted instance: the ends of its tile's range, and the mask
+// of the tile's 4 x 4 pixel blocks that its footprint can reach (the row rule
+// on the tile's four bands of four rows).  The blends read the mask in list
+// order instead of each gathering the footprint shape and evaluating the rule
+// again.
+__global__ void __launch_bounds__(256) ranges_kernel(const uint32_t* __restrict__ keys,
+                                                     const uint32_t* __restrict__ vals, int64_t K,
+                                                     int2* __restrict__ ranges, const RowGeom* __restrict__ geom,
+                                                     float rf, int tiles_x, int H, uint16_t* __restrict__ masks) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= K) return;
   const uint32_t t = keys[i];
+  const RowGeom g = geom[vals[i]];
   if (i == 0 || keys[i - 1] != t) ranges[t].x = (int)i;
   if (i == K - 1 || keys[i + 1] != t) ranges[t].y = (int)(i + 1);
+  const int tx0 = (int)(t % (uint32_t)tiles_x) * kTile, ty0 = (int)(t / (uint32_t)tiles_x) * kTile;
+  uint32_t m = 0u;
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const int ja = ty0 + 4 * b;
+    int ilo, ihi;
+    if (ja >= H || !band_pixels(g, ja, min(ja + 3, H - 1), rf, &ilo, &ihi)) continue;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (ilo <= tx0 + 4 * c + 3 && ihi >= tx0 + 4 * c)
+        m |= 1u << (4 * ((c >> 1) | (b & 2)) + ((c & 1) | ((b & 1) << 1)));
+  }
+  masks[i] = (uint16_t)m;
 }
 
 // Tiles ordered by list length, longest first (by octave of the length;
@@ -590,13 +612,13 @@ cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint3
   return cudaGetLastError();
 }
 
-cudaError_t launch_ranges(const uint32_t* keys, int64_t K, int2* ranges, int ntiles,
-                          cudaStream_t st) {
+cudaError_t launch_ranges(const uint32_t* keys, const uint32_t* vals, int64_t K, int2* ranges, int ntiles,
+                          const RowGeom* geom, float rf, const CamDev& cam, uint16_t* masks, cudaStream_t st) {
   ProfScope ps(kProfSort, st);
   cudaError_t e = cudaMemsetAsync(ranges, 0, sizeof(int2) * (size_t)ntiles, st);
   if (e != cudaSuccess || K <= 0) return e;
   count_launch();
-  ranges_kernel<<<div_up(K, 256), 256, 0, st>>>(keys, K, ranges);
+  ranges_kernel<<<div_up(K, 256), 256, 0, st>>>(keys, vals, K, ranges, geom, rf, cam.tiles_x, cam.H, masks);
   return cudaGetLastError();
 }
 
