@@ -342,11 +342,11 @@ __global__ void __launch_bounds__(256) preprocess_main_kernel(ParamsDev P, CamDe
       nref = make_float4(uh, vh, __fadd_rn(__fsub_rn(nu0.hi, uh), nu0.lo), __fadd_rn(__fsub_rn(nv0.hi, vh), nv0.lo));
       ugrid = ug;
     } else {
-      // edge-on disk: no object-space footprint (rho_obj is NaN, the
-      // screen filter decides)
+      // edge-on disk: no object-space footprint (Ji d and rho_obj are NaN,
+      // the screen filter decides; Ji itself stays finite for the backward)
       const float qnan = __int_as_float(0x7fffffff);
-      jh = make_float4(qnan, qnan, qnan, qnan);
-      jl = nref = make_float4(0.f, 0.f, 0.f, 0.f);
+      jh = jl = make_float4(0.f, 0.f, 0.f, 0.f);
+      nref = make_float4(qnan, qnan, 0.f, 0.f);
       ef = make_float2(0.f, 0.f);
     }
     // colour: SH at the world direction from the camera centre
