@@ -482,11 +482,13 @@ gs_status gs_render(gs_scene* sc, const gs_camera* c, float* out, int32_t* n_con
   gs_frame* f = new_frame(sc, c, out, "gs_render", &s);
   if (!f) return s;
   cudaStream_t st = (cudaStream_t)stream;
-  f->last = f->buf.get<int32_t>((size_t)f->cam.W * f->cam.H, st);
-  f->med = f->buf.get<int32_t>((size_t)f->cam.W * f->cam.H, st);
-  if (!f->last || !f->med) {
-    gs_frame_release(f, stream);
-    return fail(GS_ERR_OOM, "gs_render: device allocation failed");
+  if (saved) {  // what the backward needs of each pixel
+    f->last = f->buf.get<int32_t>((size_t)f->cam.W * f->cam.H, st);
+    f->med = f->buf.get<int32_t>((size_t)f->cam.W * f->cam.H, st);
+    if (!f->last || !f->med) {
+      gs_frame_release(f, stream);
+      return fail(GS_ERR_OOM, "gs_render: device allocation failed");
+    }
   }
   s = build_lists(sc, f, "gs_render", st);
   if (s == GS_OK) s = blend_forward(sc, f, out, n_contrib, st);
@@ -652,16 +654,27 @@ gs_status gs_backward(gs_scene* sc, gs_frame* f, const float* const* adj_sets,
   }
   cudaStream_t st = (cudaStream_t)stream;
   const int n = f->n;
-  float* grec = static_cast<float*>(sc->al.get(sizeof(float) * kGradRec * (size_t)(n > 0 ? n : 1), st));
-  if (!grec) return fail(GS_ERR_OOM, "gs_backward: scratch allocation failed");
-  cudaError_t e = cudaMemsetAsync(grec, 0, sizeof(float) * kGradRec * (size_t)n, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(f->counters + 2, 0, 3 * sizeof(unsigned long long), st);
+  const bool loss_layout = grad_loss_layout(adj);
+  const size_t row_bytes = sizeof(double) * grad_row_stride(loss_layout);
+  // gradient rows of all surfels, or of as many as there is memory for: the
+  // replay then runs once for each part of them
+  int rows = n > 0 ? n : 1;
+  double* grow = nullptr;
+  while (!(grow = static_cast<double*>(sc->al.get(row_bytes * (size_t)rows, st))) && rows > 1) rows = (rows + 1) / 2;
+  if (!grow) return fail(GS_ERR_OOM, "gs_backward: scratch allocation failed");
+  cudaError_t e = cudaMemsetAsync(f->counters + 2, 0, 3 * sizeof(unsigned long long), st);
   const SetDev set = to_dev(sc->settings);
-  if (e == cudaSuccess)
-    e = launch_blend_bwd(f->cam, set, f->order, f->rec, f->masks, f->vals, f->ranges, f->out, f->last, f->med, adj,
-                         grec, screen_grads, n, f->K, f->counters, st);
-  if (e == cudaSuccess) e = launch_preprocess_bwd(sc->P, f->cam, f->cand, f->ncand, f->tcount, grec, *grads, st);
-  sc->al.put(grec, sizeof(float) * kGradRec * (size_t)(n > 0 ? n : 1), st);
+  for (int64_t lo = 0; lo < n && e == cudaSuccess; lo += rows) {
+    const uint32_t part = (uint32_t)(n - lo < rows ? n - lo : rows);
+    e = launch_zero_rows(n, f->cand, f->ncand, loss_layout, grow, (uint32_t)lo, part, st);
+    if (e == cudaSuccess)
+      e = launch_blend_bwd(f->cam, set, f->order, f->rec, f->masks, f->vals, f->ranges, f->out, f->last, f->med, adj,
+                           loss_layout, grow, (uint32_t)lo, part, lo == 0 ? f->counters : nullptr, st);
+    if (e == cudaSuccess)
+      e = launch_preprocess_bwd(sc->P, f->cam, f->cand, f->ncand, f->tcount, f->rec, loss_layout, grow, (uint32_t)lo,
+                                part, n_sets, screen_grads, *grads, st);
+  }
+  sc->al.put(grow, row_bytes * (size_t)rows, st);
   if (e != cudaSuccess) return cuda_fail(e, "gs_backward");
   return GS_OK;
 }

@@ -162,10 +162,140 @@ __device__ __forceinline__ int group_lists(const uint16_t* sm, int nb, int warp,
   return g == 0 ? base[0] : (g == 1 ? base[1] : (g == 2 ? base[2] : base[3]));
 }
 
-// The longest of the four groups' lists.
-__device__ __forceinline__ int warp_longest(int n) {
-  n = max(n, __shfl_xor_sync(0xffffffffu, n, 8));
-  return max(n, __shfl_xor_sync(0xffffffffu, n, 16));
+// One warp's window on its tile's list: the entries that reach its 8 x 8
+// block, staged 32 at a time into the two halves of a ring, and for each of
+// the warp's four lane groups the ring slots of the entries that reach the
+// group's 4 x 4 block, in walking order.
+constexpr int kHalf = 32;
+constexpr int kRing = 2 * kHalf;
+constexpr int kQueue = kRing;
+constexpr int kNoMore = 1 << 30;
+struct WarpSmem {
+  // slot kRing: an entry that no pixel is near, for the groups whose list is used up
+  float4 s0[kRing + 1], s1[kRing + 1], s2[kRing + 1], s3[kRing + 1], s4[kRing + 1], s5[kRing + 1];
+  uint2 meta[kRing + 1];   // list position, surfel
+  uint2 q[kQueue];         // entries found but not yet staged (a ring): position, surfel
+  uint8_t qm[kQueue];      // and their group masks
+  uint16_t list[4][kRing];  // per group, byte offsets of ring slots (16 x slot; a ring of its own)
+};
+
+// Walks list positions [p0, p1) of a tile (front to back, or back to front
+// when kBack) for one warp.  body(k, i) is called with every lane: k is the
+// offset (16 x ring slot) of the lane's group's next entry and i the number
+// of entries of its list walked so far, this one included; a group whose list
+// is used up for now gets an entry that misses every pixel.  A lane that needs
+// no more entries sets i to kNoMore (or starts with it).  kBack: the group
+// takes only entries below its limit.  Returns the lane's i.
+//
+// The warps of a CTA share no data and no barrier: with one staging per CTA
+// and batch, a quarter of the warps' time went to waiting for the slowest
+// warp and for the staging loads.  A group may run ahead of the others by
+// up to one half of the ring, which evens out most of the difference between
+// the groups' lists (the older half is refilled when all groups are past it).
+// Element of a staged array at a byte offset that is 16 times its slot.
+__device__ __forceinline__ float4 at16(const float4* a, int k) {
+  return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(a) + k);
+}
+__device__ __forceinline__ uint2 at16(const uint2* a, int k) {
+  return *reinterpret_cast<const uint2*>(reinterpret_cast<const char*>(a) + k / 2);
+}
+
+template <bool kBack, class Body>
+__device__ __forceinline__ int walk_list(WarpSmem& sm, const float4* __restrict__ rec,
+                                         const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, int p0,
+                                         int p1, int limit, int tx0, int ty0, int blk, int i, Body body) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31, g = lane >> 3;
+  const uint32_t lt = (1u << lane) - 1u;
+  int scan = kBack ? p1 : p0, qn = 0, q0 = 0;
+  uint32_t pm = 0u, pv = 0u;  // the next 32 entries' masks and surfels, loaded ahead
+  auto left = [&] { return kBack ? scan > p0 : scan < p1; };
+  auto at = [&] { return kBack ? scan - 1 - lane : scan + lane; };
+  auto load = [&] {
+    const int e = at();
+    const bool in = kBack ? e >= p0 : e < p1;
+    pm = in ? masks[e] : 0u;
+    pv = in ? vals[e] : 0u;
+  };
+  load();
+  if (lane == 0) {
+    sm.s0[kRing] = make_float4(1e15f, 1e15f, 0.f, 0.f);
+    sm.s1[kRing] = sm.s3[kRing] = sm.s4[kRing] = make_float4(0.f, 0.f, 0.f, 0.f);
+    sm.s2[kRing] = make_float4(1.f, 0.f, 0.f, 0.f);
+    sm.s5[kRing] = make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, 0.f);
+    sm.meta[kRing] = make_uint2(0x7fffffffu, 0u);
+  }
+  // entries staged so far for the lane's group, and for all four groups modulo
+  // the ring (one byte each); mid: those of the older half
+  int end = 0, h = 0;
+  uint32_t cnt = 0u;
+  for (;;) {
+    int mid = end;
+    const bool fill = qn > 0 || left();
+    if (fill) {
+      __syncwarp();  // every lane is done with the older half
+      while (qn < kHalf && left()) {
+        const int e = at();
+        uint32_t m = (pm >> (4 * blk)) & 15u;
+        const uint32_t v = pv;
+        if constexpr (kBack) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (e >= __shfl_sync(kFull, limit, 8 * j)) m &= ~(1u << j);
+        }
+        scan += kBack ? -32 : 32;
+        if (left()) load();
+        const uint32_t b = __ballot_sync(kFull, m != 0u);
+        if (m != 0u) {
+          const int slot = (q0 + qn + __popc(b & lt)) & (kQueue - 1);
+          sm.q[slot] = make_uint2((uint32_t)e, v);
+          sm.qm[slot] = (uint8_t)m;
+        }
+        qn += __popc(b);
+      }
+      __syncwarp();
+      const int nb = min(qn, kHalf);
+      const int slot = h * kHalf + lane;
+      uint32_t m = 0u;
+      if (lane < nb) {
+        const uint2 x = sm.q[(q0 + lane) & (kQueue - 1)];
+        m = sm.qm[(q0 + lane) & (kQueue - 1)];
+        const Staged e = stage_entry(rec, x.y, tx0, ty0);
+        sm.s0[slot] = e.s0;
+        sm.s1[slot] = e.s1;
+        sm.s2[slot] = e.s2;
+        sm.s3[slot] = e.s3;
+        sm.s4[slot] = e.s4;
+        sm.s5[slot] = e.s5;
+        sm.meta[slot] = make_uint2(x.x, x.y);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const bool in = (m >> j) & 1u;
+        const uint32_t b = __ballot_sync(kFull, in);
+        if (in) sm.list[j][((cnt >> (8 * j)) + __popc(b & lt)) & (kRing - 1)] = (uint16_t)(16 * slot);
+        cnt += (uint32_t)__popc(b) << (8 * j);
+        end += g == j ? __popc(b) : 0;
+      }
+      cnt &= 0x3f3f3f3fu;
+      qn -= nb;
+      q0 += nb;
+      __syncwarp();
+      h ^= 1;
+    } else {
+      mid = end;
+    }
+    while (__any_sync(kFull, i < mid)) {
+      int k = 16 * kRing;
+      if (i < end) {
+        k = sm.list[g][i & (kRing - 1)];
+        ++i;
+      }
+      body(k, i);
+    }
+    if (!__any_sync(kFull, i < (fill ? kNoMore : end))) break;
+  }
+  return i;
 }
 
 // One entry against a thread's two pixels A and B (one column, kRowStep rows
@@ -199,14 +329,14 @@ __device__ __forceinline__ Pair eval_pair(float lx, float2 ly, float4 s0, float4
   const float2 u = mul2(q.nu, q.rden), v = mul2(q.nv, q.rden);
   const float2 ro = fma2(u, u, mul2(v, v));
   const float2 rs = mul2(bc(set.sinv), fma2(bc(q.dx), bc(q.dx), mul2(q.dy, q.dy)));
-  q.objA = den.x > 0.f && ro.x <= rs.x;  // false for NaN (edge-on disks)
-  q.objB = den.y > 0.f && ro.y <= rs.y;
+  q.objA = (den.x > 0.f) & (ro.x <= rs.x);  // false for NaN (edge-on disks)
+  q.objB = (den.y > 0.f) & (ro.y <= rs.y);
   q.rho = sel2(q.objA, q.objB, ro, rs);
   const float2 x = mul2(bc(kNegHalfLog2e), q.rho);
   const float2 a = mul2(bc(opac), make_float2(ex2_approx(x.x), ex2_approx(x.y)));
   q.alpha = make_float2(fminf(set.alpha_max, a.x), fminf(set.alpha_max, a.y));
-  q.hitA = q.rho.x <= set.rho_max && q.alpha.x >= set.alpha_min;
-  q.hitB = q.rho.y <= set.rho_max && q.alpha.y >= set.alpha_min;
+  q.hitA = (q.rho.x <= set.rho_max) & (q.alpha.x >= set.alpha_min);
+  q.hitB = (q.rho.y <= set.rho_max) & (q.alpha.y >= set.alpha_min);
   return q;
 }
 
@@ -265,24 +395,25 @@ __device__ __forceinline__ void fwd_init(FwdPair& p, bool insideA, bool insideB)
 
 // One list entry (position pos, already evaluated as q) against the two
 // pixels.  Branch-free: a pair that is not blended updates the sums with alpha
-// 0 (and a finite depth), which leaves them unchanged.  Returns whether a
-// pixel stopped at this entry.
-template <bool kFixedRef = false>
+// 0 (and a finite depth), which leaves them unchanged.  kPos: also the
+// positions of the last blended and the median entry.  kFixedRef: zr is given.
+// Returns whether a pixel stopped at this entry.
+template <bool kFixedRef, bool kPos>
 __device__ __forceinline__ bool fwd_step(FwdPair& p, const Pair& q, float4 e2, float4 e3, int pos, const SetDev& set,
                                          bool* stopA, bool* stopB) {
   const float2 one = bc(1.f);
   const float2 Tn = mul2(p.T, fma2(neg2(q.alpha), one, one));
-  const bool hA = !p.doneA && q.hitA, hB = !p.doneB && q.hitB;
-  *stopA = hA && Tn.x < set.T_min;
-  *stopB = hB && Tn.y < set.T_min;
-  const bool blA = hA && !(Tn.x < set.T_min), blB = hB && !(Tn.y < set.T_min);
+  const bool hA = !p.doneA & q.hitA, hB = !p.doneB & q.hitB;
+  *stopA = hA & (Tn.x < set.T_min);
+  *stopB = hB & (Tn.y < set.T_min);
+  const bool blA = hA & !(Tn.x < set.T_min), blB = hB & !(Tn.y < set.T_min);
   const float2 al = sel2(blA, blB, q.alpha, bc(0.f));
   const float2 w = mul2(al, p.T);
   const float2 z = sel2(q.objA, q.objB, mul2(bc(e2.x), q.rden), bc(e2.x));
   p.C0 = fma2(w, bc(e2.z), p.C0);
   p.C1 = fma2(w, bc(e2.w), p.C1);
   p.C2 = fma2(w, bc(e3.x), p.C2);
-  if constexpr (!kFixedRef) p.zr = sel2(blA && p.cntA == 0, blB && p.cntB == 0, z, p.zr);
+  if constexpr (!kFixedRef) p.zr = sel2(blA & (p.cntA == 0), blB & (p.cntB == 0), z, p.zr);
   const float2 zs = add2(z, neg2(p.zr));
   p.D = fma2(add2(w, w), fma2(zs, p.A, neg2(p.Zs)), p.D);
   p.A = add2(p.A, w);
@@ -291,21 +422,23 @@ __device__ __forceinline__ bool fwd_step(FwdPair& p, const Pair& q, float4 e2, f
   p.N0 = fma2(w, bc(e3.y), p.N0);
   p.N1 = fma2(w, bc(e3.z), p.N1);
   p.N2 = fma2(w, bc(e3.w), p.N2);
-  const bool mA = blA && p.T.x > 0.5f, mB = blB && p.T.y > 0.5f;
+  const bool mA = blA & (p.T.x > 0.5f), mB = blB & (p.T.y > 0.5f);
   p.M = sel2(mA, mB, z, p.M);
-  p.medA = mA ? pos : p.medA;
-  p.medB = mB ? pos : p.medB;
+  if constexpr (kPos) {
+    p.medA = mA ? pos : p.medA;
+    p.medB = mB ? pos : p.medB;
+    p.lastA = blA ? pos + 1 : p.lastA;
+    p.lastB = blB ? pos + 1 : p.lastB;
+  }
   p.T = mul2(p.T, fma2(neg2(al), one, one));
   p.cntA += blA ? 1 : 0;
   p.cntB += blB ? 1 : 0;
-  p.lastA = blA ? pos + 1 : p.lastA;
-  p.lastB = blB ? pos + 1 : p.lastB;
-  return *stopA || *stopB;
+  return *stopA | *stopB;
 }
 
 // A lane group's walk over its list of one batch (list positions b0 + k),
 // front to back, until both of the thread's pixels are done.
-template <bool kFixedRef>
+template <bool kFixedRef, bool kPos>
 __device__ __forceinline__ void fwd_walk(FwdPair& p, const FwdSmem& sh, const uint8_t* list, int glen, int b0, float lx,
                                          float2 ly, const SetDev& set) {
   if (p.doneA && p.doneB) return;
@@ -316,7 +449,7 @@ __device__ __forceinline__ void fwd_walk(FwdPair& p, const FwdSmem& sh, const ui
     k = list[i + 1];  // past the end: a byte of padding, not used
     const Pair q = eval_pair(lx, ly, e0, e1, e4, e5, e2.y, set);
     bool stopA, stopB;
-    if (fwd_step<kFixedRef>(p, q, e2, e3, pos, set, &stopA, &stopB)) {  // once per pixel
+    if (fwd_step<kFixedRef, kPos>(p, q, e2, e3, pos, set, &stopA, &stopB)) {  // once per pixel
       p.evaluated += (stopA ? i + 1 : 0) + (stopB ? i + 1 : 0);
       p.doneA = p.doneA || stopA;
       p.doneB = p.doneB || stopB;
@@ -369,6 +502,7 @@ __device__ __forceinline__ void stage_batch(FwdSmem& sh, const float4* __restric
 }
 
 // Forward blend of tile (bx, by) of one view by the whole CTA.
+template <bool kPos>
 __device__ __forceinline__ void blend_fwd_tile(
     FwdSmem& sh, const CamDev& cam, const SetDev& set, const float4* __restrict__ rec,
     const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
@@ -392,7 +526,7 @@ __device__ __forceinline__ void blend_fwd_tile(
     stage_batch(sh, rec, masks, vals, rg.x + b0, nb, tx0, ty0);
     __syncthreads();
     const int glen = group_lists<kBatch>(sh.sm, nb, warp, lane, sh.list[warp]);
-    fwd_walk<false>(p, sh, sh.list[warp][lane >> 3], glen, b0, lx, ly, set);
+    fwd_walk<false, kPos>(p, sh, sh.list[warp][lane >> 3], glen, b0, lx, ly, set);
   }
   fwd_store(p.a(), cam, set, px, pyA, out, n_contrib, last, med);
   fwd_store(p.b(), cam, set, px, pyB, out, n_contrib, last, med);
@@ -420,6 +554,7 @@ __device__ __forceinline__ void blend_fwd_tile(
 }
 
 // One CTA per tile; block b takes tile order[b] (longest lists first).
+template <bool kPos>
 __global__ void __launch_bounds__(kThreads, 5) blend_fwd_kernel(
     CamDev cam, SetDev set, const uint32_t* __restrict__ order, const float4* __restrict__ rec,
     const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
@@ -427,7 +562,7 @@ __global__ void __launch_bounds__(kThreads, 5) blend_fwd_kernel(
     int32_t* __restrict__ med, unsigned long long* __restrict__ counters, int lseg) {
   __shared__ FwdSmem sh;
   const int t = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
-  blend_fwd_tile(sh, cam, set, rec, masks, vals, ranges, out, n_contrib, last, med, counters,
+  blend_fwd_tile<kPos>(sh, cam, set, rec, masks, vals, ranges, out, n_contrib, last, med, counters,
                  t % cam.tiles_x, t / cam.tiles_x, lseg);
 }
 
@@ -470,7 +605,7 @@ __device__ __forceinline__ bool seg_of(const uint32_t* seg_tile, const uint32_t*
   return true;
 }
 
-__global__ void __launch_bounds__(kThreads) seg_trans_kernel(
+__global__ void __launch_bounds__(kThreads, 5) seg_trans_kernel(
     CamDev cam, SetDev set, const float4* __restrict__ rec, const uint16_t* __restrict__ masks,
     const uint32_t* __restrict__ vals, const int2* __restrict__ ranges, int lseg,
     const uint32_t* __restrict__ seg_tile, const uint32_t* __restrict__ seg_idx, const uint32_t* __restrict__ nseg,
@@ -513,7 +648,7 @@ __device__ __forceinline__ void seg_store(const FwdPix& p, bool stopped, SegPart
   part[slot] = q;
 }
 
-__global__ void __launch_bounds__(kThreads) seg_blend_kernel(
+__global__ void __launch_bounds__(kThreads, 5) seg_blend_kernel(
     CamDev cam, SetDev set, const float4* __restrict__ rec, const uint16_t* __restrict__ masks,
     const uint32_t* __restrict__ vals, const int2* __restrict__ ranges, int lseg,
     const uint32_t* __restrict__ seg_tile, const uint32_t* __restrict__ seg_idx, const uint32_t* __restrict__ nseg,
@@ -545,7 +680,7 @@ __global__ void __launch_bounds__(kThreads) seg_blend_kernel(
     stage_batch(sh, rec, masks, vals, rg.x + b0, nb, tx0, ty0);
     __syncthreads();
     const int glen = group_lists<kBatch>(sh.sm, nb, warp, lane, sh.list[warp]);
-    fwd_walk<true>(p, sh, sh.list[warp][lane >> 3], glen, b0, lx, ly, set);
+    fwd_walk<true, true>(p, sh, sh.list[warp][lane >> 3], glen, b0, lx, ly, set);
   }
   SegPart* pp = part + (size_t)blockIdx.x * kTilePix;
   seg_store(p.a(), inA && p.doneA, pp, threadIdx.x);
@@ -639,7 +774,7 @@ __global__ void seg_list_kernel(const uint32_t* __restrict__ segcnt, const uint3
 // CTA takes (view, tile) work items from a device counter until all tiles
 // of all views in the batch are done; views of different sizes and scenes
 // share one launch.
-__global__ void __launch_bounds__(kThreads) blend_fwd_batched_kernel(BlendBatch batch) {
+__global__ void __launch_bounds__(kThreads, 5) blend_fwd_batched_kernel(BlendBatch batch) {
   __shared__ FwdSmem sh;
   __shared__ int item;
   for (;;) {
@@ -652,7 +787,7 @@ __global__ void __launch_bounds__(kThreads) blend_fwd_batched_kernel(BlendBatch 
     while (j + 1 < batch.njobs && batch.job[j + 1].tile_begin <= t) ++j;
     const BlendJob& jb = batch.job[j];
     const int local = t - jb.tile_begin;
-    blend_fwd_tile(sh, jb.cam, jb.set, jb.rec, jb.masks, jb.vals, jb.ranges, jb.out, jb.n_contrib,
+    blend_fwd_tile<false>(sh, jb.cam, jb.set, jb.rec, jb.masks, jb.vals, jb.ranges, jb.out, jb.n_contrib,
                    nullptr, nullptr, batch.work, local % jb.cam.tiles_x, local / jb.cam.tiles_x);
   }
 }
@@ -661,43 +796,62 @@ __global__ void __launch_bounds__(kThreads) blend_fwd_batched_kernel(BlendBatch 
 // Backward.
 
 constexpr int kMaxSets = 3;
-// Entries staged per batch in the backward, by the CTAs per SM its variant
-// is sized for: 128 for five (a small batch leaves more of the SM's shared
-// memory to L1: 0.939 -> 0.921 ms on the 1M-surfel view, against 224), 224
-// for four (the dense variant's long lists: 128 made the 4M-surfel training
-// step 2.5 % slower).  The gradient accumulators and the six staged vectors
-// per entry fit either way.
-constexpr int batch_b(int min_ctas) { return min_ctas >= 5 ? 128 : 224; }
-// Average tile-list length from which the backward takes the 4-CTA variant:
-// 200 (the 1M-surfel aerial view) ran best with 5 CTAs per SM, 590 (the
-// 4M-surfel orbit view) with 4.
-constexpr int kDenseListLen = 400;
-
-// Per-pair gradient vector.  General layout (any adjoint planes):
-//   [0..5] d Ji, d e; [6] Zc, the depth term of the centre gradient (below);
-//   [7] d p_z, [8] opacity times d opacity, [9..11] d rgb, [12..14] d normal;
-//   [15 + 2 s, 16 + 2 s] screen-space gradient of set s.
-// Loss layout (set 0 on colour and inverse depth only, later sets on
-// colour): the normal slots are dropped, [0..11] as above without d normal,
-// [12 + 2 s, 13 + 2 s] screen gradients.
-// The centre gradient is not accumulated on its own: per pair it is set 0's
-// screen gradient plus, on the object-space branch, the term of the depth
-// z = p_z / (1 + e.d) through d, (d rden / d d) p_z dz = -e p_z rden^2 dz;
-// so d c = (screen gradient of set 0) + e * Zc with Zc the sum of
-// p_z rden^2 dz, formed once per entry at the flush.  Likewise
-// d alpha / d opacity = alpha / opacity, divided once at the flush.
+// Per-entry gradient vector, the surfel's gradient row (kRow* in
+// gs2d_internal.cuh): d Ji, d e, the screen-space gradient of set 0, the depth
+// term of the centre gradient, d p_z, opacity times d opacity, d rgb, the
+// screen-space gradients of sets 1 and 2, and in the general layout d normal.
+// The loss layout (set 0 on colour and inverse depth only, later sets on
+// colour) has no d normal.  d c is not summed from its own terms: per pair it
+// is set 0's screen gradient plus, on the object-space branch, the term of the
+// depth z = p_z / (1 + e.d) through d, (d rden / d d) p_z dz = -e p_z rden^2 dz;
+// so d c = (screen gradient of set 0) + e * (sum of p_z rden^2 dz), formed once
+// per surfel by the preprocess's backward, and d alpha / d opacity = alpha /
+// opacity, divided there.
+//
+// The reduce-scatter leaves lane r of a group the sums of up to three
+// consecutive values; nat() places the vector so that the groups' first,
+// second and third values are consecutive in the row.
 template <bool kLoss>
 struct Layout {
-  static constexpr int kRec = kLoss ? 12 : kGradRec - 1;
-  static constexpr int kN = kRec + 2 * kMaxSets;  // 18 or 21
+  static constexpr int kN = kLoss ? kRowLoss : kRowAll;
+  // first value of lane r (the halving of kN: 3 2 3 1 3 2 3 1, 3 3 3 2 3 3 3 1)
+  __host__ __device__ static constexpr int start(int r) {
+    return kLoss ? 9 * (r >> 2) + 5 * ((r >> 1) & 1) + 3 * (r & 1) : 11 * (r >> 2) + 6 * ((r >> 1) & 1) + 3 * (r & 1);
+  }
+  // the row's value at lane r's i-th place, -1 when it has none
+  __host__ __device__ static constexpr int at(int r, int i) {
+    if (i == 0) return r;
+    if (kLoss) {
+      if (i == 1) return (r & 3) == 3 ? -1 : 8 + r - (r > 3 ? 1 : 0);
+      return (r & 1) ? -1 : 14 + (r >> 1);
+    }
+    if (i == 1) return r == 7 ? -1 : 8 + r;
+    return (r & 3) == 3 ? -1 : 15 + r - (r > 3 ? 1 : 0);
+  }
+  __host__ __device__ static constexpr int nat(int m) {
+    for (int r = 0; r < 8; ++r)
+      for (int i = 0; i < 3; ++i)
+        if (at(r, i) == m) return start(r) + i;
+    return -1;
+  }
 };
+constexpr bool layout_is_permutation(bool loss) {
+  const int n = loss ? kRowLoss : kRowAll;
+  uint32_t seen = 0;
+  for (int m = 0; m < n; ++m) {
+    const int v = loss ? Layout<true>::nat(m) : Layout<false>::nat(m);
+    if (v < 0 || v >= n || ((seen >> v) & 1u)) return false;
+    seen |= 1u << v;
+  }
+  return true;
+}
+static_assert(layout_is_permutation(true) && layout_is_permutation(false), "one place per value");
 
 // Balanced reduce-scatter of N values over a lane group of eight: at each
 // halving level the lanes whose bit is clear keep the first ceil(N/2) values
 // and the others the rest, exchanging the halves they do not keep (17
 // shuffles for 18 values, and the warp's four groups reduce four entries at
-// once).  Afterwards v[0 .. kRsMax) holds the group's sums of the slots
-// given by rs_slots() for the lane.
+// once).  Afterwards v[0..2] hold the group's sums of values start(r) + 0..2.
 constexpr int kGroup = 8;
 template <int O, int N>
 __device__ __forceinline__ void rs_level(float* v, int lane) {
@@ -711,26 +865,6 @@ __device__ __forceinline__ void rs_level(float* v, int lane) {
     v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
   }
   if constexpr (O > 1) rs_level<O / 2, L>(v, lane);
-}
-
-constexpr int rs_max(int n) { return ((n + 1) / 2 + 1) / 2 / 2 + ((((n + 1) / 2 + 1) / 2) & 1); }
-
-// The lane's slots after the reduce-scatter: *n of them from the returned one.
-template <int N>
-__device__ __forceinline__ int rs_slots(int lane, int* count) {
-  int n = N, real = N, slot = 0;
-  for (int o = kGroup / 2; o >= 1; o >>= 1) {
-    const int L = (n + 1) / 2;
-    if (lane & o) {
-      slot += L;
-      real = real - L > 0 ? real - L : 0;
-    } else {
-      real = real < L ? real : L;
-    }
-    n = L;
-  }
-  *count = real;
-  return slot;
 }
 
 // State of the reverse replay of a thread's two pixels (the halves of each
@@ -838,7 +972,7 @@ __device__ __forceinline__ void bwd_pair(BwdPix& p, const Pair& q, bool hitA, bo
   using LY = Layout<kLoss>;
   const float2 one = bc(1.f), zero = bc(0.f);
   const float2 al = sel2(hitA, hitB, q.alpha, zero);
-  const bool oA = hitA && q.objA, oB = hitB && q.objB;
+  const bool oA = hitA & q.objA, oB = hitB & q.objB;
   const float2 rd = sel2(oA, oB, q.rden, one);
   const float2 nu = sel2(oA, oB, q.nu, zero), nv = sel2(oA, oB, q.nv, zero);
   const float2 rom = rcp2(fma2(neg2(al), one, one));
@@ -858,7 +992,7 @@ __device__ __forceinline__ void bwd_pair(BwdPix& p, const Pair& q, bool hitA, bo
     dLdw = fma2(p.gN2, bc(e3.w), fma2(p.gN1, bc(e3.z), fma2(p.gN0, bc(e3.y), dLdw)));
     dLdw = fma2(p.gD2, fma2(z, E, neg2(EZ)), dLdw);
     dzv = fma2(w, fma2(p.gD2, E, p.gZ), dzv);
-    dzv = add2(dzv, sel2(hitA && k == p.medA, hitB && k == p.medB, p.gMed, zero));
+    dzv = add2(dzv, sel2(hitA & (k == p.medA), hitB & (k == p.medB), p.gMed, zero));
   }
   // alpha -> rho (zero where alpha is clamped at alpha_max): d alpha / d rho =
   // -alpha / 2; every derivative of rho below carries a factor 2, so
@@ -888,181 +1022,136 @@ __device__ __forceinline__ void bwd_pair(BwdPix& p, const Pair& q, bool hitA, bo
   const float2 ks = sel2(oA, oB, zero, bc(set.sinv));
   const float2 rx = fma2(ks, bc(q.dx), fma2(c1, bc(-e0.z), fma2(up, bc(e1.x), mul2(vp, bc(e1.z)))));
   const float2 ry = fma2(ks, q.dy, fma2(c1, bc(-e0.w), fma2(up, bc(e1.y), mul2(vp, bc(e1.w)))));
-  v[0] = hsum(dnu) * q.dx;
-  v[1] = dot2(dnu, q.dy);
-  v[2] = hsum(dnv) * q.dx;
-  v[3] = dot2(dnv, q.dy);
-  v[4] = hsum(dden) * q.dx;
-  v[5] = dot2(dden, q.dy);
-  v[6] = hsum(zr2);
-  v[7] = dot2(dzv, rd);
-  v[8] = hsum(nd[0]);
-  v[9] = dot2(w, p.gC[0][0]);
-  v[10] = dot2(w, p.gC[0][1]);
-  v[11] = dot2(w, p.gC[0][2]);
+  v[LY::nat(0)] = hsum(dnu) * q.dx;
+  v[LY::nat(1)] = dot2(dnu, q.dy);
+  v[LY::nat(2)] = hsum(dnv) * q.dx;
+  v[LY::nat(3)] = dot2(dnv, q.dy);
+  v[LY::nat(4)] = hsum(dden) * q.dx;
+  v[LY::nat(5)] = dot2(dden, q.dy);
+  v[LY::nat(6)] = dot2(nd[0], rx);
+  v[LY::nat(7)] = dot2(nd[0], ry);
+  v[LY::nat(8)] = hsum(zr2);
+  v[LY::nat(9)] = dot2(dzv, rd);
+  v[LY::nat(10)] = hsum(nd[0]);
+  v[LY::nat(11)] = dot2(w, p.gC[0][0]);
+  v[LY::nat(12)] = dot2(w, p.gC[0][1]);
+  v[LY::nat(13)] = dot2(w, p.gC[0][2]);
+  v[LY::nat(14)] = dot2(nd[1], rx);
+  v[LY::nat(15)] = dot2(nd[1], ry);
+  v[LY::nat(16)] = dot2(nd[2], rx);
+  v[LY::nat(17)] = dot2(nd[2], ry);
   if constexpr (!kLoss) {
-    v[12] = dot2(w, p.gN0);
-    v[13] = dot2(w, p.gN1);
-    v[14] = dot2(w, p.gN2);
-  }
-#pragma unroll
-  for (int s = 0; s < kMaxSets; ++s) {
-    v[LY::kRec + 2 * s] = dot2(nd[s], rx);
-    v[LY::kRec + 2 * s + 1] = dot2(nd[s], ry);
+    v[LY::nat(18)] = dot2(w, p.gN0);
+    v[LY::nat(19)] = dot2(w, p.gN1);
+    v[LY::nat(20)] = dot2(w, p.gN2);
   }
 }
 
-// Shared-memory staging of the backward (one batch of kBB entries).
-template <int kAcc, int kBB>
-struct BwdSmem {
-  float4 s0[kBB], s1[kBB], s2[kBB], s3[kBB], s4[kBB], s5[kBB];
-  uint16_t sm[kBB];
-  uint32_t sid[kBB];
-  float acc[kBB][kAcc];
-  uint8_t list[kThreads / 32][4][kListStride<kBB>];
-  int smax;
-};
+constexpr float kMinNormal = 1.17549435e-38f;
 
-// Reverse replay of entry kk of the batch (list position k) for a thread's two
-// pixels, each lane group its own entry: the pairs' gradients, reduced over
-// the group into the entry's accumulator.  active is false for the lanes of a
-// group whose list is used up.
-template <bool kLoss, int kN, int kAcc, int kBB>
-__device__ __forceinline__ void bwd_entry(BwdSmem<kAcc, kBB>& sh, bool active, int kk, int k, float lx, float2 ly,
-                                          BwdPix& p, int nsets, const SetDev& set, int lane, int myslot,
-                                          int nslots, unsigned& wentries, unsigned& wlanes) {
-  const float4 e0 = sh.s0[kk], jh = sh.s1[kk], e2 = sh.s2[kk], jl = sh.s4[kk];
-  const Pair q = eval_pair(lx, ly, e0, jh, jl, sh.s5[kk], e2.y, set);
-  const bool hitA = active && k < p.lastA && q.hitA, hitB = active && k < p.lastB && q.hitB;
-  const unsigned ballot = __ballot_sync(0xffffffffu, hitA || hitB);
-  if (ballot == 0u) return;
-  ++wentries;
-  wlanes += __popc(ballot);
-  float v[kN];
-  // Ji = Jh + Jl (FP32) for the chain rule
-  const float4 e1 = make_float4(jh.x + jl.x, jh.y + jl.y, jh.z + jl.z, jh.w + jl.w);
-  bwd_pair<kLoss>(p, q, hitA, hitB, e0, e1, e2, sh.s3[kk], k, nsets, set, v);
-  rs_level<kGroup / 2, kN>(v, lane);
-  if ((ballot >> (lane & 24)) & 0xffu) {
-    constexpr int kM = rs_max(kN);
-#pragma unroll
-    for (int i = 0; i < kM; ++i)
-      if (i < nslots && v[i] != 0.f) atomicAdd(&sh.acc[kk][myslot + i], v[i]);
-  }
+// The double with the value of a normal, finite v (a conversion instruction
+// runs at one warp per 17 clocks of an SM here, measured; these are five
+// integer operations).
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v);
+  const uint32_t hi = ((uint32_t)((int)b >> 3) & 0x8fffffffu) + 0x38000000u;
+  return __hiloint2double((int)hi, (int)(b << 29));
 }
 
-// kMinCtas: the CTAs per SM the register budget is sized for (5: 96
-// registers; 4: up to 128, for dense lists of small footprints).
-template <bool kLoss, int kMinCtas>
-__global__ void __launch_bounds__(kThreads, kMinCtas) blend_bwd_kernel(
+// One CTA per tile, one warp per 8 x 8 block.  Each lane group adds its sums
+// of an entry straight to the surfel's gradient row in global memory.  That
+// leaves the warps without a barrier, an accumulator to clear or a
+// compare-and-swap loop (which is what a shared-memory float addition
+// compiles to).  The rows are double: there are three to eight times as many
+// additions to a row as with one per (surfel, tile), and in float they cost
+// accuracy (the scale gradient's error against 64 bits went from 2.3e-5 to
+// 4.8e-5 of its norm on a 300k-surfel view).  5.5 million additions of a whole
+// row, about what a 1M-surfel view has, take 0.21 ms when nothing else runs
+// (0.12 ms in float).
+// Rows [lo, lo + rows) of the surfels are present; the other surfels' sums
+// are dropped (gs_backward makes several passes when it gets no memory for
+// all rows at once).
+// Four CTAs per SM (up to 128 registers): with five the code spills (720 ->
+// 767 us on the 1M-surfel view, 5.0 -> 5.7 ms for the four backwards of a 4M
+// training step).
+template <bool kLoss>
+__global__ void __launch_bounds__(kThreads, 4) blend_bwd_kernel(
     CamDev cam, SetDev set, const uint32_t* __restrict__ order, const float4* __restrict__ rec,
     const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
     const float* __restrict__ out, const int32_t* __restrict__ last, const int32_t* __restrict__ med,
-    AdjDev adj, float* __restrict__ grec, float* __restrict__ screen, int n,
-    unsigned long long* __restrict__ counters) {
+    AdjDev adj, double* __restrict__ grow, uint32_t lo, uint32_t rows, unsigned long long* __restrict__ counters) {
   using LY = Layout<kLoss>;
   constexpr int kN = LY::kN;
-  constexpr int kAcc = kN | 1;  // odd row stride: the flush's column reads are conflict-free
-  constexpr int kBatchB = batch_b(kMinCtas);
-  __shared__ BwdSmem<kAcc, kBatchB> sh;
+  __shared__ WarpSmem sh[kThreads / 32];
   const int tile = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
+  const int blk = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
   const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
-  const int warp = threadIdx.x >> 5;
   const float lx = (float)lxi + 0.5f;
   const float2 ly = make_float2((float)lyi + 0.5f, (float)(lyi + kRowStep) + 0.5f);
   const int2 rg = ranges[tile];
   const size_t HW = (size_t)cam.W * cam.H;
-  const int lane = threadIdx.x & 31;
   const int nsets = adj.n_sets;
-  int nslots;
-  const int myslot = rs_slots<kN>(lane, &nslots);
   const bool inA = px < cam.W && pyA < cam.H, inB = px < cam.W && pyB < cam.H;
   BwdPix p;
   bwd_init(p, bwd_load<kLoss>(inA, inA ? (size_t)pyA * cam.W + px : 0, HW, out, last, med, adj, set),
            bwd_load<kLoss>(inB, inB ? (size_t)pyB * cam.W + px : 0, HW, out, last, med, adj, set));
-  if (threadIdx.x == 0) sh.smax = 0;
-  __syncthreads();
-  atomicMax(&sh.smax, max(p.lastA, p.lastB));
-  __syncthreads();
-  const int maxlast = sh.smax;
   // the lane group's own last blended position: entries behind it are dead for
   // all of its pixels and are not visited
   int glast = max(p.lastA, p.lastB);
 #pragma unroll
   for (int o = kGroup / 2; o > 0; o >>= 1) glast = max(glast, __shfl_xor_sync(0xffffffffu, glast, o));
-  unsigned replayed = 0, wentries = 0, wlanes = 0;
-
-  for (int bend = maxlast; bend > 0; bend -= kBatchB) {
-    const int b0 = bend > kBatchB ? bend - kBatchB : 0;
-    const int nb = bend - b0;
-    __syncthreads();
-    for (int t = threadIdx.x; t < nb; t += kThreads) {
-      // every entry, also one that reaches no block: a group whose list is
-      // used up evaluates entry 0 with its pairs masked
-      const uint32_t s = vals[rg.x + b0 + t];
-      sh.sid[t] = s;
-      sh.sm[t] = masks[rg.x + b0 + t];
-      const Staged e = stage_entry(rec, s, tx0, ty0);
-      sh.s0[t] = e.s0;
-      sh.s1[t] = e.s1;
-      sh.s2[t] = e.s2;
-      sh.s3[t] = e.s3;
-      sh.s4[t] = e.s4;
-      sh.s5[t] = e.s5;
-    }
-    for (int i = threadIdx.x; i < nb * kAcc; i += kThreads) (&sh.acc[0][0])[i] = 0.f;
-    __syncthreads();
-    const int glen = group_lists<kBatchB>(sh.sm, nb, warp, lane, sh.list[warp], max(glast - b0, 0));
-    const uint8_t* list = sh.list[warp][lane >> 3];
-    if (counters) {
-      // the batch's entries before each pixel's last blended one that its
-      // group visits (performance counter)
-      for (int i = 0; i < glen; ++i) {
-        const int k = b0 + list[i];
-        replayed += (k < p.lastA ? 1u : 0u) + (k < p.lastB ? 1u : 0u);
-      }
-    }
-    // back to front, the groups side by side: a group whose list is used up
-    // takes part in the warp's votes and shuffles without a pair
-    const int longest = warp_longest(glen);
-    for (int i = 1; i <= longest; ++i) {
-      const bool active = i <= glen;
-      const int kk = active ? list[glen - i] : 0;
-      bwd_entry<kLoss, kN, kAcc, kBatchB>(sh, active, kk, b0 + kk, lx, ly, p, nsets, set, lane, myslot, nslots,
-                                          wentries, wlanes);
-    }
-    __syncthreads();
-    // flush this batch: one (surfel, tile) gradient record per entry, the
-    // centre gradient formed from set 0's screen gradient and Zc
-    for (int t = threadIdx.x; t < nb; t += kThreads) {
-      const uint32_t s = sh.sid[t];
-      float* g = grec + (size_t)s * kGradRec;
-      const float* x = sh.acc[t];
-      const float4 e0 = sh.s0[t];
-      float r[kGradRec];
+  const int wlast = max(max(__shfl_sync(0xffffffffu, glast, 0), __shfl_sync(0xffffffffu, glast, 8)),
+                        max(__shfl_sync(0xffffffffu, glast, 16), __shfl_sync(0xffffffffu, glast, 24)));
+  // where the lane's sums go within a row
+  const int r = lane & (kGroup - 1);
+  double* const dst = grow + r;
+  int off1 = -1, off2 = -1;
 #pragma unroll
-      for (int i = 0; i < 6; ++i) r[i] = x[i];
-      r[6] = fmaf(e0.z, x[6], x[LY::kRec]);
-      r[7] = fmaf(e0.w, x[6], x[LY::kRec + 1]);
-#pragma unroll
-      for (int i = 7; i < LY::kRec; ++i) r[i + 1] = x[i];
-      if (r[9] != 0.f) r[9] = r[9] / sh.s2[t].y;
-#pragma unroll
-      for (int i = 0; i < LY::kRec + 1; ++i)
-        if (r[i] != 0.f) atomicAdd(&g[i], r[i]);
-      if (screen) {
-        for (int st = 0; st < nsets; ++st) {
-          const float x0 = sh.acc[t][LY::kRec + 2 * st];
-          const float x1 = sh.acc[t][LY::kRec + 2 * st + 1];
-          float* sg = screen + ((size_t)st * n + s) * 2;
-          if (x0 != 0.f) atomicAdd(&sg[0], x0);
-          if (x1 != 0.f) atomicAdd(&sg[1], x1);
-        }
-      }
+  for (int x = 0; x < kGroup; ++x) {
+    if (x == r) {
+      off1 = LY::at(x, 1) - x;
+      off2 = LY::at(x, 2) - x;
     }
   }
+  const bool has1 = off1 + r >= 0, has2 = off2 + r >= 0;
+  unsigned replayed = 0, wentries = 0, wlanes = 0;
+  WarpSmem& sm = sh[blk];
+  walk_list<true>(sm, rec, masks + rg.x, vals + rg.x, 0, wlast, glast, tx0, ty0, blk, 0,
+                  [&](int k, int&) {
+    const float4 e0 = at16(sm.s0, k), jh = at16(sm.s1, k), e2 = at16(sm.s2, k), jl = at16(sm.s4, k);
+    const uint2 meta = at16(sm.meta, k);
+    const Pair q = eval_pair(lx, ly, e0, jh, jl, at16(sm.s5, k), e2.y, set);
+    const int pos = (int)meta.x;
+    const bool liveA = pos < p.lastA, liveB = pos < p.lastB;
+    const bool hitA = liveA & q.hitA, hitB = liveB & q.hitB;
+    replayed += (liveA ? 1u : 0u) + (liveB ? 1u : 0u);  // performance counter, as wentries and wlanes
+    const unsigned ballot = __ballot_sync(0xffffffffu, hitA | hitB);
+    if (ballot == 0u) return;
+    ++wentries;
+    wlanes += __popc(ballot);
+    float v[kN];
+    // Ji = Jh + Jl (FP32) for the chain rule
+    const float4 e1 = make_float4(jh.x + jl.x, jh.y + jl.y, jh.z + jl.z, jh.w + jl.w);
+    bwd_pair<kLoss>(p, q, hitA, hitB, e0, e1, e2, at16(sm.s3, k), pos, nsets, set, v);
+    rs_level<kGroup / 2, kN>(v, lane);
+    const uint32_t row = meta.y - lo;
+    if (((ballot >> (lane & 24)) & 0xffu) && row < rows) {
+      double* const d = dst + (size_t)row * grad_row_stride(kLoss);
+      const float a0 = fabsf(v[0]), a1 = has1 ? fabsf(v[1]) : 0.f, a2 = has2 ? fabsf(v[2]) : 0.f;
+      if (a0 + a1 + a2 < INFINITY) {
+        // zeros (and what is below the normal range) add nothing
+        if (a0 >= kMinNormal) atomicAdd(d, widen(v[0]));
+        if (a1 >= kMinNormal) atomicAdd(d + off1, widen(v[1]));
+        if (a2 >= kMinNormal) atomicAdd(d + off2, widen(v[2]));
+      } else {  // infinities and NaN go through as they are
+        atomicAdd(d, (double)v[0]);
+        if (has1) atomicAdd(d + off1, (double)v[1]);
+        if (has2) atomicAdd(d + off2, (double)v[2]);
+      }
+    }
+  });
   if (counters) {
     unsigned e = replayed;
 #pragma unroll
@@ -1083,9 +1172,9 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) blend_bwd_kernel(
 // sequence), but every pixel goes through the whole list: a pair that lies
 // in the surfel's support (rho <= rho_max) counts towards |P_k| even behind
 // the pixel's stop.  A blended pair adds alpha^gamma T^(1 - gamma), T the
-// transmittance in front of it.  Per entry the warp counts its support
-// pixels with ballots and sums its contributions with shuffles; the tile sums
-// them in shared memory and adds them to the surfel's totals once.
+// transmittance in front of it.  Per entry a lane group counts its support
+// pixels with ballots, sums its contributions with shuffles and adds both to
+// the surfel's totals.
 
 __device__ __forceinline__ float contrib_step(float& T, bool& stopped, bool hit, float alpha, const SetDev& set,
                                               float gamma) {
@@ -1102,76 +1191,44 @@ __device__ __forceinline__ float contrib_step(float& T, bool& stopped, bool hit,
   return c;
 }
 
-__global__ void __launch_bounds__(kThreads) blend_contrib_kernel(
+__global__ void __launch_bounds__(kThreads, 5) blend_contrib_kernel(
     CamDev cam, SetDev set, float gamma, const uint32_t* __restrict__ order,
     const float4* __restrict__ rec, const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals,
     const int2* __restrict__ ranges, float* __restrict__ csum, uint32_t* __restrict__ ccnt) {
-  __shared__ float4 s0[kBatch], s1[kBatch], s2[kBatch], s4[kBatch], s5[kBatch];
-  __shared__ uint32_t sid[kBatch];
-  __shared__ uint16_t sm[kBatch];
-  __shared__ float asum[kBatch];
-  __shared__ uint32_t acnt[kBatch];
-  __shared__ uint8_t lists[kThreads / 32][4][kListStride<kBatch>];
+  __shared__ WarpSmem sh[kThreads / 32];
   const int tile = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
   const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int blk = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float lx = (float)lxi + 0.5f;
   const float2 ly = make_float2((float)lyi + 0.5f, (float)(lyi + kRowStep) + 0.5f);
   const bool inA = px < cam.W && pyA < cam.H, inB = px < cam.W && pyB < cam.H;
   const int2 rg = ranges[tile];
-  const int len = rg.y - rg.x;
   float TA = 1.f, TB = 1.f;
   bool stA = !inA, stB = !inB;
-  for (int b0 = 0; b0 < len; b0 += kBatch) {
-    const int nb = min(kBatch, len - b0);
-    __syncthreads();
-    for (int t = threadIdx.x; t < nb; t += kThreads) {
-      const uint32_t sidx = vals[rg.x + b0 + t];
-      const uint16_t m = masks[rg.x + b0 + t];
-      sm[t] = m;
-      sid[t] = sidx;
-      asum[t] = 0.f;
-      acnt[t] = 0u;
-      if (m == 0u) continue;
-      const Staged e = stage_entry(rec, sidx, tx0, ty0);
-      s0[t] = e.s0;
-      s1[t] = e.s1;
-      s2[t] = e.s2;
-      s4[t] = e.s4;
-      s5[t] = e.s5;
-    }
-    __syncthreads();
-    const int glen = group_lists<kBatch>(sm, nb, warp, lane, lists[warp]);
-    const uint8_t* list = lists[warp][lane >> 3];
-    const int longest = warp_longest(glen);
-    for (int i = 0; i < longest; ++i) {
-      const bool active = i < glen;
-      const int k = active ? list[i] : 0;
-      const Pair q = eval_pair(lx, ly, s0[k], s1[k], s4[k], s5[k], s2[k].y, set);
-      const unsigned ba = __ballot_sync(0xffffffffu, active && inA && q.rho.x <= set.rho_max);
-      const unsigned bb = __ballot_sync(0xffffffffu, active && inB && q.rho.y <= set.rho_max);
-      if ((ba | bb) == 0u) continue;
-      const int sft = lane & 24;
-      const uint32_t cnt = (uint32_t)(__popc((ba >> sft) & 0xffu) + __popc((bb >> sft) & 0xffu));
-      float c = active ? contrib_step(TA, stA, q.hitA, q.alpha.x, set, gamma) +
-                             contrib_step(TB, stB, q.hitB, q.alpha.y, set, gamma) : 0.f;
+  WarpSmem& sm = sh[blk];
+  walk_list<false>(sm, rec, masks + rg.x, vals + rg.x, 0, rg.y - rg.x, 0, tx0, ty0, blk, 0,
+                   [&](int k, int&) {
+    const Pair q = eval_pair(lx, ly, at16(sm.s0, k), at16(sm.s1, k), at16(sm.s4, k), at16(sm.s5, k), at16(sm.s2, k).y,
+                             set);
+    const unsigned ba = __ballot_sync(0xffffffffu, inA & (q.rho.x <= set.rho_max));
+    const unsigned bb = __ballot_sync(0xffffffffu, inB & (q.rho.y <= set.rho_max));
+    if ((ba | bb) == 0u) return;
+    const int sft = lane & 24;
+    const uint32_t cnt = (uint32_t)(__popc((ba >> sft) & 0xffu) + __popc((bb >> sft) & 0xffu));
+    float c = contrib_step(TA, stA, q.hitA, q.alpha.x, set, gamma) +
+              contrib_step(TB, stB, q.hitB, q.alpha.y, set, gamma);
+    if (__any_sync(0xffffffffu, c != 0.f)) {
 #pragma unroll
       for (int o = kGroup / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-      if ((lane & 7) == 0 && cnt != 0u) {
-        atomicAdd(&acnt[k], cnt);
-        if (c != 0.f) atomicAdd(&asum[k], c);
-      }
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nb; t += kThreads) {
-      if (acnt[t] != 0u) {
-        atomicAdd(&ccnt[sid[t]], acnt[t]);
-        if (asum[t] != 0.f) atomicAdd(&csum[sid[t]], asum[t]);
-      }
+    if (cnt != 0u && (lane & 7) == 0) {
+      const uint32_t sid = at16(sm.meta, k).y;
+      atomicAdd(&ccnt[sid], cnt);
+      if (c != 0.f) atomicAdd(&csum[sid], c);
     }
-  }
+  });
 }
 
 }  // namespace
@@ -1182,8 +1239,13 @@ cudaError_t launch_blend_fwd(const CamDev& cam, const SetDev& set, const uint32_
                              unsigned long long* counters, cudaStream_t st) {
   const unsigned grid = (unsigned)cam.tiles_x * (unsigned)cam.tiles_y;
   ProfScope ps(kProfBlendFwd, st);
-  blend_fwd_kernel<<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, n_contrib,
-                                              last, med, counters, 0);
+  // the positions are the backward's; a render that keeps no frame does without
+  if (last || med)
+    blend_fwd_kernel<true><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, n_contrib, last,
+                                                      med, counters, 0);
+  else
+    blend_fwd_kernel<false><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, n_contrib, last,
+                                                       med, counters, 0);
   count_launch();
   return cudaGetLastError();
 }
@@ -1204,7 +1266,7 @@ cudaError_t launch_blend_fwd_split(const CamDev& cam, const SetDev& set, const u
   // the whole tiles, then the segments (grids sized for the bound, the device
   // count decides)
   count_launch(4);
-  blend_fwd_kernel<<<(unsigned)ntiles, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out,
+  blend_fwd_kernel<true><<<(unsigned)ntiles, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out,
                                                           n_contrib, last, med, counters, sb.lseg);
   seg_trans_kernel<<<sb.nseg_max, kThreads, 0, st>>>(cam, set, rec, masks, vals, ranges, sb.lseg, sb.seg_tile,
                                                      sb.seg_idx, sb.nseg, sb.trans);
@@ -1227,28 +1289,16 @@ cudaError_t launch_blend_fwd_batched(const BlendBatch& batch, int grid, cudaStre
 cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
                              const uint16_t* masks, const uint32_t* vals, const int2* ranges, const float* out,
                              const int32_t* last, const int32_t* med, const AdjDev& adj,
-                             float* grec, float* screen, int n, int64_t K, unsigned long long* counters,
-                             cudaStream_t st) {
+                             bool loss_layout, double* grow, uint32_t lo, uint32_t rows,
+                             unsigned long long* counters, cudaStream_t st) {
   const unsigned grid = (unsigned)cam.tiles_x * (unsigned)cam.tiles_y;
-  // the training loss drives set 0 through colour and inverse depth only and
-  // the other sets through colour: a leaner kernel for that layout
-  bool loss_layout = (adj.mask[0] & ~(GS_MASK_RGB | (1u << GS_PLANE_INVDEPTH))) == 0u;
-  for (int s = 1; s < adj.n_sets; ++s) loss_layout = loss_layout && (adj.mask[s] & ~GS_MASK_RGB) == 0u;
-  // long lists (many small footprints per tile) run faster with more
-  // registers per thread than with a fifth CTA per SM; both compute the same
-  const bool dense = K >= (int64_t)kDenseListLen * (int64_t)grid;
   ProfScope ps(kProfBlendBwd, st);
-#define GS_BWD(L, M)                                                                                           \
-  blend_bwd_kernel<L, M><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, last, med, \
-                                                    adj, grec, screen, n, counters)
-  if (loss_layout) {
-    if (dense) GS_BWD(true, 4);
-    else GS_BWD(true, 5);
-  } else {
-    if (dense) GS_BWD(false, 4);
-    else GS_BWD(false, 5);
-  }
-#undef GS_BWD
+  if (loss_layout)
+    blend_bwd_kernel<true><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, last, med, adj,
+                                                      grow, lo, rows, counters);
+  else
+    blend_bwd_kernel<false><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, last, med, adj,
+                                                       grow, lo, rows, counters);
   count_launch();
   return cudaGetLastError();
 }

@@ -391,11 +391,11 @@ bool launch_batch(gs_server* s, const std::vector<int>& ready, std::string* msg)
   b.work = s->work;
   cudaError_t e = nj ? cudaMemsetAsync(b.counter, 0, sizeof(unsigned), s->blend_st) : cudaSuccess;
   if (e == cudaSuccess && nj) {
-    // persistent grid: four CTAs per SM (the blend's occupancy), no more
+    // persistent grid: five CTAs per SM (the blend's occupancy), no more
     // CTAs than tiles
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
-    e = launch_blend_fwd_batched(b, std::max(1, std::min(4 * sms, tiles)), s->blend_st);
+    e = launch_blend_fwd_batched(b, std::max(1, std::min(5 * sms, tiles)), s->blend_st);
   }
   Batch bt;
   bt.ev = get_event(s);
