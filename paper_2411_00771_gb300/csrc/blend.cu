@@ -869,11 +869,10 @@ __device__ __forceinline__ void rs_level(float* v, int lane) {
 
 // State of the reverse replay of a thread's two pixels (the halves of each
 // pair): transmittance, suffix sums S of each adjoint set, the pixels'
-// adjoints, and (general layout) F = A_front - A_behind and G = Z_front -
-// Z_behind around the current entry (opacity and depth sums in front of and
-// behind it) for the distortion; gD2 is twice the distortion's adjoint.
+// adjoints, and (general layout) the running opacity A and depth sum Z with
+// their final values for the distortion; gD2 is twice the distortion's adjoint.
 struct BwdPix {
-  float2 T, F, G;
+  float2 T, A, Z, Af, Zf;
   float2 S[kMaxSets];
   float2 gC[kMaxSets][3];
   float2 gA, gZ, gI, gMed, gD2, gN0, gN1, gN2;
@@ -882,7 +881,7 @@ struct BwdPix {
 
 // One half of the state: the pixel at index pix (nothing when outside).
 struct BwdInit {
-  float T, F, G, S[kMaxSets], gC[kMaxSets][3], gA, gZ, gI, gMed, gD2, gN0, gN1, gN2;
+  float T, A, Z, S[kMaxSets], gC[kMaxSets][3], gA, gZ, gI, gMed, gD2, gN0, gN1, gN2;
   int last, med;
 };
 
@@ -892,7 +891,7 @@ __device__ __forceinline__ BwdInit bwd_load(bool inside, size_t pix, size_t HW, 
                                             const AdjDev& adj, const SetDev& set) {
   BwdInit p;
   p.T = 1.f;
-  p.F = p.G = 0.f;
+  p.A = p.Z = 0.f;
   p.gA = p.gZ = p.gI = p.gMed = p.gD2 = p.gN0 = p.gN1 = p.gN2 = 0.f;
   p.last = 0;
   p.med = -1;
@@ -918,8 +917,8 @@ __device__ __forceinline__ BwdInit bwd_load(bool inside, size_t pix, size_t HW, 
   if (m & (1u << 5)) p.gI = a[5 * HW + pix];
   if constexpr (!kLoss) {
     p.med = med[pix];
-    p.F = out[3 * HW + pix];
-    p.G = out[4 * HW + pix];
+    p.A = out[3 * HW + pix];
+    p.Z = out[4 * HW + pix];
     if (m & (1u << 3)) p.gA = a[3 * HW + pix];
     if (m & (1u << 4)) p.gZ = a[4 * HW + pix];
     if (m & (1u << 6)) p.gMed = a[6 * HW + pix];
@@ -933,8 +932,8 @@ __device__ __forceinline__ BwdInit bwd_load(bool inside, size_t pix, size_t HW, 
 
 __device__ __forceinline__ void bwd_init(BwdPix& p, const BwdInit& a, const BwdInit& b) {
   p.T = make_float2(a.T, b.T);
-  p.F = make_float2(a.F, b.F);
-  p.G = make_float2(a.G, b.G);
+  p.A = p.Af = make_float2(a.A, b.A);
+  p.Z = p.Zf = make_float2(a.Z, b.Z);
 #pragma unroll
   for (int s = 0; s < kMaxSets; ++s) {
     p.S[s] = make_float2(a.S[s], b.S[s]);
@@ -956,7 +955,7 @@ __device__ __forceinline__ void bwd_init(BwdPix& p, const BwdInit& a, const BwdI
 }
 
 __device__ __forceinline__ float hsum(float2 x) { return x.x + x.y; }
-__device__ __forceinline__ float dot2(float2 a, float2 b) { return hsum(mul2(a, b)); }
+__device__ __forceinline__ float dot2(float2 a, float2 b) { return fmaf(a.y, b.y, a.x * b.x); }
 
 // Gradients of the thread's two pairs at list position k, added up into v
 // (gradient-vector layout), and the pixels' replay state moved past the entry.
@@ -980,19 +979,20 @@ __device__ __forceinline__ void bwd_pair(BwdPix& p, const Pair& q, bool hitA, bo
   const float2 w = mul2(al, p.T);
   const float2 z = mul2(bc(e2.x), rd);
   const float2 rz = rcp2(z);
-  const float2 gIz = mul2(p.gI, rz);
-  float2 dLdw = fma2(p.gC[0][2], bc(e3.x), fma2(p.gC[0][1], bc(e2.w), fma2(p.gC[0][0], bc(e2.z), gIz)));
-  float2 dzv = mul2(mul2(w, gIz), neg2(rz));
+  float2 dLdw = fma2(p.gC[0][0], bc(e2.z), mul2(p.gC[0][1], bc(e2.w)));
+  dLdw = fma2(p.gI, rz, fma2(p.gC[0][2], bc(e3.x), dLdw));
+  float2 dzv = mul2(mul2(mul2(neg2(w), p.gI), rz), rz);
   if constexpr (!kLoss) {
-    const float2 E = add2(p.F, neg2(w)), EZ = fma2(neg2(w), z, p.G);
-    p.F = add2(E, neg2(w));
-    p.G = fma2(neg2(w), z, EZ);
-    dLdw = add2(dLdw, p.gA);
-    dLdw = fma2(p.gZ, z, dLdw);
+    const float2 Ap = add2(p.A, neg2(w)), Zp = fma2(neg2(w), z, p.Z);  // in front of this pair
+    const float2 Ab = add2(p.Af, neg2(p.A)), Zb = add2(p.Zf, neg2(p.Z));  // behind it
+    const float2 dD = fma2(neg2(z), Ab, add2(fma2(z, Ap, neg2(Zp)), Zb));
+    dLdw = fma2(p.gZ, z, add2(dLdw, p.gA));
     dLdw = fma2(p.gN2, bc(e3.w), fma2(p.gN1, bc(e3.z), fma2(p.gN0, bc(e3.y), dLdw)));
-    dLdw = fma2(p.gD2, fma2(z, E, neg2(EZ)), dLdw);
-    dzv = fma2(w, fma2(p.gD2, E, p.gZ), dzv);
+    dLdw = fma2(p.gD2, dD, dLdw);
+    dzv = fma2(w, fma2(p.gD2, add2(Ap, neg2(Ab)), p.gZ), dzv);
     dzv = add2(dzv, sel2(hitA & (k == p.medA), hitB & (k == p.medB), p.gMed, zero));
+    p.A = Ap;
+    p.Z = Zp;
   }
   // alpha -> rho (zero where alpha is clamped at alpha_max): d alpha / d rho =
   // -alpha / 2; every derivative of rho below carries a factor 2, so
@@ -1004,7 +1004,7 @@ __device__ __forceinline__ void bwd_pair(BwdPix& p, const Pair& q, bool hitA, bo
 #pragma unroll
   for (int s = 1; s < kMaxSets; ++s) {
     if (s < nsets) {
-      const float2 dw = fma2(p.gC[s][2], bc(e3.x), fma2(p.gC[s][1], bc(e2.w), mul2(p.gC[s][0], bc(e2.z))));
+      const float2 dw = fma2(p.gC[s][2], bc(e3.x), fma2(p.gC[s][0], bc(e2.z), mul2(p.gC[s][1], bc(e2.w))));
       nd[s] = mul2(fma2(p.T, dw, neg2(mul2(p.S[s], rom))), am);
       p.S[s] = fma2(w, dw, p.S[s]);
     } else {
@@ -1016,17 +1016,19 @@ __device__ __forceinline__ void bwd_pair(BwdPix& p, const Pair& q, bool hitA, bo
   const float2 u = mul2(nu, rd), vv = mul2(nv, rd);
   const float2 up = mul2(u, rd), vp = mul2(vv, rd);
   const float2 c1 = fma2(u, up, mul2(vv, vp));
-  const float2 zr2 = sel2(oA, oB, mul2(mul2(dzv, bc(e2.x)), mul2(rd, rd)), zero);
+  const float2 r2d = mul2(rd, rd), dzp = sel2(oA, oB, mul2(dzv, bc(e2.x)), zero);
+  const float2 zr2 = mul2(dzp, r2d);
   const float2 dnu = mul2(up, neg2(nd[0])), dnv = mul2(vp, neg2(nd[0]));
+  // d L / d rden, then through rden = 1 / (1 + e.d)
   const float2 dden = fma2(nd[0], c1, neg2(zr2));
   const float2 ks = sel2(oA, oB, zero, bc(set.sinv));
   const float2 rx = fma2(ks, bc(q.dx), fma2(c1, bc(-e0.z), fma2(up, bc(e1.x), mul2(vp, bc(e1.z)))));
   const float2 ry = fma2(ks, q.dy, fma2(c1, bc(-e0.w), fma2(up, bc(e1.y), mul2(vp, bc(e1.w)))));
-  v[LY::nat(0)] = hsum(dnu) * q.dx;
+  v[LY::nat(0)] = dot2(dnu, bc(q.dx));
   v[LY::nat(1)] = dot2(dnu, q.dy);
-  v[LY::nat(2)] = hsum(dnv) * q.dx;
+  v[LY::nat(2)] = dot2(dnv, bc(q.dx));
   v[LY::nat(3)] = dot2(dnv, q.dy);
-  v[LY::nat(4)] = hsum(dden) * q.dx;
+  v[LY::nat(4)] = dot2(dden, bc(q.dx));
   v[LY::nat(5)] = dot2(dden, q.dy);
   v[LY::nat(6)] = dot2(nd[0], rx);
   v[LY::nat(7)] = dot2(nd[0], ry);
