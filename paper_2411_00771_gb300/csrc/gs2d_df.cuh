@@ -104,6 +104,67 @@ __device__ __forceinline__ df df_sqrt(df a) {
   return df_make(s) + r * __frcp_rn(2.f * s);
 }
 
+// Two double-floats at a time on the packed FP32 instructions: each half of a
+// pair gets exactly the operations, in the order, of the forms above, so a
+// pair's values are those of the single forms bit for bit.
+struct df2 {
+  float2 hi, lo;
+};
+
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ df2 df2_make(df x, df y) { return {make_float2(x.hi, y.hi), make_float2(x.lo, y.lo)}; }
+__device__ __forceinline__ df2 df2_both(df a) { return {both(a.hi), both(a.lo)}; }
+__device__ __forceinline__ df df2_x(const df2& a) { return {a.hi.x, a.lo.x}; }
+__device__ __forceinline__ df df2_y(const df2& a) { return {a.hi.y, a.lo.y}; }
+__device__ __forceinline__ float2 df2_float(const df2& a) { return __fadd2_rn(a.hi, a.lo); }
+
+__device__ __forceinline__ df2 two_sum(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b);
+  const float2 bb = __fadd2_rn(s, neg2(a));
+  const float2 e = __fadd2_rn(__fadd2_rn(a, neg2(__fadd2_rn(s, neg2(bb)))), __fadd2_rn(b, neg2(bb)));
+  return {s, e};
+}
+__device__ __forceinline__ df2 fast_two_sum(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b);
+  return {s, __fadd2_rn(b, neg2(__fadd2_rn(s, neg2(a))))};
+}
+__device__ __forceinline__ df2 two_prod(float2 a, float2 b) {
+  const float2 p = __fmul2_rn(a, b);
+  return {p, __ffma2_rn(a, b, neg2(p))};
+}
+__device__ __forceinline__ df2 operator-(const df2& a) { return {neg2(a.hi), neg2(a.lo)}; }
+__device__ __forceinline__ df2 operator+(const df2& a, const df2& b) {
+  const df2 s = two_sum(a.hi, b.hi);
+  const df2 t = two_sum(a.lo, b.lo);
+  const df2 r = fast_two_sum(s.hi, __fadd2_rn(s.lo, t.hi));
+  return fast_two_sum(r.hi, __fadd2_rn(r.lo, t.lo));
+}
+__device__ __forceinline__ df2 operator-(const df2& a, const df2& b) { return a + (-b); }
+__device__ __forceinline__ df2 operator+(const df2& a, float2 b) {
+  const df2 s = two_sum(a.hi, b);
+  return fast_two_sum(s.hi, __fadd2_rn(s.lo, a.lo));
+}
+__device__ __forceinline__ df2 operator*(const df2& a, const df2& b) {
+  const df2 p = two_prod(a.hi, b.hi);
+  return fast_two_sum(p.hi, __ffma2_rn(a.hi, b.lo, __ffma2_rn(a.lo, b.hi, p.lo)));
+}
+__device__ __forceinline__ df2 operator*(const df2& a, float2 b) {
+  const df2 p = two_prod(a.hi, b);
+  return fast_two_sum(p.hi, __ffma2_rn(a.lo, b, p.lo));
+}
+__device__ __forceinline__ df2 operator*(const df2& a, df b) { return a * df2_both(b); }
+// 2 a: exact
+__device__ __forceinline__ df2 twice(const df2& a) { return {__fadd2_rn(a.hi, a.hi), __fadd2_rn(a.lo, a.lo)}; }
+__device__ __forceinline__ df twice(df a) { return {__fadd_rn(a.hi, a.hi), __fadd_rn(a.lo, a.lo)}; }
+__device__ __forceinline__ df2 df_sqrt(const df2& a) {
+  const float2 s = make_float2(__fsqrt_rn(a.hi.x), __fsqrt_rn(a.hi.y));
+  const df2 r = a - two_prod(s, s);
+  const df2 q = df2{s, both(0.f)} + r * make_float2(__frcp_rn(2.f * s.x), __frcp_rn(2.f * s.y));
+  const bool px = a.hi.x > 0.f, py = a.hi.y > 0.f;
+  return {make_float2(px ? q.hi.x : 0.f, py ? q.hi.y : 0.f), make_float2(px ? q.lo.x : 0.f, py ? q.lo.y : 0.f)};
+}
+
 // floor and ceil of hi + lo: when hi is not an integer, |lo| <= ulp(hi)/2
 // cannot carry the sum across one.
 __device__ __forceinline__ float df_floor(df a) {

@@ -178,6 +178,7 @@ __device__ __forceinline__ float4 load_quat(const ParamsDev& P, int n) {
     return make_float4(h2f((uint16_t)(v.x & 0xFFFFu)), h2f((uint16_t)(v.x >> 16)), h2f((uint16_t)(v.y & 0xFFFFu)),
                        h2f((uint16_t)(v.y >> 16)));
   }
+  if (((uintptr_t)P.quat & 15u) == 0) return reinterpret_cast<const float4*>(P.quat)[n];
   return make_float4(P.quat[4 * n], P.quat[4 * n + 1], P.quat[4 * n + 2], P.quat[4 * n + 3]);
 }
 __device__ __forceinline__ float2 load_scale(const ParamsDev& P, int n) {
@@ -185,6 +186,7 @@ __device__ __forceinline__ float2 load_scale(const ParamsDev& P, int n) {
     const uint32_t v = *reinterpret_cast<const uint32_t*>(P.scale16 + 2 * (size_t)n);
     return make_float2(h2f((uint16_t)(v & 0xFFFFu)), h2f((uint16_t)(v >> 16)));
   }
+  if (((uintptr_t)P.scale & 7u) == 0) return reinterpret_cast<const float2*>(P.scale)[n];
   return make_float2(P.scale[2 * n], P.scale[2 * n + 1]);
 }
 __device__ __forceinline__ float load_opacity(const ParamsDev& P, int n) {

@@ -165,35 +165,9 @@ __global__ void __launch_bounds__(256) compact_kernel(const uint32_t* __restrict
   if (i < n && flags[i]) cand[pos[i]] = (uint32_t)i;
 }
 
-// Double-float vector helpers for the preprocess geometry.
-struct D3 {
-  df x, y, z;
-};
-__device__ __forceinline__ df dot3(const D3& a, const D3& b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
-// R v with R the camera rotation in double-float (row-major)
-__device__ __forceinline__ D3 cam_rot(const CamDev& c, const D3& v) {
-  D3 r;
-  df* o[3] = {&r.x, &r.y, &r.z};
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const df r0 = df_make(c.Rf[3 * i], c.Rlo[3 * i]);
-    const df r1 = df_make(c.Rf[3 * i + 1], c.Rlo[3 * i + 1]);
-    const df r2 = df_make(c.Rf[3 * i + 2], c.Rlo[3 * i + 2]);
-    *o[i] = r0 * v.x + r1 * v.y + r2 * v.z;
-  }
-  return r;
-}
-__device__ __forceinline__ D3 cam_rot(const CamDev& c, float x, float y, float z) {
-  D3 r;
-  df* o[3] = {&r.x, &r.y, &r.z};
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const df r0 = df_make(c.Rf[3 * i], c.Rlo[3 * i]);
-    const df r1 = df_make(c.Rf[3 * i + 1], c.Rlo[3 * i + 1]);
-    const df r2 = df_make(c.Rf[3 * i + 2], c.Rlo[3 * i + 2]);
-    *o[i] = r0 * x + r1 * y + r2 * z;
-  }
-  return r;
+// Element (i, k) of the camera rotation, double-float.
+__device__ __forceinline__ df cam_r(const CamDev& c, int i, int k) {
+  return df_make(c.Rf[3 * i + k], c.Rlo[3 * i + k]);
 }
 
 // Stage 2 (candidates only): the definition's preprocess, the footprint's
@@ -202,190 +176,336 @@ __device__ __forceinline__ D3 cam_rot(const CamDev& c, float x, float y, float z
 // homography, the bound of {rho <= rho_max} and its tile rectangle) is
 // computed in double-float (about 48 bits; the FP64 pipe is too slow for a
 // million surfels per view), colour and normal in FP32.
-template <int DEG>
-__global__ void __launch_bounds__(256) preprocess_main_kernel(ParamsDev P, CamDev cam, SetDev set,
-                                                              const uint32_t* __restrict__ cand,
-                                                              const uint32_t* __restrict__ ncand,
-                                                              float4* __restrict__ rec,
-                                                              uint2* __restrict__ rect,
-                                                              uint32_t* __restrict__ tcount,
-                                                              uint32_t* __restrict__ dkey,
-                                                              uint32_t* __restrict__ idx,
-                                                              RowGeom* __restrict__ geom) {
+
+// Geometry of surfel n: its tile rectangle and count, depth key, and the blend
+// record R (with the given colour) followed by the footprint; false (and no
+// record) when it is not visible.
+__device__ __forceinline__ bool surfel_geometry(const ParamsDev& P, const CamDev& cam, const SetDev& set, int n,
+                                                const df& rf, float rff, uint2* rect, uint32_t* tcount,
+                                                uint32_t* dkey, const float (&col)[3], float4* R) {
+  const float4 q4 = load_quat(P, n);
+  const df2 sa = two_prod(make_float2(q4.x, q4.y), make_float2(q4.x, q4.y));
+  const df2 sb = two_prod(make_float2(q4.z, q4.w), make_float2(q4.z, q4.w));
+  const df qn2 = df2_x(sa) + df2_y(sa) + df2_x(sb) + df2_y(sb);
+  if (!df_pos(qn2)) return false;
+  const df iq = df_rsqrt(qn2);
+  const df2 qwx = df2_both(iq) * make_float2(q4.x, q4.y), qyz = df2_both(iq) * make_float2(q4.z, q4.w);
+  const df qw = df2_x(qwx), qx = df2_y(qwx), qy = df2_x(qyz), qz = df2_y(qyz);
+  // columns of the rotation of the unit quaternion, the first two as pairs
+  // t[k] = (r1_k, r2_k)
+  const df one = df_make(1.f);
+  const df2 m1 = df2_make(qx, qw) * df2_make(qy, qz);  // x y, w z
+  const df2 m2 = df2_make(qx, qw) * df2_make(qz, qy);  // x z, w y
+  const df2 m3 = df2_make(qy, qw) * df2_make(qz, qx);  // y z, w x
+  const df2 xxyy = df2_make(qx, qy) * df2_make(qx, qy);
+  const df zz = qz * qz;
+  const df2 o1 = twice(df2_both(df2_x(m1)) + df2_make(df2_y(m1), -df2_y(m1)));  // r1_y, r2_x
+  const df2 o2 = twice(df2_both(df2_x(m2)) + df2_make(-df2_y(m2), df2_y(m2)));  // r1_z, r3_x
+  const df2 o3 = twice(df2_both(df2_x(m3)) + df2_make(df2_y(m3), -df2_y(m3)));  // r2_z, r3_y
+  const df2 dg = df2_both(one) - twice(df2_make(df2_y(xxyy), df2_x(xxyy)) + df2_both(zz));  // r1_x, r2_y
+  const df2 t[3] = {df2_make(df2_x(dg), df2_y(o1)), df2_make(df2_x(o1), df2_y(dg)), df2_make(df2_x(o2), df2_x(o3))};
+  const df r3[3] = {df2_y(o2), df2_y(o3), one - twice(df2_x(xxyy) + df2_y(xxyy))};
+  // camera space: centre and normal as pairs (x, y) with z apart, the
+  // tangents as pairs (t_u, t_v) per component
+  const float mu[3] = {P.mu[3 * n], P.mu[3 * n + 1], P.mu[3 * n + 2]};
+  const df2 rxy0 = df2_make(cam_r(cam, 0, 0), cam_r(cam, 1, 0)), rxy1 = df2_make(cam_r(cam, 0, 1), cam_r(cam, 1, 1)),
+            rxy2 = df2_make(cam_r(cam, 0, 2), cam_r(cam, 1, 2));
+  const df rz0 = cam_r(cam, 2, 0), rz1 = cam_r(cam, 2, 1), rz2 = cam_r(cam, 2, 2);
+  const df2 pxy = rxy0 * both(mu[0]) + rxy1 * both(mu[1]) + rxy2 * both(mu[2]) +
+                  df2_make(df_make(cam.tf[0], cam.tlo[0]), df_make(cam.tf[1], cam.tlo[1]));
+  const df pz = rz0 * mu[0] + rz1 * mu[1] + rz2 * mu[2] + df_make(cam.tf[2], cam.tlo[2]);
+  const df2 nxy = rxy0 * r3[0] + rxy1 * r3[1] + rxy2 * r3[2];
+  const df nz = rz0 * r3[0] + rz1 * r3[1] + rz2 * r3[2];
+  const float2 s2 = load_scale(P, n);
+  df2 ab[3];  // (a, b) = (s_u t_u, s_v t_v)
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    ab[i] = (df2_both(cam_r(cam, i, 0)) * t[0] + df2_both(cam_r(cam, i, 1)) * t[1] + df2_both(cam_r(cam, i, 2)) * t[2]) *
+            s2;
+  }
+  const df2 zsq = ab[2] * ab[2];
+  const df zmin = pz - df_sqrt((df2_x(zsq) + df2_y(zsq)) * set.rho_max);
+  if (!df_pos(zmin - set.near_plane)) return false;
+  const df iz = df_rcp(pz);
+  const df2 xyi = pxy * iz;
+  const df fx = df_make(cam.fxf, cam.fxlo), fy = df_make(cam.fyf, cam.fylo);
+  const df2 c = df2_make(fx, fy) * xyi + df2_make(df_make(cam.cxf, cam.cxlo), df_make(cam.cyf, cam.cylo));
+  const df cx = df2_x(c), cy = df2_y(c);
+  const df2 J1 = df2_both(fx) * (ab[0] - ab[2] * df2_x(xyi)) * iz;  // J11, J12
+  const df2 J2 = df2_both(fy) * (ab[1] - ab[2] * df2_y(xyi)) * iz;  // J21, J22
+  const df2 w = ab[2] * iz;
+  // bounding box of {rho_obj <= rho_max} in offsets from c: dual conic of
+  // the centred homography H = [[J, 0], [w^T, 1]]; scaled to C33 = 1 it is
+  // [[e0 e0^T - G, e0], [e0^T, 1]] for the ellipse (d - e0)^T G^-1 (d - e0) <= 1
+  const float2 rm = both(set.rho_max);
+  const df2 v11 = J1 * J1, v22 = J2 * J2, v12 = J1 * J2, v13 = J1 * w, v23 = J2 * w, v33 = w * w;
+  const df2 Cd = (df2_make(df2_x(v11), df2_x(v22)) + df2_make(df2_y(v11), df2_y(v22))) * rm;  // C11, C22
+  const df2 C3 = (df2_make(df2_x(v13), df2_x(v23)) + df2_make(df2_y(v13), df2_y(v23))) * rm;  // C13, C23
+  const df2 Co = (df2_make(df2_x(v12), df2_x(v33)) + df2_make(df2_y(v12), df2_y(v33))) * rm;
+  const df C12 = df2_x(Co), C33 = df2_y(Co) - 1.f;
+  const df2 disc = C3 * C3 - Cd * C33;
+  const df zero = df_make(0.f);
+  const df2 ext = df_sqrt(df2_make(df_max(df2_x(disc), zero), df_max(df2_y(disc), zero)));
+  const df i33 = df_rcp(C33);
+  const df2 e0v = (C3 - ext) * i33, e1v = (C3 + ext) * i33;
+  const df x0 = df2_x(e0v), x1 = df2_x(e1v), y0 = df2_y(e0v), y1 = df2_y(e1v);
+  const df2 cmin = c + df2_make(df_min(df_min(x0, x1), -rf), df_min(df_min(y0, y1), -rf));
+  const df2 cmax = c + df2_make(df_max(df_max(x0, x1), rf), df_max(df_max(y0, y1), rf));
+  const df2 clo = cmin + both(-0.5f), chi = cmax + both(-0.5f);
+  float ilo = df_ceil(df2_x(clo)), ihi = df_floor(df2_x(chi));
+  float jlo = df_ceil(df2_y(clo)), jhi = df_floor(df2_y(chi));
+  ilo = fmaxf(ilo, 0.f); jlo = fmaxf(jlo, 0.f);
+  ihi = fminf(ihi, (float)(cam.W - 1)); jhi = fminf(jhi, (float)(cam.H - 1));
+  if (!(ilo <= ihi && jlo <= jhi)) return false;
+  RowGeom gm;
+  {
+    const df2 e0 = C3 * i33;
+    const df2 gd = e0 * e0 - Cd * i33;
+    const df g11 = df2_x(gd), g22 = df2_y(gd), g12 = df2_x(e0) * df2_y(e0) - C12 * i33;
+    const float2 e0f = df2_float(e0);
+    gm.cx_hi = cx.hi; gm.cx_lo = cx.lo;
+    gm.cy_hi = cy.hi; gm.cy_lo = cy.lo;
+    gm.e0x = e0f.x; gm.e0y = e0f.y;
+    if (df_pos(g11) && df_pos(g22)) {
+      // rounded once to FP32; the row rule's margin covers their error
+      const df dg = g11 * g22 - g12 * g12;
+      const float det = df_pos(dg) ? df_float(dg) : 0.f;
+      const float f11 = df_float(g11), f12 = df_float(g12), f22 = df_float(g22);
+      gm.hy = sqrtf(f22);
+      gm.t = f12 * rsqrtf(f11);
+      gm.slope = f12 / f22;
+      gm.wsc = sqrtf(det) / f22;
+    } else {
+      gm.hy = -1.f; gm.t = 0.f; gm.slope = 0.f; gm.wsc = 0.f;  // disk only
+    }
+  }
+  gm.ilo = (int)ilo; gm.ihi = (int)ihi; gm.jlo = (int)jlo; gm.jhi = (int)jhi;
+  const int tx0 = gm.ilo / kTile, tx1 = gm.ihi / kTile + 1;
+  const int ty0 = gm.jlo / kTile, ty1 = gm.jhi / kTile + 1;
+  *rect = make_uint2((uint32_t)tx0 | ((uint32_t)ty0 << 16), (uint32_t)tx1 | ((uint32_t)ty1 << 16));
+  uint32_t cnt = 0;
+  for (int ty = ty0; ty < ty1; ++ty) {
+    int a0, a1;
+    if (row_tiles(gm, ty, rff, &a0, &a1)) cnt += (uint32_t)(a1 - a0);
+  }
+  if (cnt == 0) return false;
+  *tcount = cnt;
+  const float pzf = df_float(pz);
+  *dkey = __float_as_uint(pzf);
+  const df2 dt = J1 * df2_make(df2_y(J2), df2_x(J2));  // J11 J22, J12 J21
+  const df det = df2_x(dt) - df2_y(dt);
+  // Ji, split for the blends' exact tile-relative evaluation of (u, v):
+  // on a power-of-two grid 2^g chosen so that |Ji d| < 2^(g+22) for every
+  // pixel and tile origin of the surfel's tile rectangle, Jh (multiples of
+  // 2^(g+1)) and nref_h (Ji (o_ref - c) on multiples of 2^g, o_ref the
+  // rectangle's first tile origin) make every partial sum of
+  // nref_h + Jh (o - o_ref) + Jh (lx, ly) exact in FP32; the low parts Jl =
+  // Ji - Jh and nref_l = Ji (o_ref - c) - nref_h (both about 2^g) carry the
+  // rest (see blend.cu).
+  float4 jh, jl, nref;  // nref = (nref_h.u, nref_h.v, nref_l.u, nref_l.v)
+  float ugrid = 1.f;    // 2^-g
+  float2 ef;
+  const float orx = (float)(tx0 * kTile), ory = (float)(ty0 * kTile);
+  if (df_nonzero(det)) {
+    const df id = df_rcp(det);
+    // columns of Ji: (i11, i21), (i12, i22)
+    const df2 k1 = df2_make(df2_y(J2), -df2_x(J2)) * id, k2 = df2_make(-df2_y(J1), df2_x(J1)) * id;
+    const float2 k1f = df2_float(k1), k2f = df2_float(k2);
+    const float4 r1f = make_float4(k1f.x, k2f.x, k1f.y, k2f.y);
+    const float2 k1l = df2_float(k1 + neg2(k1f)), k2l = df2_float(k2 + neg2(k2f));
+    const float4 r5f = make_float4(k1l.x, k2l.x, k1l.y, k2l.y);
+    const df2 ew = df2_make(df2_x(k1), df2_x(k2)) * df2_x(w) + df2_make(df2_y(k1), df2_y(k2)) * df2_y(w);
+    ef = df2_float(-ew);
+    const df2 d0 = two_sum(make_float2(orx, ory), neg2(c.hi)) + neg2(c.lo);
+    const df2 nuv = k1 * df2_x(d0) + k2 * df2_y(d0);
+    const df nu0 = df2_x(nuv), nv0 = df2_y(nuv);
+    const float Dx = fmaxf(fabsf(orx - cx.hi), fabsf((float)(tx1 * kTile) - cx.hi));
+    const float Dy = fmaxf(fabsf(ory - cy.hi), fabsf((float)(ty1 * kTile) - cy.hi));
+    const float Rs = fmaxf(fabsf(r1f.x) + fabsf(r1f.y), fabsf(r1f.z) + fabsf(r1f.w));
+    const float M = __fmul_rn(__fmul_rn(Rs, fmaxf(Dx, Dy) + 2.f), 1.0009765625f);
+    const int E = min(max(((__float_as_int(M) >> 23) & 0xff) - 127, -100), 100);  // M < 2^(E+1)
+    const int g = E - 21;
+    const float ug = __int_as_float((127 - g) << 23), dg = __int_as_float((127 + g) << 23);
+    const float uj = __int_as_float((126 - g) << 23), dj = __int_as_float((128 + g) << 23);
+    jh = make_float4(__fmul_rn(rintf(__fmul_rn(r1f.x, uj)), dj), __fmul_rn(rintf(__fmul_rn(r1f.y, uj)), dj),
+                     __fmul_rn(rintf(__fmul_rn(r1f.z, uj)), dj), __fmul_rn(rintf(__fmul_rn(r1f.w, uj)), dj));
+    jl = make_float4(__fadd_rn(__fsub_rn(r1f.x, jh.x), r5f.x), __fadd_rn(__fsub_rn(r1f.y, jh.y), r5f.y),
+                     __fadd_rn(__fsub_rn(r1f.z, jh.z), r5f.z), __fadd_rn(__fsub_rn(r1f.w, jh.w), r5f.w));
+    const float uh = __fmul_rn(rintf(__fmul_rn(nu0.hi, ug)), dg);
+    const float vh = __fmul_rn(rintf(__fmul_rn(nv0.hi, ug)), dg);
+    nref = make_float4(uh, vh, __fadd_rn(__fsub_rn(nu0.hi, uh), nu0.lo), __fadd_rn(__fsub_rn(nv0.hi, vh), nv0.lo));
+    ugrid = ug;
+  } else {
+    // edge-on disk: no object-space footprint (Ji d and rho_obj are NaN,
+    // the screen filter decides; Ji itself stays finite for the backward)
+    const float qnan = __int_as_float(0x7fffffff);
+    jh = jl = make_float4(0.f, 0.f, 0.f, 0.f);
+    nref = make_float4(qnan, qnan, 0.f, 0.f);
+    ef = make_float2(0.f, 0.f);
+  }
+  const df2 np = nxy * pxy;
+  const float sg = df_pos(df2_x(np) + df2_y(np) + nz * pz) ? -1.f : 1.f;
+  const float2 nf = df2_float(nxy);
+  R[0] = make_float4(cx.hi, cy.hi, cx.lo, cy.lo);
+  R[1] = jh;
+  R[2] = make_float4(ef.x, ef.y, pzf, load_opacity(P, n));
+  R[3] = make_float4(col[0], col[1], col[2], sg * nf.x);
+  R[4] = make_float4(sg * nf.y, sg * df_float(nz), nref.x, nref.y);
+  R[5] = jl;
+  // the first tile of the rectangle (tile indices, packed) and 2^-g, g the grid's exponent
+  R[6] = make_float4(nref.z, nref.w, __uint_as_float((uint32_t)tx0 | ((uint32_t)ty0 << 16)), ugrid);
+  *reinterpret_cast<RowGeom*>(R + kRecF4) = gm;
+  return true;
+}
+
+// A lane's own loads of its SH row and stores of its record would each touch
+// 32 cache lines per instruction (48 loads and 21 stores at degree 3).  So a
+// warp moves the rows of its 32 candidates together: SH rows into shared
+// memory by asynchronous copies of kPiece bytes, consecutive lanes on
+// consecutive pieces; records and footprints into shared memory and out piece
+// by piece.  The colour comes first, so that only its three values are held
+// over the geometry.  kPiece 0 (rows that are not a whole number of aligned
+// 4-byte words) reads the SH rows directly.
+//
+// What bounds it is the straight run of about 4000 instructions per surfel:
+// longer than the instruction cache, so warps wait for instructions first
+// (fetch was the top stall reason) and on the double-float chains next.
+// Hence the geometry in pairs (half the instructions of two of everything),
+// the barriers at both halves of the loop body, which keep a block's warps on
+// the same instructions, and small blocks.  Degree 3, kernel time of a
+// 1M-surfel 900p view / four views of 4M / one 4K view of 8M in binary16, us:
+//   lanes on their own rows, single forms           131 / 1431 / 888
+//   rows moved by warps, 768 threads, no barriers   140 / 1400 / 937
+//   256 threads x 3, barriers                       126 / 1265 / 797
+//   and pairs                                       117 / 1160 / 762
+//   and 128 threads x 7 (x 6, x 8: 1171, 1142)      114 / 1125 / 721
+constexpr int kMainThreads = 128;
+constexpr int kMainCtas = 7;
+constexpr int kOutRow = 176;  // record (112 bytes) and footprint (56), padded to an odd number of 16-byte units
+template <int DEG, bool kHalf, int kPiece>
+struct ShRow {
+  static constexpr int kBytes = (DEG + 1) * (DEG + 1) * 3 * (kHalf ? 2 : 4);
+  static constexpr int kPieces = kPiece ? kBytes / (kPiece ? kPiece : 1) : 0;
+  // an odd number of pieces between staged rows keeps the lanes' reads apart
+  static constexpr int kStride = (kPieces | 1) * kPiece;
+  static constexpr int kWarpBytes = 32 * (kStride > kOutRow ? kStride : kOutRow);
+};
+template <int kBytes>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if constexpr (kBytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+
+template <int DEG, bool kHalf, int kPiece>
+__global__ void __launch_bounds__(kMainThreads, kMainCtas)
+    preprocess_main_kernel(ParamsDev P, CamDev cam, SetDev set, const uint32_t* __restrict__ cand,
+                           const uint32_t* __restrict__ ncand, float4* __restrict__ rec, uint2* __restrict__ rect,
+                           uint32_t* __restrict__ tcount, uint32_t* __restrict__ dkey, uint32_t* __restrict__ idx,
+                           RowGeom* __restrict__ geom) {
+  using SR = ShRow<DEG, kHalf, kPiece>;
+  constexpr unsigned kFull = 0xffffffffu;
+  constexpr int K = (DEG + 1) * (DEG + 1);
+  extern __shared__ __align__(16) unsigned char stage_all[];
+  const int lane = threadIdx.x & 31;
+  unsigned char* const stage = stage_all + (threadIdx.x >> 5) * SR::kWarpBytes;
   const uint32_t total = *ncand;
   const df rf = df_sqrt(df_make(set.rho_max) / df_make(set.sinv));
   const float rff = df_float(rf);
-  const df fx = df_make(cam.fxf, cam.fxlo), fy = df_make(cam.fyf, cam.fylo);
-  const df cx0 = df_make(cam.cxf, cam.cxlo), cy0 = df_make(cam.cyf, cam.cylo);
-  for (uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x; ci < total; ci += gridDim.x * blockDim.x) {
-    const int n = (int)cand[ci];
-    idx[ci] = (uint32_t)n;
-    dkey[ci] = 0xFFFFFFFFu;  // not visible unless set below
-    const float4 q4 = load_quat(P, n);
-    const float qw0 = q4.x, qx0 = q4.y, qy0 = q4.z, qz0 = q4.w;
-    const df qn2 = two_prod(qw0, qw0) + two_prod(qx0, qx0) + two_prod(qy0, qy0) + two_prod(qz0, qz0);
-    if (!df_pos(qn2)) continue;
-    const df iq = df_rsqrt(qn2);
-    const df qw = iq * qw0, qx = iq * qx0, qy = iq * qy0, qz = iq * qz0;
-    // columns of the rotation of the unit quaternion
-    const df one = df_make(1.f);
-    const D3 r1 = {one - 2.f * (qy * qy + qz * qz), 2.f * (qx * qy + qw * qz), 2.f * (qx * qz - qw * qy)};
-    const D3 r2 = {2.f * (qx * qy - qw * qz), one - 2.f * (qx * qx + qz * qz), 2.f * (qy * qz + qw * qx)};
-    const D3 r3 = {2.f * (qx * qz + qw * qy), 2.f * (qy * qz - qw * qx), one - 2.f * (qx * qx + qy * qy)};
-    const float mux = P.mu[3 * n], muy = P.mu[3 * n + 1], muz = P.mu[3 * n + 2];
-    D3 p = cam_rot(cam, mux, muy, muz);
-    p.x = p.x + df_make(cam.tf[0], cam.tlo[0]);
-    p.y = p.y + df_make(cam.tf[1], cam.tlo[1]);
-    p.z = p.z + df_make(cam.tf[2], cam.tlo[2]);
-    const D3 tu = cam_rot(cam, r1), tv = cam_rot(cam, r2), nv = cam_rot(cam, r3);
-    const float2 s2 = load_scale(P, n);
-    const float su = s2.x, sv = s2.y;
-    const D3 a = {tu.x * su, tu.y * su, tu.z * su}, b = {tv.x * sv, tv.y * sv, tv.z * sv};
-    const df zmin = p.z - df_sqrt((a.z * a.z + b.z * b.z) * set.rho_max);
-    if (!df_pos(zmin - set.near_plane)) continue;
-    const df iz = df_rcp(p.z);
-    const df xi = p.x * iz, yi = p.y * iz;
-    const df cx = fx * xi + cx0, cy = fy * yi + cy0;
-    const df J11 = fx * (a.x - a.z * xi) * iz, J12 = fx * (b.x - b.z * xi) * iz;
-    const df J21 = fy * (a.y - a.z * yi) * iz, J22 = fy * (b.y - b.z * yi) * iz;
-    const df w1 = a.z * iz, w2 = b.z * iz;
-    // bounding box of {rho_obj <= rho_max} in offsets from c: dual conic of
-    // the centred homography H = [[J, 0], [w^T, 1]]; scaled to C33 = 1 it is
-    // [[e0 e0^T - G, e0], [e0^T, 1]] for the ellipse (d - e0)^T G^-1 (d - e0) <= 1
-    const float rm = set.rho_max;
-    const df C11 = (J11 * J11 + J12 * J12) * rm, C22 = (J21 * J21 + J22 * J22) * rm;
-    const df C12 = (J11 * J21 + J12 * J22) * rm;
-    const df C13 = (J11 * w1 + J12 * w2) * rm, C23 = (J21 * w1 + J22 * w2) * rm;
-    const df C33 = (w1 * w1 + w2 * w2) * rm - 1.f;
-    const df ex = df_sqrt(df_max(C13 * C13 - C11 * C33, df_make(0.f)));
-    const df ey = df_sqrt(df_max(C23 * C23 - C22 * C33, df_make(0.f)));
-    const df i33 = df_rcp(C33);
-    const df x0 = (C13 - ex) * i33, x1 = (C13 + ex) * i33;
-    const df y0 = (C23 - ey) * i33, y1 = (C23 + ey) * i33;
-    const df xmin = cx + df_min(df_min(x0, x1), -rf), xmax = cx + df_max(df_max(x0, x1), rf);
-    const df ymin = cy + df_min(df_min(y0, y1), -rf), ymax = cy + df_max(df_max(y0, y1), rf);
-    float ilo = df_ceil(xmin - 0.5f), ihi = df_floor(xmax - 0.5f);
-    float jlo = df_ceil(ymin - 0.5f), jhi = df_floor(ymax - 0.5f);
-    ilo = fmaxf(ilo, 0.f); jlo = fmaxf(jlo, 0.f);
-    ihi = fminf(ihi, (float)(cam.W - 1)); jhi = fminf(jhi, (float)(cam.H - 1));
-    if (!(ilo <= ihi && jlo <= jhi)) continue;
-    RowGeom gm;
-    {
-      const df e0x = C13 * i33, e0y = C23 * i33;
-      const df g11 = e0x * e0x - C11 * i33, g12 = e0x * e0y - C12 * i33, g22 = e0y * e0y - C22 * i33;
-      gm.cx_hi = cx.hi; gm.cx_lo = cx.lo;
-      gm.cy_hi = cy.hi; gm.cy_lo = cy.lo;
-      gm.e0x = df_float(e0x); gm.e0y = df_float(e0y);
-      if (df_pos(g11) && df_pos(g22)) {
-        // rounded once to FP32; the row rule's margin covers their error
-        const df dg = g11 * g22 - g12 * g12;
-        const float det = df_pos(dg) ? df_float(dg) : 0.f;
-        const float f11 = df_float(g11), f12 = df_float(g12), f22 = df_float(g22);
-        gm.hy = sqrtf(f22);
-        gm.t = f12 * rsqrtf(f11);
-        gm.slope = f12 / f22;
-        gm.wsc = sqrtf(det) / f22;
-      } else {
-        gm.hy = -1.f; gm.t = 0.f; gm.slope = 0.f; gm.wsc = 0.f;  // disk only
+  for (uint32_t cta0 = blockIdx.x * blockDim.x; cta0 < total; cta0 += gridDim.x * blockDim.x) {
+    const uint32_t c0 = cta0 + (threadIdx.x & ~31u);
+    __syncthreads();
+    const uint32_t ci = c0 + lane;
+    const bool live = ci < total;
+    const int n = live ? (int)cand[ci] : 0;
+    if constexpr (kPiece > 0) {
+      const char* const table = kHalf ? reinterpret_cast<const char*>(P.sh_table) : reinterpret_cast<const char*>(P.sh);
+      const uint32_t mine = live ? (kHalf ? P.sh_row[n] : (uint32_t)n) : 0u;
+      const int rows = c0 < total ? (int)min(total - c0, 32u) : 0;
+#pragma unroll 1  // unrolled, the indices of all pieces are held over the geometry
+      for (int p = 0; p < SR::kPieces; ++p) {
+        const int k = p * 32 + lane, row = k / SR::kPieces, col = k - row * SR::kPieces;
+        const uint32_t r = __shfl_sync(kFull, mine, row);
+        if (row < rows)
+          copy_async<kPiece>(stage + row * SR::kStride + col * kPiece, table + (size_t)r * SR::kBytes + col * kPiece);
       }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncwarp();
     }
-    gm.ilo = (int)ilo; gm.ihi = (int)ihi; gm.jlo = (int)jlo; gm.jhi = (int)jhi;
-    const int tx0 = gm.ilo / kTile, tx1 = gm.ihi / kTile + 1;
-    const int ty0 = gm.jlo / kTile, ty1 = gm.jhi / kTile + 1;
-    rect[n] = make_uint2((uint32_t)tx0 | ((uint32_t)ty0 << 16), (uint32_t)tx1 | ((uint32_t)ty1 << 16));
-    uint32_t cnt = 0;
-    for (int ty = ty0; ty < ty1; ++ty) {
-      int a0, a1;
-      if (row_tiles(gm, ty, rff, &a0, &a1)) cnt += (uint32_t)(a1 - a0);
-    }
-    if (cnt == 0) continue;
-    geom[n] = gm;
-    tcount[n] = cnt;
-    const float pz = df_float(p.z);
-    dkey[ci] = __float_as_uint(pz);
-    const df det = J11 * J22 - J12 * J21;
-    // Ji, split for the blends' exact tile-relative evaluation of (u, v):
-    // on a power-of-two grid 2^g chosen so that |Ji d| < 2^(g+22) for every
-    // pixel and tile origin of the surfel's tile rectangle, Jh (multiples of
-    // 2^(g+1)) and nref_h (Ji (o_ref - c) on multiples of 2^g, o_ref the
-    // rectangle's first tile origin) make every partial sum of
-    // nref_h + Jh (o - o_ref) + Jh (lx, ly) exact in FP32; the low parts Jl =
-    // Ji - Jh and nref_l = Ji (o_ref - c) - nref_h (both about 2^g) carry the
-    // rest (see blend.cu).
-    float4 jh, jl, nref;  // nref = (nref_h.u, nref_h.v, nref_l.u, nref_l.v)
-    float ugrid = 1.f;    // 2^-g
-    float2 ef;
-    const float orx = (float)(tx0 * kTile), ory = (float)(ty0 * kTile);
-    if (df_nonzero(det)) {
-      const df id = df_rcp(det);
-      const df i11 = J22 * id, i12 = -(J12 * id), i21 = -(J21 * id), i22 = J11 * id;
-      const float4 r1f = make_float4(df_float(i11), df_float(i12), df_float(i21), df_float(i22));
-      const float4 r5f = make_float4(df_float(i11 - r1f.x), df_float(i12 - r1f.y), df_float(i21 - r1f.z),
-                                     df_float(i22 - r1f.w));
-      ef = make_float2(df_float(-(i11 * w1 + i21 * w2)), df_float(-(i12 * w1 + i22 * w2)));
-      const df d0x = two_sum(orx, -cx.hi) - cx.lo, d0y = two_sum(ory, -cy.hi) - cy.lo;
-      const df nu0 = i11 * d0x + i12 * d0y, nv0 = i21 * d0x + i22 * d0y;
-      const float Dx = fmaxf(fabsf(orx - cx.hi), fabsf((float)(tx1 * kTile) - cx.hi));
-      const float Dy = fmaxf(fabsf(ory - cy.hi), fabsf((float)(ty1 * kTile) - cy.hi));
-      const float Rs = fmaxf(fabsf(r1f.x) + fabsf(r1f.y), fabsf(r1f.z) + fabsf(r1f.w));
-      const float M = __fmul_rn(__fmul_rn(Rs, fmaxf(Dx, Dy) + 2.f), 1.0009765625f);
-      const int E = min(max(((__float_as_int(M) >> 23) & 0xff) - 127, -100), 100);  // M < 2^(E+1)
-      const int g = E - 21;
-      const float ug = __int_as_float((127 - g) << 23), dg = __int_as_float((127 + g) << 23);
-      const float uj = __int_as_float((126 - g) << 23), dj = __int_as_float((128 + g) << 23);
-      jh = make_float4(__fmul_rn(rintf(__fmul_rn(r1f.x, uj)), dj), __fmul_rn(rintf(__fmul_rn(r1f.y, uj)), dj),
-                       __fmul_rn(rintf(__fmul_rn(r1f.z, uj)), dj), __fmul_rn(rintf(__fmul_rn(r1f.w, uj)), dj));
-      jl = make_float4(__fadd_rn(__fsub_rn(r1f.x, jh.x), r5f.x), __fadd_rn(__fsub_rn(r1f.y, jh.y), r5f.y),
-                       __fadd_rn(__fsub_rn(r1f.z, jh.z), r5f.z), __fadd_rn(__fsub_rn(r1f.w, jh.w), r5f.w));
-      const float uh = __fmul_rn(rintf(__fmul_rn(nu0.hi, ug)), dg);
-      const float vh = __fmul_rn(rintf(__fmul_rn(nv0.hi, ug)), dg);
-      nref = make_float4(uh, vh, __fadd_rn(__fsub_rn(nu0.hi, uh), nu0.lo), __fadd_rn(__fsub_rn(nv0.hi, vh), nv0.lo));
-      ugrid = ug;
-    } else {
-      // edge-on disk: no object-space footprint (Ji d and rho_obj are NaN,
-      // the screen filter decides; Ji itself stays finite for the backward)
-      const float qnan = __int_as_float(0x7fffffff);
-      jh = jl = make_float4(0.f, 0.f, 0.f, 0.f);
-      nref = make_float4(qnan, qnan, 0.f, 0.f);
-      ef = make_float2(0.f, 0.f);
-    }
-    // colour: SH at the world direction from the camera centre
-    const float dx = mux - cam.camposf[0], dy = muy - cam.camposf[1], dz = muz - cam.camposf[2];
-    const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
-    constexpr int K = (DEG + 1) * (DEG + 1);
-    float Y[16];
-    sh_basis(dx * il, dy * il, dz * il, DEG, Y);
     float col[3] = {0.f, 0.f, 0.f};
-    if (P.sh_table) {
-      const uint16_t* f = P.sh_table + (size_t)P.sh_row[n] * K * 3;
+    if (live) {
+      // colour: SH at the world direction from the camera centre
+      const float dx = P.mu[3 * n] - cam.camposf[0], dy = P.mu[3 * n + 1] - cam.camposf[1],
+                  dz = P.mu[3 * n + 2] - cam.camposf[2];
+      const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
+      float Y[16];
+      sh_basis(dx * il, dy * il, dz * il, DEG, Y);
+      const unsigned char* const row = stage + lane * SR::kStride;
+      const uint16_t* const fh = kHalf && kPiece == 0 ? P.sh_table + (size_t)P.sh_row[n] * (K * 3) : nullptr;
+      const float* const ff = !kHalf && kPiece == 0 ? P.sh + (size_t)n * (K * 3) : nullptr;
+      float buf[8];  // the piece at hand
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        col[0] = fmaf(h2f(f[k * 3]), Y[k], col[0]);
-        col[1] = fmaf(h2f(f[k * 3 + 1]), Y[k], col[1]);
-        col[2] = fmaf(h2f(f[k * 3 + 2]), Y[k], col[2]);
+      for (int j = 0; j < K * 3; ++j) {
+        float f;
+        if constexpr (kPiece == 16 && !kHalf) {
+          if (j % 4 == 0) *reinterpret_cast<float4*>(buf) = reinterpret_cast<const float4*>(row)[j / 4];
+          f = buf[j % 4];
+        } else if constexpr (kPiece == 16) {
+          if (j % 8 == 0) {
+            const uint4 x = reinterpret_cast<const uint4*>(row)[j / 8];
+            const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+              buf[2 * h] = h2f((uint16_t)(w[h] & 0xFFFFu));
+              buf[2 * h + 1] = h2f((uint16_t)(w[h] >> 16));
+            }
+          }
+          f = buf[j % 8];
+        } else if constexpr (kPiece == 4) {
+          f = reinterpret_cast<const float*>(row)[j];
+        } else {
+          f = kHalf ? h2f(fh[j]) : ff[j];
+        }
+        col[j % 3] = fmaf(f, Y[j / 3], col[j % 3]);
       }
-    } else {
-      const float* f = P.sh + (size_t)n * K * 3;
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        col[0] = fmaf(f[k * 3], Y[k], col[0]);
-        col[1] = fmaf(f[k * 3 + 1], Y[k], col[1]);
-        col[2] = fmaf(f[k * 3 + 2], Y[k], col[2]);
+      for (int c = 0; c < 3; ++c) col[c] = fmaxf(col[c] + 0.5f, 0.f);
+    }
+    __syncthreads();  // and the SH rows are read: the same memory takes the records
+    bool vis = false;
+    if (live) {
+      idx[ci] = (uint32_t)n;
+      uint32_t key = 0xFFFFFFFFu;  // not visible
+      vis = surfel_geometry(P, cam, set, n, rf, rff, rect + n, tcount + n, &key, col,
+                            reinterpret_cast<float4*>(stage + lane * kOutRow));
+      dkey[ci] = key;
+    }
+    const int out_n = vis ? n : -1;
+    __syncwarp();
+    static_assert(sizeof(RowGeom) == 7 * 8 && kRecF4 == 7, "seven pieces of a record and of a footprint");
+#pragma unroll 1
+    for (int p = 0; p < 7; ++p) {
+      const int k = p * 32 + lane, row = k / 7, colp = k - row * 7;
+      const int r = __shfl_sync(kFull, out_n, row);
+      if (r >= 0) {
+        const unsigned char* const src = stage + row * kOutRow;
+        rec[(size_t)r * kRecF4 + colp] = reinterpret_cast<const float4*>(src)[colp];
+        reinterpret_cast<uint2*>(geom + r)[colp] = reinterpret_cast<const uint2*>(src + 16 * kRecF4)[colp];
       }
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) col[c] = fmaxf(col[c] + 0.5f, 0.f);
-    const float sg = df_pos(dot3(nv, p)) ? -1.f : 1.f;
-    float4* Rr = rec + (size_t)n * kRecF4;
-    Rr[0] = make_float4(cx.hi, cy.hi, cx.lo, cy.lo);
-    Rr[1] = jh;
-    Rr[2] = make_float4(ef.x, ef.y, pz, load_opacity(P, n));
-    Rr[3] = make_float4(col[0], col[1], col[2], sg * df_float(nv.x));
-    Rr[4] = make_float4(sg * df_float(nv.y), sg * df_float(nv.z), nref.x, nref.y);
-    Rr[5] = jl;
-    // the first tile of the rectangle (tile indices, packed) and 2^-g, g the grid's exponent
-    Rr[6] = make_float4(nref.z, nref.w, __uint_as_float((uint32_t)tx0 | ((uint32_t)ty0 << 16)), ugrid);
+    __syncwarp();  // before the next candidates' copies
   }
+}
+
+template <int DEG, bool kHalf, int kPiece>
+cudaError_t launch_main(const ParamsDev& P, const CamDev& cam, const SetDev& set, const uint32_t* cand,
+                        const uint32_t* ncand, float4* rec, uint2* rect, uint32_t* tcount, uint32_t* dkey,
+                        uint32_t* idx, RowGeom* geom, unsigned blocks, cudaStream_t st) {
+  constexpr int smem = (kMainThreads / 32) * ShRow<DEG, kHalf, kPiece>::kWarpBytes;
+  static_assert(smem <= 48 * 1024, "within the shared memory of any launch");
+  preprocess_main_kernel<DEG, kHalf, kPiece><<<blocks, kMainThreads, smem, st>>>(P, cam, set, cand, ncand, rec, rect,
+                                                                                 tcount, dkey, idx, geom);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -673,20 +793,38 @@ cudaError_t launch_preprocess(const ParamsDev& P, const CamDev& cam, const SetDe
   if (e != cudaSuccess) return e;
   compact_kernel<<<div_up(P.n, 256), 256, 0, st>>>(flags, dkey, P.n, cand);
   // candidates are a subset of the surfels; a grid-stride loop over the
-  // device-side count, three CTAs per SM (what its registers allow)
+  // device-side count, as many CTAs per SM as its registers allow
   static const unsigned resident = [] {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return 3u * (unsigned)sms;
+    return (unsigned)kMainCtas * (unsigned)sms;
   }();
-  const unsigned blocks = div_up(P.n, 256) < resident ? div_up(P.n, 256) : resident;
-  switch (P.sh_degree) {
-    case 0: preprocess_main_kernel<0><<<blocks, 256, 0, st>>>(P, cam, set, cand, ncand, rec, rect, tcount, dkey, idx, geom); break;
-    case 1: preprocess_main_kernel<1><<<blocks, 256, 0, st>>>(P, cam, set, cand, ncand, rec, rect, tcount, dkey, idx, geom); break;
-    case 2: preprocess_main_kernel<2><<<blocks, 256, 0, st>>>(P, cam, set, cand, ncand, rec, rect, tcount, dkey, idx, geom); break;
-    default: preprocess_main_kernel<3><<<blocks, 256, 0, st>>>(P, cam, set, cand, ncand, rec, rect, tcount, dkey, idx, geom); break;
+  const unsigned blocks = div_up(P.n, kMainThreads) < resident ? div_up(P.n, kMainThreads) : resident;
+#define GS_MAIN(D, HALF, PIECE) \
+  launch_main<D, HALF, PIECE>(P, cam, set, cand, ncand, rec, rect, tcount, dkey, idx, geom, blocks, st)
+  // 16-byte pieces where the rows and their base allow it, else 4-byte words;
+  // binary16 rows that are no whole number of words are read directly, as are
+  // degree-0 rows (three values)
+  if (P.sh_table) {
+    const bool a16 = (uintptr_t)P.sh_table % 16u == 0;
+    switch (P.sh_degree) {
+      case 0: e = GS_MAIN(0, true, 0); break;
+      case 1: e = GS_MAIN(1, true, 0); break;
+      case 2: e = GS_MAIN(2, true, 0); break;
+      default: e = a16 ? GS_MAIN(3, true, 16) : GS_MAIN(3, true, 0); break;
+    }
+  } else {
+    const bool a16 = (uintptr_t)P.sh % 16u == 0;
+    switch (P.sh_degree) {
+      case 0: e = GS_MAIN(0, false, 0); break;
+      case 1: e = a16 ? GS_MAIN(1, false, 16) : GS_MAIN(1, false, 4); break;
+      case 2: e = GS_MAIN(2, false, 4); break;
+      default: e = a16 ? GS_MAIN(3, false, 16) : GS_MAIN(3, false, 4); break;
+    }
   }
+#undef GS_MAIN
+  if (e != cudaSuccess) return e;
   count_launch(2);
   return cudaGetLastError();
 }
