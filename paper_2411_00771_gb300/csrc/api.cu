@@ -732,13 +732,15 @@ gs_status gs_visibility_count(int64_t n, const float* points, float sigma, const
   cudaStream_t st = (cudaStream_t)stream;
   set_pool_threshold();
   Alloc al;
-  const size_t bytes = sizeof(VisCam) * (size_t)n_views;
-  VisCam* dc = static_cast<VisCam*>(al.get(bytes, st));
-  if (!dc) return fail(GS_ERR_OOM, "gs_visibility_count: device allocation failed");
+  const size_t cam_bytes = sizeof(VisCam) * (size_t)n_views, tmp_bytes = visibility_tmp_bytes(n_views);
+  char* const tmp = static_cast<char*>(al.get(tmp_bytes + cam_bytes, st));
+  if (!tmp) return fail(GS_ERR_OOM, "gs_visibility_count: device allocation failed");
+  VisCam* dc = reinterpret_cast<VisCam*>(tmp + tmp_bytes);
   // pageable source: the copy is staged before the call returns
-  cudaError_t e = cudaMemcpyAsync(dc, hc.data(), bytes, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_visibility_count(points, n, sigma, lowpass, near_plane, dc, n_views, counts, st);
-  al.put(dc, bytes, st);
+  cudaError_t e = cudaMemcpyAsync(dc, hc.data(), cam_bytes, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = launch_visibility_count(points, n, sigma, lowpass, near_plane, dc, n_views, tmp, counts, st);
+  al.put(tmp, tmp_bytes + cam_bytes, st);
   if (e != cudaSuccess) return cuda_fail(e, "gs_visibility_count");
   return GS_OK;
 }

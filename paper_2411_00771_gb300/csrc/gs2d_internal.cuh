@@ -351,8 +351,10 @@ struct VisCam {
   float R[9], t[3];
   float fx, fy, cx, cy, W, H;
 };
+// tmp: visibility_tmp_bytes(nviews) of device scratch (16-byte aligned).
+size_t visibility_tmp_bytes(int nviews);
 cudaError_t launch_visibility_count(const float* pts, int64_t n, float sigma, float lowpass, float near_plane,
-                                    const VisCam* cams, int nviews, uint32_t* counts, cudaStream_t st);
+                                    const VisCam* cams, int nviews, void* tmp, uint32_t* counts, cudaStream_t st);
 // keep[j] = counts[j] >= min_count; zrange = (min z, max z) of the kept
 // points (NaN when none); tmp: 2 ints of device scratch.
 cudaError_t launch_visibility_keep(const float* pts, int64_t n, const uint32_t* counts, uint32_t min_count,
