@@ -317,7 +317,7 @@ gs_status build_lists(gs_scene* sc, gs_frame* f, const char* who, cudaStream_t s
   if (!keys || !vals || !keys2 || !vals2 || !ktmp)
     return failed(fail(GS_ERR_OOM, std::string(who) + ": device allocation failed (tile lists)"));
   const float rf = (float)sqrt((double)sc->settings.rho_max / (double)sc->settings.screen_inv_sigma2);
-  GS_CKC(launch_emit(sidx, offs, cnts, f->rect, f->geom, rf, n, cam.tiles_x, keys, vals, st, ncand));
+  GS_CKC(launch_emit(sidx, offs, cnts, f->rect, f->geom, rf, n, cam, keys, vals, st, ncand));
   uint32_t *tk = keys, *tv = vals;
   GS_CKC(radix_sort_pairs(keys, vals, keys2, vals2, K, bits_for(ntiles), ktmp, &tk, &tv, st));
   f->vals = tv;

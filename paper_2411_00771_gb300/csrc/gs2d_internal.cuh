@@ -223,13 +223,16 @@ cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
 
 cudaError_t launch_gather_counts(const uint32_t* order, const uint32_t* tcount, uint32_t* out,
                                  int64_t n, cudaStream_t st, const uint32_t* n_dev = nullptr);
+// Instances of the surfels in `order`: keys (tile index, and in images of up
+// to 65536 tiles the block mask above it) and vals (surfel index).
 cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint32_t* counts,
-                        const uint2* rect, const RowGeom* geom, float rf, int64_t n, int tiles_x,
+                        const uint2* rect, const RowGeom* geom, float rf, int64_t n, const CamDev& cam,
                         uint32_t* keys, uint32_t* vals, cudaStream_t st, const uint32_t* n_dev = nullptr);
 // Per-tile ranges of the sorted instances, and per instance the mask of the
 // tile's sixteen 4 x 4 pixel blocks that the footprint can reach: bit 4 w + g,
 // w = the 8 x 8 block's (column | row << 1), g = the 4 x 4 block's within it
-// (a superset, from the footprint's row rule on bands of four rows).
+// (a superset, from the footprint's row rule on bands of four rows): out of the
+// keys that launch_emit made for the same image.
 cudaError_t launch_ranges(const uint32_t* keys, const uint32_t* vals, int64_t K, int2* ranges, int ntiles,
                           const RowGeom* geom, float rf, const CamDev& cam, uint16_t* masks, cudaStream_t st);
 // Tile ids ordered by list length, longest first (launch order of the blends);

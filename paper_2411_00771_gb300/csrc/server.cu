@@ -308,7 +308,7 @@ int stage_b(gs_server* s, Slot& sl, std::string* msg) {
   int bits = 0;
   while ((int64_t(1) << bits) < ntiles) ++bits;
   cudaError_t e = launch_emit(sl.sidx, (uint32_t*)sl.offs.p, (uint32_t*)sl.cnts.p, (uint2*)sl.rect.p,
-                              (RowGeom*)sl.geom.p, sl.rf, sl.P.n, sl.cam.tiles_x, (uint32_t*)sl.keys.p,
+                              (RowGeom*)sl.geom.p, sl.rf, sl.P.n, sl.cam, (uint32_t*)sl.keys.p,
                               (uint32_t*)sl.vals.p, st, sl.ncand);
   uint32_t *tk = nullptr, *tv = nullptr;
   if (e == cudaSuccess)

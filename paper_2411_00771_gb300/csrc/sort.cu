@@ -328,26 +328,60 @@ __global__ void gather_counts_kernel(const uint32_t* __restrict__ order,
 // Instances of surfel order[r] at offsets offs[r]..: for every tile row of
 // its rectangle, the tile columns its footprint reaches (the same row rule,
 // on the same stored doubles, that counted them in the preprocess), row by
-// row, left to right.  A warp takes 32 consecutive candidates and spreads
-// their tile rows over its lanes (a long footprint's rows go to several
-// lanes instead of keeping one lane busy while the others wait); each row's
-// place within its surfel's run comes from a segmented prefix sum of the
-// rows' tile counts.
+// row, left to right.  A warp takes 32 consecutive candidates, whose instances
+// are one run of the output.  It moves their footprints into shared memory
+// (a lane's own loads of its 56 bytes would touch 32 cache lines each), spreads
+// their tile rows over its lanes, then the rows' tiles, so that neither a long
+// footprint nor a long row keeps one lane busy while the others wait, and
+// consecutive lanes write consecutive instances.
+//
+// kMask: the tile index takes the key's lower 16 bits and the upper 16 hold
+// the mask of the tile's 4 x 4 pixel blocks that the footprint can reach (the
+// row rule on the tile row's four bands of four pixel rows, found once per
+// row of tiles).  The sort carries it along.  Made per sorted instance
+// instead, from a gather of the footprints, the masks alone took 287 us of
+// four 900p views of 4M surfels and 354 us of a 4K view of 8M; emission and
+// ranges together went from 623 to 466 and from 563 to 310 us there (1M
+// surfels at 900p: 65 to 51).  What bounds it is the latency of the footprints'
+// gather and of the steps between a row's tiles and their places (with
+// searches by shuffles instead of marked starts 567 and 369 us); four blocks
+// per SM, three and five measured 685 and 478, 446 and 321.
+__device__ __forceinline__ uint32_t band_nibble(uint32_t blocks, int tx) {
+  // blocks: first and last of the band's 4-pixel block columns (16 bits each)
+  const int lo = max((int)(blocks & 0xffffu) - 4 * tx, 0), hi = min((int)(blocks >> 16) - 4 * tx, 3);
+  return lo <= hi ? (15u >> (3 - hi)) & (15u << lo) : 0u;
+}
+
+struct EmitSmem {
+  uint2 geom[32 * sizeof(RowGeom) / sizeof(uint2)];
+  uint4 cand[32];    // candidates with rows, in order: surfel, first tile row - first flattened row, lane
+  uint4 row[32][2];  // tile rows with tiles, in order: key of flattened tile 0, surfel, tile column of it; bands
+};
+
+template <bool kMask>
 __device__ __forceinline__ void emit_warp(int64_t r, int64_t n, int lane, const uint32_t* __restrict__ order,
                                           const uint32_t* __restrict__ offs, const uint32_t* __restrict__ counts,
                                           const uint2* __restrict__ rect, const RowGeom* __restrict__ geom,
-                                          float rf, int tiles_x, uint32_t* __restrict__ keys,
+                                          float rf, int tiles_x, EmitSmem& sm, uint32_t* __restrict__ keys,
                                           uint32_t* __restrict__ vals) {
   constexpr unsigned kFull = 0xffffffffu;
+  constexpr int kPieces = (int)(sizeof(RowGeom) / sizeof(uint2));
+  const uint32_t lt = (1u << lane) - 1u, upto = lt | (1u << lane);
   const bool valid = r < n && counts[r] > 0u;
-  uint32_t s = 0u, base = 0u;
+  uint32_t s = 0xffffffffu;
   int ty0 = 0, nrows = 0;
   if (valid) {
     s = order[r];
     const uint2 rc = rect[s];
     ty0 = (int)(rc.x >> 16);
     nrows = (int)(rc.y >> 16) - ty0;
-    base = offs[r];
+  }
+  uint32_t out = __shfl_sync(kFull, r < n ? offs[r] : 0u, 0);  // the run's next position
+#pragma unroll
+  for (int p = 0; p < kPieces; ++p) {
+    const int k = p * 32 + lane, row = k / kPieces;
+    const uint32_t sr = __shfl_sync(kFull, s, row);
+    if (sr != 0xffffffffu) sm.geom[k] = reinterpret_cast<const uint2*>(geom + sr)[k - row * kPieces];
   }
   // exclusive prefix of the row counts over the warp: lane i's rows are
   // flattened rows [first, first + nrows)
@@ -359,72 +393,129 @@ __device__ __forceinline__ void emit_warp(int64_t r, int64_t n, int lane, const 
   }
   const int first = incl - nrows;
   const int total = __shfl_sync(kFull, incl, 31);
-  uint32_t done = 0u;  // tiles written so far for lane's own surfel
+  const uint32_t has = __ballot_sync(kFull, nrows > 0);
+  if (nrows > 0) sm.cand[__popc(has & lt)] = make_uint4(s, (uint32_t)(ty0 - first), (uint32_t)lane, 0u);
+  __syncwarp();
+  int before = -1;  // owners of earlier chunks' rows, less one
   for (int c0 = 0; c0 < total; c0 += 32) {
     const int j = c0 + lane;
-    // the row's owner: the last lane whose first row is <= j (lanes with no
-    // rows share the next lane's first row and are passed over)
-    int own = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-      const int cand = own + step;
-      const int fc = __shfl_sync(kFull, first, cand & 31);
-      if (cand < 32 && fc <= j) own = cand;
-    }
-    const bool live = j < total;
-    const uint32_t so = __shfl_sync(kFull, s, own);
-    const int tyo = __shfl_sync(kFull, ty0, own) + (j - __shfl_sync(kFull, first, own));
-    const uint32_t bo = __shfl_sync(kFull, base, own);
-    const uint32_t prev = __shfl_sync(kFull, done, own);
+    // a row's owner: the last candidate whose first row is at or before it
+    const uint32_t heads =
+        __reduce_or_sync(kFull, nrows > 0 && first >= c0 && first < c0 + 32 ? 1u << (first - c0) : 0u);
+    const uint4 cd = sm.cand[before + __popc(heads & upto)];
+    before += __popc(heads);
+    const int ty = (int)cd.y + j;
     int a = 0, b = 0;
-    if (live) {
-      const RowGeom g = geom[so];
-      if (!row_tiles(g, tyo, rf, &a, &b)) a = b = 0;
+    uint32_t band[4] = {0xffffu, 0xffffu, 0xffffu, 0xffffu};  // none
+    if (j < total) {
+      const RowGeom g = reinterpret_cast<const RowGeom*>(sm.geom)[cd.z];
+      if (!row_tiles(g, ty, rf, &a, &b)) a = b = 0;
+      if constexpr (kMask) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int ja = ty * kTile + 4 * q;
+          int ilo, ihi;
+          if (band_pixels(g, ja, ja + 3, rf, &ilo, &ihi)) band[q] = (uint32_t)(ilo >> 2) | ((uint32_t)(ihi >> 2) << 16);
+        }
+      }
     }
-    const int t = b - a;
-    // tiles of the owner's earlier rows in this chunk: segmented exclusive scan
-    int sc = t;
+    // the chunk's tiles: this row has [sx, sx + b - a) of them
+    int sc = b - a;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int x = __shfl_up_sync(kFull, sc, o);
       if (lane >= o) sc += x;
     }
-    const int sx = sc - t;  // exclusive
-    const int seg0 = max(__shfl_sync(kFull, first, own) - c0, 0);  // owner's first lane in this chunk
-    const int within = sx - __shfl_sync(kFull, sx, seg0);
-    uint32_t o = bo + prev + (uint32_t)within;
-    for (int tx = a; tx < b; ++tx, ++o) {
-      keys[o] = (uint32_t)(tyo * tiles_x + tx);
-      vals[o] = so;
+    const int sx = sc - (b - a);
+    const int tiles = __shfl_sync(kFull, sc, 31);
+    const uint32_t some = __ballot_sync(kFull, b > a);
+    if (b > a) {
+      const int q = __popc(some & lt);
+      sm.row[q][0] = make_uint4((uint32_t)(ty * tiles_x + a - sx), cd.x, (uint32_t)(a - sx), 0u);
+      if constexpr (kMask) sm.row[q][1] = make_uint4(band[0], band[1], band[2], band[3]);
     }
-    // each surfel's tiles in this chunk, added to its running count
-    const int l0 = max(first - c0, 0), l1 = min(first + nrows - c0, 32) - 1;
-    const int sum = __shfl_sync(kFull, sc, max(l1, 0)) - __shfl_sync(kFull, sx, min(l0, 31));
-    if (nrows > 0 && l0 <= l1) done += (uint32_t)sum;
+    __syncwarp();
+    int rows = -1;  // rows that start in earlier windows, less one
+    for (int t0 = 0; t0 < tiles; t0 += 32) {
+      const int t = t0 + lane;
+      const uint32_t starts = __reduce_or_sync(kFull, b > a && sx >= t0 && sx < t0 + 32 ? 1u << (sx - t0) : 0u);
+      const int q = rows + __popc(starts & upto);
+      rows += __popc(starts);
+      if (t >= tiles) continue;
+      const uint4 rw = sm.row[q][0];
+      uint32_t key = rw.x + (uint32_t)t;
+      if constexpr (kMask) {
+        const uint4 bd = sm.row[q][1];
+        const int tx = (int)rw.z + t;
+        uint32_t m = 0u;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const uint32_t nib = band_nibble(h == 0 ? bd.x : (h == 1 ? bd.y : (h == 2 ? bd.z : bd.w)), tx);
+          // block columns 0, 1 and 2, 3 of block row h
+          m |= ((nib & 3u) | ((nib & 12u) << 2)) << (8 * (h >> 1) + 2 * (h & 1));
+        }
+        key |= m << 16;
+      }
+      keys[out + (uint32_t)t] = key;
+      vals[out + (uint32_t)t] = rw.y;
+    }
+    out += (uint32_t)tiles;
+    __syncwarp();  // before the next chunk's rows, the next candidates' footprints
   }
 }
 
-__global__ void __launch_bounds__(256) emit_kernel(const uint32_t* __restrict__ order,
+template <bool kMask>
+__global__ void __launch_bounds__(256, 4) emit_kernel(const uint32_t* __restrict__ order,
                                                    const uint32_t* __restrict__ offs,
                                                    const uint32_t* __restrict__ counts,
                                                    const uint2* __restrict__ rect,
                                                    const RowGeom* __restrict__ geom, float rf, int64_t n_max,
                                                    const uint32_t* __restrict__ n_dev, int tiles_x,
                                                    uint32_t* __restrict__ keys, uint32_t* __restrict__ vals) {
+  __shared__ EmitSmem stage[8];
   const int64_t n = item_count(n_max, n_dev);
   const int lane = threadIdx.x & 31;
   // grid-stride over warps of 32 candidates (the grid is sized for the
   // resident CTAs, the count is known on the device only)
   for (int64_t r0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); r0 < n;
        r0 += (int64_t)gridDim.x * blockDim.x)
-    emit_warp(r0 + lane, n, lane, order, offs, counts, rect, geom, rf, tiles_x, keys, vals);
+    emit_warp<kMask>(r0 + lane, n, lane, order, offs, counts, rect, geom, rf, tiles_x, stage[threadIdx.x >> 5], keys,
+                     vals);
 }
 
-// One thread per sorted instance: the ends of its tile's range, and the mask
-// of the tile's 4 x 4 pixel blocks that its footprint can reach (the row rule
-// on the tile's four bands of four rows).  The blends read the mask in list
-// order instead of each gathering the footprint shape and evaluating the rule
-// again.
+// Four sorted instances a thread: the ends of their tiles' ranges, and the
+// masks out of their keys.  Bound by the keys' and masks' traffic.
+__global__ void __launch_bounds__(256) ranges_of_keys(const uint32_t* __restrict__ keys, int64_t K,
+                                                      int2* __restrict__ ranges, uint16_t* __restrict__ masks) {
+  const int64_t i0 = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (i0 >= K) return;
+  uint32_t k[6];  // the four and their neighbours
+  const int m = (int)min((int64_t)4, K - i0);
+  if (m == 4) {
+    const uint4 v = *reinterpret_cast<const uint4*>(keys + i0);
+    k[1] = v.x; k[2] = v.y; k[3] = v.z; k[4] = v.w;
+    *reinterpret_cast<uint2*>(masks + i0) = make_uint2((v.x >> 16) | (v.y & 0xffff0000u), (v.z >> 16) | (v.w & 0xffff0000u));
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      k[q + 1] = q < m ? keys[i0 + q] : 0u;
+      if (q < m) masks[i0 + q] = (uint16_t)(k[q + 1] >> 16);
+    }
+  }
+  k[0] = i0 > 0 ? keys[i0 - 1] : 0u;
+  k[5] = i0 + 4 < K ? keys[i0 + 4] : 0u;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int64_t i = i0 + q;
+    const uint32_t t = k[q + 1] & 0xffffu;
+    if (q >= m) continue;
+    if (i == 0 || (k[q] & 0xffffu) != t) ranges[t].x = (int)i;
+    if (i == K - 1 || (k[q + 2] & 0xffffu) != t) ranges[t].y = (int)(i + 1);
+  }
+}
+
+// Keys without masks: one thread per sorted instance, the mask from the
+// footprint as emit_warp<true> makes it.
 __global__ void __launch_bounds__(256) ranges_kernel(const uint32_t* __restrict__ keys,
                                                      const uint32_t* __restrict__ vals, int64_t K,
                                                      int2* __restrict__ ranges, const RowGeom* __restrict__ geom,
@@ -593,14 +684,18 @@ cudaError_t launch_gather_counts(const uint32_t* order, const uint32_t* tcount, 
   return cudaGetLastError();
 }
 
+// Masks in the keys wherever the tile indices leave them 16 bits: images of up
+// to 16.7 million pixels.
+static bool masks_in_keys(int ntiles) { return ntiles <= 65536; }
+
 cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint32_t* counts,
-                        const uint2* rect, const RowGeom* geom, float rf, int64_t n, int tiles_x,
+                        const uint2* rect, const RowGeom* geom, float rf, int64_t n, const CamDev& cam,
                         uint32_t* keys, uint32_t* vals, cudaStream_t st, const uint32_t* n_dev) {
   if (n <= 0) return cudaSuccess;
   ProfScope ps(kProfSort, st);
   count_launch();
-  // at most eight CTAs per SM (the count of candidates is on the device; the
-  // bound n is usually several times larger)
+  // at most two waves (the count of candidates is on the device; the bound n
+  // is usually several times larger)
   static const unsigned resident = [] {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
@@ -608,7 +703,10 @@ cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint3
     return 8u * (unsigned)sms;
   }();
   const unsigned blocks = div_up(n, 256) < resident ? div_up(n, 256) : resident;
-  emit_kernel<<<blocks, 256, 0, st>>>(order, offs, counts, rect, geom, rf, n, n_dev, tiles_x, keys, vals);
+  if (masks_in_keys(cam.tiles_x * cam.tiles_y))
+    emit_kernel<true><<<blocks, 256, 0, st>>>(order, offs, counts, rect, geom, rf, n, n_dev, cam.tiles_x, keys, vals);
+  else
+    emit_kernel<false><<<blocks, 256, 0, st>>>(order, offs, counts, rect, geom, rf, n, n_dev, cam.tiles_x, keys, vals);
   return cudaGetLastError();
 }
 
@@ -618,7 +716,10 @@ cudaError_t launch_ranges(const uint32_t* keys, const uint32_t* vals, int64_t K,
   cudaError_t e = cudaMemsetAsync(ranges, 0, sizeof(int2) * (size_t)ntiles, st);
   if (e != cudaSuccess || K <= 0) return e;
   count_launch();
-  ranges_kernel<<<div_up(K, 256), 256, 0, st>>>(keys, vals, K, ranges, geom, rf, cam.tiles_x, cam.H, masks);
+  if (masks_in_keys(ntiles))
+    ranges_of_keys<<<div_up((K + 3) / 4, 256), 256, 0, st>>>(keys, K, ranges, masks);
+  else
+    ranges_kernel<<<div_up(K, 256), 256, 0, st>>>(keys, vals, K, ranges, geom, rf, cam.tiles_x, cam.H, masks);
   return cudaGetLastError();
 }
 
