@@ -15,18 +15,24 @@
 //
 // Backward: the same tiles replay each pixel's list back to front from the
 // final transmittance, T_before = T_after / (1 - alpha), with suffix sums
-// for d L / d alpha.  A thread adds the gradients of its two pixels, the
-// group reduces them with a reduce-scatter of shuffles (one reduction per
-// four entries and 16 pixels each), the tile sums them in shared memory, and
-// they reach global memory once per (surfel, tile).
+// for d L / d alpha.  Each warp stages and walks its own window on the list,
+// without barriers of the CTA.  A thread adds the gradients of its two pixels,
+// the group reduces them with a reduce-scatter of shuffles (one reduction per
+// four entries and 16 pixels each) and adds its sums to the surfel's gradient
+// row in global memory, in double: in float the order of the many small
+// additions doubled the gradients' error.
 //
 // Both are bound by instruction issue, so the time is (group, entry) steps
 // times instructions per step.  With one list per warp (8 x 8 pixels) only 10
 // (4M-surfel orbit view) to 18 (1M aerial view) of a step's 32 lanes blended
 // anything; 4 x 4 blocks cost a warp the longest of its four lists instead of
-// their union: forward 501 -> 335 us and backward 1160 -> 980 us on a
-// 1M-surfel 1600 x 900 view, 1148 -> 690 us (forward) on a 4M-surfel 1080p
-// view, and 9.6 -> 7.4 ms for the four backwards of a 4M-surfel training step.
+// their union, and packed FP32 does a thread's two pixels in one instruction.
+// Measured, us (1M-surfel 1600 x 900 view forward and backward, 4M-surfel
+// 1080p view forward, the four backwards of a 4M-surfel training step):
+//   one list per warp, scalar FP32          501  1160  1148  9640
+//   one list per group                      335   980   690  7400
+//   packed FP32                             294   912   583  6550
+//   backward without CTA barriers           296   768   583  5390
 #include <math.h>
 
 #include "gs2d_internal.cuh"
@@ -574,12 +580,15 @@ __global__ void __launch_bounds__(kThreads, 5) blend_fwd_kernel(
 // of lseg entries that separate CTAs process:
 //   1. seg_trans_kernel: per segment and pixel, the product of (1 - alpha)
 //      over the segment's pairs that pass the support and cutoff tests (no
-//      stop);
+//      stop).  Below T_min the product's value decides nothing any more, so a
+//      segment ends once it is there for all pixels.  The same launch
+//      composites the tiles with short lists whole: one after the other, the
+//      two left the GPU half empty;
 //   2. seg_blend_kernel: per segment, the pixel enters with the product of
 //      the segments in front (the transmittance it would have there had
 //      nothing stopped) and composites the segment with the forward's rules,
 //      the stop included.  A pixel that stopped in an earlier segment enters
-//      below T_min and blends nothing;
+//      below T_min and is done;
 //   3. seg_merge_kernel: per tile and pixel, the segments are combined in
 //      order.  Sums add; the distortion adds the cross terms
 //      2 (A_front Zs_seg - Zs_front A_seg) (depths relative to one reference,
@@ -606,13 +615,22 @@ __device__ __forceinline__ bool seg_of(const uint32_t* seg_tile, const uint32_t*
 }
 
 __global__ void __launch_bounds__(kThreads, 5) seg_trans_kernel(
-    CamDev cam, SetDev set, const float4* __restrict__ rec, const uint16_t* __restrict__ masks,
-    const uint32_t* __restrict__ vals, const int2* __restrict__ ranges, int lseg,
-    const uint32_t* __restrict__ seg_tile, const uint32_t* __restrict__ seg_idx, const uint32_t* __restrict__ nseg,
-    float* __restrict__ trans) {
+    CamDev cam, SetDev set, const uint32_t* __restrict__ order, const float4* __restrict__ rec,
+    const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
+    float* __restrict__ out, int32_t* __restrict__ n_contrib, int32_t* __restrict__ last, int32_t* __restrict__ med,
+    unsigned long long* __restrict__ counters, int lseg, const uint32_t* __restrict__ seg_tile,
+    const uint32_t* __restrict__ seg_idx, const uint32_t* __restrict__ nseg, float* __restrict__ trans) {
   __shared__ FwdSmem sh;
+  const int ntiles = cam.tiles_x * cam.tiles_y;
+  if ((int)blockIdx.x < ntiles) {
+    const int t = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
+    blend_fwd_tile<true>(sh, cam, set, rec, masks, vals, ranges, out, n_contrib, last, med, counters, t % cam.tiles_x,
+                         t / cam.tiles_x, lseg);
+    return;
+  }
+  const int seg = (int)blockIdx.x - ntiles;
   int tile, s;
-  if (!seg_of(seg_tile, seg_idx, nseg, blockIdx.x, &tile, &s)) return;
+  if (!seg_of(seg_tile, seg_idx, nseg, seg, &tile, &s)) return;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -620,13 +638,18 @@ __global__ void __launch_bounds__(kThreads, 5) seg_trans_kernel(
   const float2 ly = make_float2((float)lyi + 0.5f, (float)(lyi + kRowStep) + 0.5f);
   const int2 rg = ranges[tile];
   const int e0 = s * lseg, e1 = min(rg.y - rg.x, e0 + lseg);
-  float2 T = bc(1.f);
+  // pixels outside the image enter no product
+  const bool inA = tx0 + lxi < cam.W && ty0 + lyi < cam.H, inB = tx0 + lxi < cam.W && ty0 + lyi + kRowStep < cam.H;
+  float2 T = make_float2(inA ? 1.f : 0.f, inB ? 1.f : 0.f);
   for (int b0 = e0; b0 < e1; b0 += kBatch) {
     const int nb = min(kBatch, e1 - b0);
-    __syncthreads();
+    const bool below = !(T.x >= set.T_min) && !(T.y >= set.T_min);
+    if (__syncthreads_count(below) == kThreads) break;
     stage_batch(sh, rec, masks, vals, rg.x + b0, nb, tx0, ty0);
     __syncthreads();
-    const int glen = group_lists<kBatch>(sh.sm, nb, warp, lane, sh.list[warp]);
+    if (__all_sync(0xffffffffu, below)) continue;
+    int glen = group_lists<kBatch>(sh.sm, nb, warp, lane, sh.list[warp]);
+    if (below) glen = 0;
     const uint8_t* list = sh.list[warp][lane >> 3];
     for (int i = 0; i < glen; ++i) {
       const int k = list[i];
@@ -635,8 +658,8 @@ __global__ void __launch_bounds__(kThreads, 5) seg_trans_kernel(
       T = mul2(T, fma2(neg2(al), bc(1.f), bc(1.f)));
     }
   }
-  trans[(size_t)blockIdx.x * kTilePix + threadIdx.x] = T.x;
-  trans[(size_t)blockIdx.x * kTilePix + kThreads + threadIdx.x] = T.y;
+  trans[(size_t)seg * kTilePix + threadIdx.x] = T.x;
+  trans[(size_t)seg * kTilePix + kThreads + threadIdx.x] = T.y;
 }
 
 __device__ __forceinline__ void seg_store(const FwdPix& p, bool stopped, SegPart* __restrict__ part, int slot) {
@@ -673,6 +696,8 @@ __global__ void __launch_bounds__(kThreads, 5) seg_blend_kernel(
     p.T.x *= trans[(size_t)(first + q) * kTilePix + threadIdx.x];
     p.T.y *= trans[(size_t)(first + q) * kTilePix + kThreads + threadIdx.x];
   }
+  p.doneA = p.doneA || p.T.x < set.T_min;
+  p.doneB = p.doneB || p.T.y < set.T_min;
   p.zr = bc(rec[(size_t)vals[rg.x] * kRecF4 + 2].z);  // the tile's first centre depth
   for (int b0 = e0; b0 < e1; b0 += kBatch) {
     if (__syncthreads_count(p.doneA && p.doneB) == kThreads) break;
@@ -1265,13 +1290,11 @@ cudaError_t launch_blend_fwd_split(const CamDev& cam, const SetDev& set, const u
   cudaError_t e = launch_scan(sb.segcnt, sb.segoff, ntiles, sb.nseg, sb.scan_tmp, st);
   if (e != cudaSuccess) return e;
   seg_list_kernel<<<div_up(ntiles, 256), 256, 0, st>>>(sb.segcnt, sb.segoff, ntiles, sb.seg_tile, sb.seg_idx);
-  // the whole tiles, then the segments (grids sized for the bound, the device
-  // count decides)
-  count_launch(4);
-  blend_fwd_kernel<true><<<(unsigned)ntiles, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out,
-                                                          n_contrib, last, med, counters, sb.lseg);
-  seg_trans_kernel<<<sb.nseg_max, kThreads, 0, st>>>(cam, set, rec, masks, vals, ranges, sb.lseg, sb.seg_tile,
-                                                     sb.seg_idx, sb.nseg, sb.trans);
+  // grids sized for the bound, the device count decides
+  count_launch(3);
+  seg_trans_kernel<<<(unsigned)ntiles + sb.nseg_max, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out,
+                                                                        n_contrib, last, med, counters, sb.lseg,
+                                                                        sb.seg_tile, sb.seg_idx, sb.nseg, sb.trans);
   seg_blend_kernel<<<sb.nseg_max, kThreads, 0, st>>>(cam, set, rec, masks, vals, ranges, sb.lseg, sb.seg_tile,
                                                      sb.seg_idx, sb.nseg, sb.trans,
                                                      static_cast<SegPart*>(sb.part), counters);
