@@ -317,6 +317,140 @@ __global__ void __launch_bounds__(kThreads) radix_downsweep(
   }
 }
 
+// ---- few items ------------------------------------------------------------
+//
+// Up to kSmallMax items one block does a whole scan, or all passes of a sort:
+// each launch costs a small scene more than its work.  A view of 2000 to 4096
+// surfels at 128 x 128 with loss and backward: 345 us with three launches a
+// pass (15 to 18 for its two sorts) and two a scan, 289 so.  With four times
+// as many items a thread, up to 16384 in all, one SM's ranking of them eats the
+// launches: 6000 surfels 352 against 357 us, 10000 396 and 394, 16000 432 and 414.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallIt = 4;
+constexpr int kSmallMax = kSmallIt * kSmallThreads;
+
+// Exclusive scan of one value per thread (1024 threads).
+__device__ __forceinline__ uint32_t small_excl_scan(uint32_t v, uint32_t* total) {
+  __shared__ uint32_t ws[kSmallWarps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t inc = warp_incl_scan(v);
+  if (lane == 31) ws[w] = inc;
+  __syncthreads();
+  if (w == 0) {
+    const uint32_t x = ws[lane], xi = warp_incl_scan(x);
+    ws[lane] = xi - x;
+    if (lane == 31) *total = xi;
+  }
+  __syncthreads();
+  return ws[w] + inc - v;
+}
+
+__global__ void __launch_bounds__(kSmallThreads) scan_small(const uint32_t* in, uint32_t* out, int64_t n_max,
+                                                            const uint32_t* __restrict__ n_dev,
+                                                            uint32_t* __restrict__ total) {
+  constexpr int kIt = kSmallIt;
+  __shared__ uint32_t tot;
+  const int n = (int)item_count(n_max, n_dev);
+  const int t0 = (int)threadIdx.x * kIt;
+  uint32_t x[kIt], s = 0;
+#pragma unroll
+  for (int i = 0; i < kIt; ++i) {
+    x[i] = t0 + i < n ? in[t0 + i] : 0u;
+    s += x[i];
+  }
+  uint32_t pre = small_excl_scan(s, &tot);
+#pragma unroll
+  for (int i = 0; i < kIt; ++i) {
+    if (t0 + i < n) out[t0 + i] = pre;
+    pre += x[i];
+  }
+  if (total && threadIdx.x == 0) *total = tot;
+}
+
+struct SmallSort {
+  uint32_t k[kSmallMax], v[kSmallMax];
+  uint16_t wh[kSmallWarps][kBins];  // per warp and digit: counts, then the warp's start within the digit
+  uint32_t dbase[kBins];
+  uint32_t tot;
+};
+
+// All passes, in place: the items stay in registers between a pass's ranking
+// (as in radix_downsweep) and its exchange through shared memory.
+__global__ void __launch_bounds__(kSmallThreads) radix_small(uint32_t* keys, uint32_t* vals, int64_t n_max,
+                                                             const uint32_t* __restrict__ n_dev, int bits,
+                                                             const uint32_t* __restrict__ gsrc,
+                                                             uint32_t* __restrict__ gout) {
+  extern __shared__ __align__(16) unsigned char small_smem[];
+  constexpr int kIt = kSmallIt;
+  SmallSort& S = *reinterpret_cast<SmallSort*>(small_smem);
+  const int n = (int)item_count(n_max, n_dev);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int i0 = w * (32 * kIt) + lane;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t kk[kIt], vv[kIt];
+#pragma unroll
+  for (int it = 0; it < kIt; ++it) {
+    const int i = i0 + it * 32;
+    kk[it] = i < n ? keys[i] : 0u;
+    vv[it] = i < n ? vals[i] : 0u;
+  }
+  for (int shift = 0; shift < bits; shift += kRadixBits) {
+    const uint32_t mask = (1u << min(bits - shift, kRadixBits)) - 1u;
+    for (int i = threadIdx.x; i < kSmallWarps * kBins / 2; i += kSmallThreads)
+      reinterpret_cast<uint32_t*>(&S.wh[0][0])[i] = 0u;
+    __syncthreads();
+    uint32_t pos[kIt];
+#pragma unroll
+    for (int it = 0; it < kIt; ++it) {
+      const bool valid = i0 + it * 32 < n;
+      const uint32_t d = valid ? (kk[it] >> shift) & mask : 0x100u;
+      const uint32_t peers = digit_peers(d);
+      uint32_t cur = 0u;
+      if (valid) cur = S.wh[w][d];
+      __syncwarp();
+      if (valid && lane == 31 - __clz(peers)) S.wh[w][d] = (uint16_t)(cur + (uint32_t)__popc(peers));
+      __syncwarp();
+      pos[it] = cur + (uint32_t)__popc(peers & lt);
+    }
+    __syncthreads();
+    uint32_t run = 0u;
+    if (threadIdx.x < kBins)
+      for (int ww = 0; ww < kSmallWarps; ++ww) {
+        const uint32_t c = S.wh[ww][threadIdx.x];
+        S.wh[ww][threadIdx.x] = (uint16_t)run;
+        run += c;
+      }
+    const uint32_t base = small_excl_scan(run, &S.tot);
+    if (threadIdx.x < kBins) S.dbase[threadIdx.x] = base;
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kIt; ++it) {
+      if (i0 + it * 32 >= n) continue;
+      const uint32_t d = (kk[it] >> shift) & mask;
+      const uint32_t dst = S.dbase[d] + S.wh[w][d] + pos[it];
+      S.k[dst] = kk[it];
+      S.v[dst] = vv[it];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kIt; ++it) {
+      const int i = i0 + it * 32;
+      if (i >= n) continue;
+      kk[it] = S.k[i];
+      vv[it] = S.v[i];
+    }
+  }
+#pragma unroll
+  for (int it = 0; it < kIt; ++it) {
+    const int i = i0 + it * 32;
+    if (i >= n) continue;
+    keys[i] = kk[it];
+    vals[i] = vv[it];
+    if (gout) gout[i] = gsrc[vv[it]];
+  }
+}
+
 __global__ void gather_counts_kernel(const uint32_t* __restrict__ order,
                                      const uint32_t* __restrict__ tcount, uint32_t* __restrict__ out,
                                      int64_t n_max, const uint32_t* __restrict__ n_dev) {
@@ -604,9 +738,14 @@ cudaError_t launch_scan(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* 
   if (n <= 0) {
     return total_dev ? cudaMemsetAsync(total_dev, 0, sizeof(uint32_t), st) : cudaSuccess;
   }
+  ProfScope ps(kProfSort, st);
+  if (n <= kSmallMax) {
+    count_launch();
+    scan_small<<<1, kSmallThreads, 0, st>>>(in, out, n, n_dev, total_dev);
+    return cudaGetLastError();
+  }
   const unsigned nb = (unsigned)blocks_for(n);
   uint32_t* done = tmp + nb + 1;
-  ProfScope ps(kProfSort, st);
   cudaError_t e = cudaMemsetAsync(done, 0, sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
   count_launch(2);
@@ -639,6 +778,16 @@ void radix_pass(const uint32_t* ki, const uint32_t* vi, uint32_t* ko, uint32_t* 
   radix_offsets<<<nbins, kThreads, 0, st>>>(hist, (int)nb, kThreads * kIt, n, n_dev, dtot);
   radix_downsweep<kIt><<<nb, kThreads, 0, st>>>(ki, vi, ko, vo, n, n_dev, shift, nbins, hist, dtot, gsrc, gout);
 }
+
+cudaError_t sort_small(uint32_t* keys, uint32_t* vals, int64_t n, const uint32_t* n_dev, int bits,
+                       const uint32_t* gsrc, uint32_t* gout, cudaStream_t st) {
+  const int smem = (int)sizeof(SmallSort);
+  const cudaError_t e = cudaFuncSetAttribute(radix_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  count_launch();
+  radix_small<<<1, kSmallThreads, smem, st>>>(keys, vals, n, n_dev, bits, gsrc, gout);
+  return cudaGetLastError();
+}
 }  // namespace
 
 cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
@@ -652,6 +801,7 @@ cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
     return gout ? launch_gather_counts(vals, gsrc, gout, n, st, n_dev) : cudaSuccess;
   }
   ProfScope ps(kProfSort, st);
+  if (n <= kSmallMax) return sort_small(keys, vals, n, n_dev, bits, gsrc, gout, st);
   const unsigned nb = (unsigned)blocks_for(n);
   const int it = items_per_thread(n);
   uint32_t* hist = tmp;
