@@ -87,7 +87,8 @@ class _Loss(torch.autograd.Function):
         adj = grad[:B.ADJ_PLANES]
         sets = [None, None]
         if densify is not None:
-            sets = [torch.zeros_like(adj), torch.zeros_like(adj)]
+            # the loss writes their colour planes and nothing reads the others
+            sets = [torch.empty_like(adj), torch.empty_like(adj)]
         vec = torch.empty(6, device=out.device)
         B.loss(out, target, tinv, weights, adj_total=adj, adj_ssim=sets[0], adj_l1=sets[1], losses=vec[:4])
         vec[4:] = B.geometry_loss(out, cam, w_normal, w_dist, adj)
@@ -198,7 +199,9 @@ class Trainer:
         for cam, tgt, tinv in views:
             H, W = int(cam["height"]), int(cam["width"])
             out, frame = self.scene.render(cam)
-            adj = [torch.zeros((B.ADJ_PLANES, H, W), device=out.device) for _ in range(3)]
+            adj = [torch.zeros((B.ADJ_PLANES, H, W), device=out.device)]
+            # the loss writes the colour planes of these and the backward reads no others
+            adj += [torch.empty_like(adj[0]), torch.empty_like(adj[0])]
             losses, _, _, _ = B.loss(out, tgt, tinv, (0.8, 0.2, wd), adj_total=adj[0], adj_ssim=adj[1],
                                      adj_l1=adj[2])
             geo = B.geometry_loss(out, cam, self.w_normal, self.w_dist, adj[0])
