@@ -1,7 +1,7 @@
 """The update of K-means, exact for every binary16 input: the objective is the
 sum of squared distances (an integer in units of 2^-48), the centroid the
 rounded mean, at the edges of the kernel's steps, at every alignment of the
-codebook and for values whose differences need more than 32 bits."""
+codebook and the SH rows and for values whose differences need more than 32 bits."""
 import ctypes
 
 import numpy as np
@@ -29,7 +29,9 @@ def test_objective_and_centroids_are_exact(m, deg, offset, big):
     if big:
         x[:, 0] = 150.0
         x[0, 0] = -150.0  # 300 apart: more than 2^32 units
-    sh = torch.from_numpy(x.astype(np.float16).astype(np.float32).reshape(m, C // 3, 3)).cuda()
+    buf = torch.empty(m * C + offset, device="cuda")
+    sh = buf[offset:].view(m, C // 3, 3)
+    sh.copy_(torch.from_numpy(x.astype(np.float16).astype(np.float32).reshape(m, C // 3, 3)))
     keep = torch.zeros(m, dtype=torch.uint8, device="cuda")
     u = torch.from_numpy(rng.random(K).astype(np.float32)).cuda()
     xi = _fixed(x.astype(np.float16))
