@@ -224,7 +224,8 @@ cudaError_t radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt,
 cudaError_t launch_gather_counts(const uint32_t* order, const uint32_t* tcount, uint32_t* out,
                                  int64_t n, cudaStream_t st, const uint32_t* n_dev = nullptr);
 // Instances of the surfels in `order`: keys (tile index, and in images of up
-// to 65536 tiles the block mask above it) and vals (surfel index).
+// to 65536 tiles, 16384 in a row, the block mask above it) and vals (surfel
+// index).
 cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint32_t* counts,
                         const uint2* rect, const RowGeom* geom, float rf, int64_t n, const CamDev& cam,
                         uint32_t* keys, uint32_t* vals, cudaStream_t st, const uint32_t* n_dev = nullptr);

@@ -834,9 +834,11 @@ cudaError_t launch_gather_counts(const uint32_t* order, const uint32_t* tcount, 
   return cudaGetLastError();
 }
 
-// Masks in the keys wherever the tile indices leave them 16 bits: images of up
-// to 16.7 million pixels.
-static bool masks_in_keys(int ntiles) { return ntiles <= 65536; }
+// Masks in the keys wherever the tile indices leave them 16 bits (images of up
+// to 16.7 million pixels) and the 4-pixel block columns fit 16 bits.
+static bool masks_in_keys(const CamDev& cam) {
+  return (int64_t)cam.tiles_x * cam.tiles_y <= 65536 && cam.tiles_x <= 16384;
+}
 
 cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint32_t* counts,
                         const uint2* rect, const RowGeom* geom, float rf, int64_t n, const CamDev& cam,
@@ -853,7 +855,7 @@ cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint3
     return 8u * (unsigned)sms;
   }();
   const unsigned blocks = div_up(n, 256) < resident ? div_up(n, 256) : resident;
-  if (masks_in_keys(cam.tiles_x * cam.tiles_y))
+  if (masks_in_keys(cam))
     emit_kernel<true><<<blocks, 256, 0, st>>>(order, offs, counts, rect, geom, rf, n, n_dev, cam.tiles_x, keys, vals);
   else
     emit_kernel<false><<<blocks, 256, 0, st>>>(order, offs, counts, rect, geom, rf, n, n_dev, cam.tiles_x, keys, vals);
@@ -866,7 +868,7 @@ cudaError_t launch_ranges(const uint32_t* keys, const uint32_t* vals, int64_t K,
   cudaError_t e = cudaMemsetAsync(ranges, 0, sizeof(int2) * (size_t)ntiles, st);
   if (e != cudaSuccess || K <= 0) return e;
   count_launch();
-  if (masks_in_keys(ntiles))
+  if (masks_in_keys(cam))
     ranges_of_keys<<<div_up((K + 3) / 4, 256), 256, 0, st>>>(keys, K, ranges, masks);
   else
     ranges_kernel<<<div_up(K, 256), 256, 0, st>>>(keys, vals, K, ranges, geom, rf, cam.tiles_x, cam.H, masks);

@@ -24,3 +24,16 @@ def test_masks_in_keys_and_per_instance_agree(W, H, n, scales):
     assert int((cs[:my, :mx] > 0).sum()) > 0
     assert torch.equal(cs[:my, :mx], cl[:my, :mx])
     assert torch.equal(small[:, :my, :mx], large[:, :my, :mx])
+
+
+@pytest.mark.parametrize("scales", [(-13.0, -11.0), (-11.0, -8.5)], ids=["dots", "wide"])
+def test_rows_of_many_tiles(scales):
+    """16384 tiles in a row take the masks in the keys, 16385 do not."""
+    scene, cam, _, _ = syn.tiny_scene(seed=8, n=20000, width=16384 * 16, height=16, fx=2.0e5, log_scale_range=scales)
+    scene["mu"][:, 1] *= 2e-5
+    _, _, small, cs, _ = gu.gpu_render(scene, cam)
+    _, _, large, cl, _ = gu.gpu_render(scene, dict(cam, width=16385 * 16))
+    mx = 16384 * 16 - 1000
+    assert int((cs[:, 66000:mx] > 0).sum()) > 0
+    assert torch.equal(cs[:, :mx], cl[:, :mx])
+    assert torch.equal(small[:, :, :mx], large[:, :, :mx])
