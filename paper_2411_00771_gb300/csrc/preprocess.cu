@@ -220,8 +220,9 @@ __device__ __forceinline__ bool surfel_geometry(const ParamsDev& P, const CamDev
   df2 ab[3];  // (a, b) = (s_u t_u, s_v t_v)
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    ab[i] = (df2_both(cam_r(cam, i, 0)) * t[0] + df2_both(cam_r(cam, i, 1)) * t[1] + df2_both(cam_r(cam, i, 2)) * t[2]) *
-            s2;
+    const df2 v =
+        df2_both(cam_r(cam, i, 0)) * t[0] + df2_both(cam_r(cam, i, 1)) * t[1] + df2_both(cam_r(cam, i, 2)) * t[2];
+    ab[i] = v * s2;
   }
   const df2 zsq = ab[2] * ab[2];
   const df zmin = pz - df_sqrt((df2_x(zsq) + df2_y(zsq)) * set.rho_max);
@@ -768,13 +769,13 @@ void launch_bwd_deg(const ParamsDev& P, const CamDev& cam, const uint32_t* cand,
   const bool vec = K3 % 4 == 0 && ((uintptr_t)P.sh % 16u) == 0 && ((uintptr_t)G.sh % 16u) == 0;
   if constexpr (K3 % 4 == 0) {
     if (vec) {
-      preprocess_bwd_kernel<DEG, true><<<blocks, 256, 0, st>>>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows, n_sets,
-                                                           screen, G);
+      preprocess_bwd_kernel<DEG, true><<<blocks, 256, 0, st>>>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows,
+                                                               n_sets, screen, G);
       return;
     }
   }
-  preprocess_bwd_kernel<DEG, false><<<blocks, 256, 0, st>>>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows, n_sets,
-                                                           screen, G);
+  preprocess_bwd_kernel<DEG, false><<<blocks, 256, 0, st>>>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows,
+                                                            n_sets, screen, G);
 }
 
 }  // namespace
@@ -832,7 +833,7 @@ cudaError_t launch_preprocess(const ParamsDev& P, const CamDev& cam, const SetDe
 cudaError_t launch_zero_rows(int64_t n, const uint32_t* cand, const uint32_t* ncand, bool loss_layout, double* grow,
                              uint32_t lo, uint32_t rows, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  ProfScope ps(kProfBlendBwd, st);
+  ProfScope ps(kProfPreprocessBwd, st);  // beside the rows' reader: the blend's group is its launches alone
   count_launch();
   const int64_t blocks = (n * (grad_row_stride(loss_layout) / 2) + 255) / 256;
   zero_rows_kernel<<<(unsigned)(blocks < 2432 ? blocks : 2432), 256, 0, st>>>(cand, ncand, grad_row_stride(loss_layout),

@@ -364,8 +364,8 @@ bool launch_batch(gs_server* s, const std::vector<int>& ready, std::string* msg)
       sb.trans = (float*)sl.seg_trans.p;
       sb.part = sl.seg_part.p;
       const cudaError_t es = launch_blend_fwd_split(sl.cam, sl.set, nullptr, (const float4*)sl.rec.p,
-                                                    sl.masks, sl.vals_final, (const int2*)sl.ranges.p, sl.t->req.out, sl.t->req.n_contrib,
-                                                    nullptr, nullptr, s->work, sb, s->blend_st);
+                                                    sl.masks, sl.vals_final, (const int2*)sl.ranges.p, sl.t->req.out,
+                                                    sl.t->req.n_contrib, nullptr, nullptr, s->work, sb, s->blend_st);
       if (es != cudaSuccess) {
         *msg = std::string("blend: ") + cudaGetErrorString(es);
         return false;
