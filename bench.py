@@ -122,8 +122,8 @@ def measured_peak(key):
 # DRAM bytes (read + write) of one blend_bwd launch on this workload, from one
 # ncu capture (dram__bytes_read.sum + dram__bytes_write.sum, one pass, the
 # full-size view); valid only for the kernel sources it was taken on.
-BLEND_BWD_TRAFFIC = {"bytes": 182110720 + 11200000,
-                     "sources_sha256": "9e2ec483cf2f2ccf617b3be5632442872007dd758d5f2653c7ac9ce78650129b"}
+BLEND_BWD_TRAFFIC = {"bytes": 242747904 + 48148992,
+                     "sources_sha256": "f79e75ab42e91d4da9d57bde8b192e2b0f367752923f11da84cb48181b82bc92"}
 
 
 def blend_sources_sha256():
