@@ -654,27 +654,25 @@ gs_status gs_backward(gs_scene* sc, gs_frame* f, const float* const* adj_sets,
   }
   cudaStream_t st = (cudaStream_t)stream;
   const int n = f->n;
-  const bool loss_layout = grad_loss_layout(adj);
-  const size_t row_bytes = sizeof(double) * grad_row_stride(loss_layout);
-  // gradient rows of all surfels, or of as many as there is memory for: the
+  constexpr size_t rec_bytes = sizeof(float) * kGradRec;
+  // gradient records of all surfels, or of as many as there is memory for: the
   // replay then runs once for each part of them
   int rows = n > 0 ? n : 1;
-  double* grow = nullptr;
-  while (!(grow = static_cast<double*>(sc->al.get(row_bytes * (size_t)rows, st))) && rows > 1) rows = (rows + 1) / 2;
-  if (!grow) return fail(GS_ERR_OOM, "gs_backward: scratch allocation failed");
+  float* grec = nullptr;
+  while (!(grec = static_cast<float*>(sc->al.get(rec_bytes * (size_t)rows, st))) && rows > 1) rows = (rows + 1) / 2;
+  if (!grec) return fail(GS_ERR_OOM, "gs_backward: scratch allocation failed");
   cudaError_t e = cudaMemsetAsync(f->counters + 2, 0, 3 * sizeof(unsigned long long), st);
   const SetDev set = to_dev(sc->settings);
   for (int64_t lo = 0; lo < n && e == cudaSuccess; lo += rows) {
     const uint32_t part = (uint32_t)(n - lo < rows ? n - lo : rows);
-    e = launch_zero_rows(n, f->cand, f->ncand, loss_layout, grow, (uint32_t)lo, part, st);
+    e = launch_zero_records(n, f->cand, f->ncand, grec, (uint32_t)lo, part, st);
     if (e == cudaSuccess)
       e = launch_blend_bwd(f->cam, set, f->order, f->rec, f->masks, f->vals, f->ranges, f->out, f->last, f->med, adj,
-                           loss_layout, grow, (uint32_t)lo, part, lo == 0 ? f->counters : nullptr, st);
+                           grec, (uint32_t)lo, part, screen_grads, n, f->K, lo == 0 ? f->counters : nullptr, st);
     if (e == cudaSuccess)
-      e = launch_preprocess_bwd(sc->P, f->cam, f->cand, f->ncand, f->tcount, f->rec, loss_layout, grow, (uint32_t)lo,
-                                part, n_sets, screen_grads, *grads, st);
+      e = launch_preprocess_bwd(sc->P, f->cam, f->cand, f->ncand, f->tcount, grec, (uint32_t)lo, part, *grads, st);
   }
-  sc->al.put(grow, row_bytes * (size_t)rows, st);
+  sc->al.put(grec, rec_bytes * (size_t)rows, st);
   if (e != cudaSuccess) return cuda_fail(e, "gs_backward");
   return GS_OK;
 }

@@ -15,24 +15,32 @@
 //
 // Backward: the same tiles replay each pixel's list back to front from the
 // final transmittance, T_before = T_after / (1 - alpha), with suffix sums
-// for d L / d alpha.  Each warp stages and walks its own window on the list,
-// without barriers of the CTA.  A thread adds the gradients of its two pixels,
-// the group reduces them with a reduce-scatter of shuffles (one reduction per
-// four entries and 16 pixels each) and adds its sums to the surfel's gradient
-// row in global memory, in double: in float the order of the many small
-// additions doubled the gradients' error.
+// for d L / d alpha.  A warp takes 8 x 8 pixels, two per thread, and the
+// entries that reach any of its four 4 x 4 blocks.  A thread adds the
+// gradients of its two pixels, the warp reduces them with a reduce-scatter of
+// shuffles (one reduction per 64 pixels), the tile sums them in shared memory,
+// and they reach global memory once per (surfel, tile).
 //
-// Both are bound by instruction issue, so the time is (group, entry) steps
-// times instructions per step.  With one list per warp (8 x 8 pixels) only 10
-// (4M-surfel orbit view) to 18 (1M aerial view) of a step's 32 lanes blended
-// anything; 4 x 4 blocks cost a warp the longest of its four lists instead of
-// their union, and packed FP32 does a thread's two pixels in one instruction.
-// Measured, us (1M-surfel 1600 x 900 view forward and backward, 4M-surfel
-// 1080p view forward, the four backwards of a 4M-surfel training step):
-//   one list per warp, scalar FP32          501  1160  1148  9640
-//   one list per group                      335   980   690  7400
-//   packed FP32                             294   912   583  6550
-//   backward without CTA barriers           296   768   583  5390
+// The order of those FP32 sums is part of the result.  For a long disk seen
+// nearly edge-on they cancel, and the gradients of its rotation and size follow
+// the rounding of every term and of every partial sum: with other orders of
+// the additions, or sums in double, single values moved by up to 2e-3 of the
+// gradient's root mean square (seen in a third of the training steps of 4M
+// surfels).  So the pairs' terms and the levels of the sum stay as they are,
+// although lane groups of eight that walk their own lists and add their sums
+// to the surfel's row in double took 768 instead of 1050 us (1M-surfel 1600 x
+// 900 view) and 4930 instead of 8420 (the four backwards of the training step).
+//
+// All are bound by instruction issue, so the time is (group, entry) or (warp,
+// entry) steps times instructions per step.  With one list per warp (8 x 8
+// pixels) only 10 (4M-surfel orbit view) to 18 (1M aerial view) of a step's 32
+// lanes blend anything; 4 x 4 blocks cost a forward warp the longest of its
+// four lists instead of their union, and packed FP32 does a thread's two
+// pixels in one instruction.  Forward, us (1M-surfel 1600 x 900 view, 4M-surfel
+// 1080p view):
+//   one list per warp, scalar FP32          501  1148
+//   one list per group                      335   690
+//   packed FP32                             294   583
 #include <math.h>
 
 #include "gs2d_internal.cuh"
@@ -74,7 +82,7 @@ __device__ __forceinline__ float2 sel2(bool a, bool b, float2 x, float2 y) {
 }
 constexpr float kNegHalfLog2e = -0.72134752044448170f;  // -log2(e) / 2
 
-// Pixels of thread t within its tile: warp w covers columns 8 (w & 1) .. +7
+// Pixels of thread t within its tile (not in the backward): warp w covers columns 8 (w & 1) .. +7
 // and rows 8 (w >> 1) .. +7, its lane group g = (l >> 3) the 4 x 4 block at
 // column 4 (g & 1), row 4 (g >> 1) of those, and lane l column l & 3 and rows
 // (l >> 2) & 1 and that + kRowStep of the group's block.
@@ -312,7 +320,8 @@ struct Pair {
   float2 nu, nv;   // Ji d
   float2 rden;     // 1 / (1 + e.d)
   float2 rho;      // min(rho_obj, rho_scr)
-  float2 alpha;    // min(alpha_max, o exp(-rho / 2))
+  float2 G;        // exp(-rho / 2)
+  float2 alpha;    // min(alpha_max, o G)
   bool objA, objB; // object-space branch
   bool hitA, hitB; // rho <= rho_max and alpha >= alpha_min
 };
@@ -320,14 +329,19 @@ struct Pair {
 // The exact grid sums nu0h + Jh (lx, ly) plus the small low-part corrections
 // (see Staged), then the ray-splat distance, the screen filter and alpha.
 // Shared by every blend; explicit round-to-nearest operations so that
-// the forward and the backward take bit-identical decisions.
-__device__ __forceinline__ Pair eval_pair(float lx, float2 ly, float4 s0, float4 jh, float4 jl, float4 n0, float opac,
-                                          const SetDev& set) {
+// the forward and the backward take bit-identical decisions.  The rows are
+// lb + off: lb the row four above where the pixel lies in the lower half of its
+// 8 x 8 block (off 4), else its own (off 0).  The low part reaches a lower row
+// by a step of 4 Jl from the upper one, in every blend.
+__device__ __forceinline__ Pair eval_pair(float lx, float2 lb, float2 off, float4 s0, float4 jh, float4 jl, float4 n0,
+                                          float opac, const SetDev& set) {
   Pair q;
+  const float2 ly = add2(lb, off);
   const float su = __fmaf_rn(jh.x, lx, n0.x), sv = __fmaf_rn(jh.z, lx, n0.y);  // exact, the column's part
-  const float cu = __fmaf_rn(jl.x, lx, n0.z), cv = __fmaf_rn(jl.z, lx, n0.w);
-  q.nu = add2(fma2(bc(jh.y), ly, bc(su)), fma2(bc(jl.y), ly, bc(cu)));
-  q.nv = add2(fma2(bc(jh.w), ly, bc(sv)), fma2(bc(jl.w), ly, bc(cv)));
+  const float2 cu = fma2(bc(jl.y), off, fma2(bc(jl.x), bc(lx), fma2(bc(jl.y), lb, bc(n0.z))));
+  const float2 cv = fma2(bc(jl.w), off, fma2(bc(jl.z), bc(lx), fma2(bc(jl.w), lb, bc(n0.w))));
+  q.nu = add2(fma2(bc(jh.y), ly, bc(su)), cu);
+  q.nv = add2(fma2(bc(jh.w), ly, bc(sv)), cv);
   q.dx = __fadd_rn(lx, s0.x);
   q.dy = add2(ly, bc(s0.y));
   const float2 den = fma2(bc(s0.z), bc(q.dx), fma2(bc(s0.w), q.dy, bc(1.0f)));
@@ -339,7 +353,8 @@ __device__ __forceinline__ Pair eval_pair(float lx, float2 ly, float4 s0, float4
   q.objB = (den.y > 0.f) & (ro.y <= rs.y);
   q.rho = sel2(q.objA, q.objB, ro, rs);
   const float2 x = mul2(bc(kNegHalfLog2e), q.rho);
-  const float2 a = mul2(bc(opac), make_float2(ex2_approx(x.x), ex2_approx(x.y)));
+  q.G = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+  const float2 a = mul2(bc(opac), q.G);
   q.alpha = make_float2(fminf(set.alpha_max, a.x), fminf(set.alpha_max, a.y));
   q.hitA = (q.rho.x <= set.rho_max) & (q.alpha.x >= set.alpha_min);
   q.hitB = (q.rho.y <= set.rho_max) & (q.alpha.y >= set.alpha_min);
@@ -446,14 +461,14 @@ __device__ __forceinline__ bool fwd_step(FwdPair& p, const Pair& q, float4 e2, f
 // front to back, until both of the thread's pixels are done.
 template <bool kFixedRef, bool kPos>
 __device__ __forceinline__ void fwd_walk(FwdPair& p, const FwdSmem& sh, const uint8_t* list, int glen, int b0, float lx,
-                                         float2 ly, const SetDev& set) {
+                                         float2 lb, float2 off, const SetDev& set) {
   if (p.doneA && p.doneB) return;
   int k = list[0];
   for (int i = 0; i < glen; ++i) {
     const float4 e0 = sh.s0[k], e1 = sh.s1[k], e2 = sh.s2[k], e3 = sh.s3[k], e4 = sh.s4[k], e5 = sh.s5[k];
     const int pos = b0 + k;
     k = list[i + 1];  // past the end: a byte of padding, not used
-    const Pair q = eval_pair(lx, ly, e0, e1, e4, e5, e2.y, set);
+    const Pair q = eval_pair(lx, lb, off, e0, e1, e4, e5, e2.y, set);
     bool stopA, stopB;
     if (fwd_step<kFixedRef, kPos>(p, q, e2, e3, pos, set, &stopA, &stopB)) {  // once per pixel
       p.evaluated += (stopA ? i + 1 : 0) + (stopB ? i + 1 : 0);
@@ -520,7 +535,8 @@ __device__ __forceinline__ void blend_fwd_tile(
   const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float lx = (float)lxi + 0.5f;
-  const float2 ly = make_float2((float)lyi + 0.5f, (float)(lyi + kRowStep) + 0.5f);
+  const float2 off = bc((float)(lyi & 4));
+  const float2 lb = make_float2((float)(lyi & ~4) + 0.5f, (float)((lyi & ~4) + kRowStep) + 0.5f);
   const int2 rg = ranges[tile];
   const int len = rg.y - rg.x;
   if (lseg > 0 && len > lseg) return;  // a long list: composited in segments
@@ -532,7 +548,7 @@ __device__ __forceinline__ void blend_fwd_tile(
     stage_batch(sh, rec, masks, vals, rg.x + b0, nb, tx0, ty0);
     __syncthreads();
     const int glen = group_lists<kBatch>(sh.sm, nb, warp, lane, sh.list[warp]);
-    fwd_walk<false, kPos>(p, sh, sh.list[warp][lane >> 3], glen, b0, lx, ly, set);
+    fwd_walk<false, kPos>(p, sh, sh.list[warp][lane >> 3], glen, b0, lx, lb, off, set);
   }
   fwd_store(p.a(), cam, set, px, pyA, out, n_contrib, last, med);
   fwd_store(p.b(), cam, set, px, pyB, out, n_contrib, last, med);
@@ -635,7 +651,8 @@ __global__ void __launch_bounds__(kThreads, 5) seg_trans_kernel(
   const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float lx = (float)lxi + 0.5f;
-  const float2 ly = make_float2((float)lyi + 0.5f, (float)(lyi + kRowStep) + 0.5f);
+  const float2 off = bc((float)(lyi & 4));
+  const float2 lb = make_float2((float)(lyi & ~4) + 0.5f, (float)((lyi & ~4) + kRowStep) + 0.5f);
   const int2 rg = ranges[tile];
   const int e0 = s * lseg, e1 = min(rg.y - rg.x, e0 + lseg);
   // pixels outside the image enter no product
@@ -653,7 +670,7 @@ __global__ void __launch_bounds__(kThreads, 5) seg_trans_kernel(
     const uint8_t* list = sh.list[warp][lane >> 3];
     for (int i = 0; i < glen; ++i) {
       const int k = list[i];
-      const Pair q = eval_pair(lx, ly, sh.s0[k], sh.s1[k], sh.s4[k], sh.s5[k], sh.s2[k].y, set);
+      const Pair q = eval_pair(lx, lb, off, sh.s0[k], sh.s1[k], sh.s4[k], sh.s5[k], sh.s2[k].y, set);
       const float2 al = sel2(q.hitA, q.hitB, q.alpha, bc(0.f));
       T = mul2(T, fma2(neg2(al), bc(1.f), bc(1.f)));
     }
@@ -684,7 +701,8 @@ __global__ void __launch_bounds__(kThreads, 5) seg_blend_kernel(
   const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float lx = (float)lxi + 0.5f;
-  const float2 ly = make_float2((float)lyi + 0.5f, (float)(lyi + kRowStep) + 0.5f);
+  const float2 off = bc((float)(lyi & 4));
+  const float2 lb = make_float2((float)(lyi & ~4) + 0.5f, (float)((lyi & ~4) + kRowStep) + 0.5f);
   const int2 rg = ranges[tile];
   const int e0 = s * lseg, e1 = min(rg.y - rg.x, e0 + lseg);
   const bool inA = px < cam.W && pyA < cam.H, inB = px < cam.W && pyB < cam.H;
@@ -705,7 +723,7 @@ __global__ void __launch_bounds__(kThreads, 5) seg_blend_kernel(
     stage_batch(sh, rec, masks, vals, rg.x + b0, nb, tx0, ty0);
     __syncthreads();
     const int glen = group_lists<kBatch>(sh.sm, nb, warp, lane, sh.list[warp]);
-    fwd_walk<true, true>(p, sh, sh.list[warp][lane >> 3], glen, b0, lx, ly, set);
+    fwd_walk<true, true>(p, sh, sh.list[warp][lane >> 3], glen, b0, lx, lb, off, set);
   }
   SegPart* pp = part + (size_t)blockIdx.x * kTilePix;
   seg_store(p.a(), inA && p.doneA, pp, threadIdx.x);
@@ -821,63 +839,41 @@ __global__ void __launch_bounds__(kThreads, 5) blend_fwd_batched_kernel(BlendBat
 // Backward.
 
 constexpr int kMaxSets = 3;
-// Per-entry gradient vector, the surfel's gradient row (kRow* in
-// gs2d_internal.cuh): d Ji, d e, the screen-space gradient of set 0, the depth
-// term of the centre gradient, d p_z, opacity times d opacity, d rgb, the
-// screen-space gradients of sets 1 and 2, and in the general layout d normal.
-// The loss layout (set 0 on colour and inverse depth only, later sets on
-// colour) has no d normal.  d c is not summed from its own terms: per pair it
-// is set 0's screen gradient plus, on the object-space branch, the term of the
-// depth z = p_z / (1 + e.d) through d, (d rden / d d) p_z dz = -e p_z rden^2 dz;
-// so d c = (screen gradient of set 0) + e * (sum of p_z rden^2 dz), formed once
-// per surfel by the preprocess's backward, and d alpha / d opacity = alpha /
-// opacity, divided there.
-//
-// The reduce-scatter leaves lane r of a group the sums of up to three
-// consecutive values; nat() places the vector so that the groups' first,
-// second and third values are consecutive in the row.
+// Entries staged per batch in the backward, by the CTAs per SM its variant
+// is sized for: 128 for five (a small batch leaves more of the SM's shared
+// memory to L1: 0.939 -> 0.921 ms on the 1M-surfel view, against 224), 224
+// for four (the dense variant's long lists: 128 made the 4M-surfel training
+// step 2.5 % slower).  The gradient accumulators and the six staged vectors
+// per entry fit either way.
+constexpr int batch_b(int min_ctas) { return min_ctas >= 5 ? 128 : 224; }
+// Average tile-list length from which the backward takes the 4-CTA variant:
+// 200 (the 1M-surfel aerial view) ran best with 5 CTAs per SM, 590 (the
+// 4M-surfel orbit view) with 4.
+constexpr int kDenseListLen = 400;
+
+// Per-pair gradient vector.  General layout (any adjoint planes):
+//   [0..5] d Ji, d e; [6] Zc, the depth term of the centre gradient (below);
+//   [7] d p_z, [8] d opacity, [9..11] d rgb, [12..14] d normal;
+//   [15 + 2 s, 16 + 2 s] screen-space gradient of set s.
+// Loss layout (set 0 on colour and inverse depth only, later sets on
+// colour): the normal slots are dropped, [0..11] as above without d normal,
+// [12 + 2 s, 13 + 2 s] screen gradients.
+// The centre gradient is not accumulated on its own: per pair it is set 0's
+// screen gradient plus, on the object-space branch, the term of the depth
+// z = p_z / (1 + e.d) through d, (d rden / d d) p_z dz = -e p_z rden^2 dz;
+// so d c = (screen gradient of set 0) + e * Zc with Zc the sum of
+// p_z rden^2 dz, formed once per entry at the flush.
 template <bool kLoss>
 struct Layout {
-  static constexpr int kN = kLoss ? kRowLoss : kRowAll;
-  // first value of lane r (the halving of kN: 3 2 3 1 3 2 3 1, 3 3 3 2 3 3 3 1)
-  __host__ __device__ static constexpr int start(int r) {
-    return kLoss ? 9 * (r >> 2) + 5 * ((r >> 1) & 1) + 3 * (r & 1) : 11 * (r >> 2) + 6 * ((r >> 1) & 1) + 3 * (r & 1);
-  }
-  // the row's value at lane r's i-th place, -1 when it has none
-  __host__ __device__ static constexpr int at(int r, int i) {
-    if (i == 0) return r;
-    if (kLoss) {
-      if (i == 1) return (r & 3) == 3 ? -1 : 8 + r - (r > 3 ? 1 : 0);
-      return (r & 1) ? -1 : 14 + (r >> 1);
-    }
-    if (i == 1) return r == 7 ? -1 : 8 + r;
-    return (r & 3) == 3 ? -1 : 15 + r - (r > 3 ? 1 : 0);
-  }
-  __host__ __device__ static constexpr int nat(int m) {
-    for (int r = 0; r < 8; ++r)
-      for (int i = 0; i < 3; ++i)
-        if (at(r, i) == m) return start(r) + i;
-    return -1;
-  }
+  static constexpr int kRec = kLoss ? 12 : kGradRec - 1;
+  static constexpr int kN = kRec + 2 * kMaxSets;  // 18 or 21
 };
-constexpr bool layout_is_permutation(bool loss) {
-  const int n = loss ? kRowLoss : kRowAll;
-  uint32_t seen = 0;
-  for (int m = 0; m < n; ++m) {
-    const int v = loss ? Layout<true>::nat(m) : Layout<false>::nat(m);
-    if (v < 0 || v >= n || ((seen >> v) & 1u)) return false;
-    seen |= 1u << v;
-  }
-  return true;
-}
-static_assert(layout_is_permutation(true) && layout_is_permutation(false), "one place per value");
 
-// Balanced reduce-scatter of N values over a lane group of eight: at each
-// halving level the lanes whose bit is clear keep the first ceil(N/2) values
-// and the others the rest, exchanging the halves they do not keep (17
-// shuffles for 18 values, and the warp's four groups reduce four entries at
-// once).  Afterwards v[0..2] hold the group's sums of values start(r) + 0..2.
-constexpr int kGroup = 8;
+// Balanced reduce-scatter of N values over the warp: at each halving level
+// the lanes whose bit is clear keep the first ceil(N/2) values and the others
+// the rest, exchanging the halves they do not keep; N values need about
+// N + 5 shuffles.  Afterwards v[0] holds the warp sum of one slot, given by
+// rs_slot() for the lane (or nothing when rs_slot() returns -1).
 template <int O, int N>
 __device__ __forceinline__ void rs_level(float* v, int lane) {
   constexpr int L = (N + 1) / 2, H = N - L;
@@ -892,32 +888,73 @@ __device__ __forceinline__ void rs_level(float* v, int lane) {
   if constexpr (O > 1) rs_level<O / 2, L>(v, lane);
 }
 
-// State of the reverse replay of a thread's two pixels (the halves of each
-// pair): transmittance, suffix sums S of each adjoint set, the pixels'
-// adjoints, and (general layout) the running opacity A and depth sum Z with
-// their final values for the distortion; gD2 is twice the distortion's adjoint.
-struct BwdPix {
-  float2 T, A, Z, Af, Zf;
-  float2 S[kMaxSets];
-  float2 gC[kMaxSets][3];
-  float2 gA, gZ, gI, gMed, gD2, gN0, gN1, gN2;
-  int lastA, lastB, medA, medB;
-};
+template <int N>
+__device__ __forceinline__ int rs_slot(int lane) {
+  int n = N, real = N, slot = 0;
+  for (int o = 16; o >= 1; o >>= 1) {
+    const int L = (n + 1) / 2;
+    if (lane & o) {
+      slot += L;
+      real = real - L > 0 ? real - L : 0;
+    } else {
+      real = real < L ? real : L;
+    }
+    n = L;
+  }
+  return real > 0 ? slot : -1;
+}
 
-// One half of the state: the pixel at index pix (nothing when outside).
-struct BwdInit {
-  float T, A, Z, S[kMaxSets], gC[kMaxSets][3], gA, gZ, gI, gMed, gD2, gN0, gN1, gN2;
+// Pixels of thread t: lane l takes column l & 7 and rows l >> 3 and
+// (l >> 3) + kBwdRowStep of its warp's 8 x 8 block.
+constexpr int kBwdRowStep = 4;
+__device__ __forceinline__ int bwd_x(int t) { return (((t >> 5) & 1) << 3) | (t & 7); }
+__device__ __forceinline__ int bwd_y(int t) { return ((t >> 6) << 3) | ((t >> 3) & 3); }
+
+// Per warp, the batch's entries that reach any of the warp's four 4 x 4 blocks
+// (bits 4 w .. 4 w + 3 of the block masks), as NW bit words; the loops below
+// visit only their set bits.
+template <int NW>
+__device__ __forceinline__ void warp_entry_bits(const uint16_t* sm, int nb, int warp, int lane, uint32_t* wb) {
+#pragma unroll
+  for (int j = 0; j < NW; ++j) {
+    const int e = 32 * j + lane;
+    const uint32_t w = __ballot_sync(0xffffffffu, e < nb && ((sm[e] >> (4 * warp)) & 15u));
+    if (lane == 0) wb[j] = w;
+  }
+  __syncwarp();
+}
+
+// One pixel's half of a Pair.
+struct PixPair {
+  float dx, dy, nu, nv, rden, rho, G, alpha;
+  bool obj, hit;
+};
+__device__ __forceinline__ PixPair pair_a(const Pair& q) {
+  return {q.dx, q.dy.x, q.nu.x, q.nv.x, q.rden.x, q.rho.x, q.G.x, q.alpha.x, q.objA, q.hitA};
+}
+__device__ __forceinline__ PixPair pair_b(const Pair& q) {
+  return {q.dx, q.dy.y, q.nu.y, q.nv.y, q.rden.y, q.rho.y, q.G.y, q.alpha.y, q.objB, q.hitB};
+}
+
+// Per-pixel state of the reverse replay: transmittance, suffix sums S of
+// each adjoint set, the pixel's adjoints, and (general layout) the running
+// opacity A and depth sum Z with their final values for the distortion.
+struct BwdPix {
+  float T, A, Z, Af, Zf;
+  float S[kMaxSets];
+  float gC[kMaxSets][3];
+  float gA, gZ, gI, gMed, gD, gN0, gN1, gN2;
   int last, med;
 };
 
 template <bool kLoss>
-__device__ __forceinline__ BwdInit bwd_load(bool inside, size_t pix, size_t HW, const float* __restrict__ out,
-                                            const int32_t* __restrict__ last, const int32_t* __restrict__ med,
-                                            const AdjDev& adj, const SetDev& set) {
-  BwdInit p;
+__device__ __forceinline__ void bwd_init(BwdPix& p, bool inside, size_t pix, size_t HW,
+                                         const float* __restrict__ out, const int32_t* __restrict__ last,
+                                         const int32_t* __restrict__ med, const AdjDev& adj,
+                                         const SetDev& set) {
   p.T = 1.f;
-  p.A = p.Z = 0.f;
-  p.gA = p.gZ = p.gI = p.gMed = p.gD2 = p.gN0 = p.gN1 = p.gN2 = 0.f;
+  p.A = p.Z = p.Af = p.Zf = 0.f;
+  p.gA = p.gZ = p.gI = p.gMed = p.gD = p.gN0 = p.gN1 = p.gN2 = 0.f;
   p.last = 0;
   p.med = -1;
 #pragma unroll
@@ -925,7 +962,7 @@ __device__ __forceinline__ BwdInit bwd_load(bool inside, size_t pix, size_t HW, 
     p.gC[s][0] = p.gC[s][1] = p.gC[s][2] = 0.f;
     p.S[s] = 0.f;
   }
-  if (!inside) return p;
+  if (!inside) return;
   p.last = last[pix];
   p.T = out[11 * HW + pix];
 #pragma unroll
@@ -942,243 +979,295 @@ __device__ __forceinline__ BwdInit bwd_load(bool inside, size_t pix, size_t HW, 
   if (m & (1u << 5)) p.gI = a[5 * HW + pix];
   if constexpr (!kLoss) {
     p.med = med[pix];
-    p.A = out[3 * HW + pix];
-    p.Z = out[4 * HW + pix];
+    p.Af = p.A = out[3 * HW + pix];
+    p.Zf = p.Z = out[4 * HW + pix];
     if (m & (1u << 3)) p.gA = a[3 * HW + pix];
     if (m & (1u << 4)) p.gZ = a[4 * HW + pix];
     if (m & (1u << 6)) p.gMed = a[6 * HW + pix];
     if (m & (1u << 7)) p.gN0 = a[7 * HW + pix];
     if (m & (1u << 8)) p.gN1 = a[8 * HW + pix];
     if (m & (1u << 9)) p.gN2 = a[9 * HW + pix];
-    if (m & (1u << 10)) p.gD2 = 2.f * a[10 * HW + pix];
+    if (m & (1u << 10)) p.gD = a[10 * HW + pix];
   }
-  return p;
 }
 
-__device__ __forceinline__ void bwd_init(BwdPix& p, const BwdInit& a, const BwdInit& b) {
-  p.T = make_float2(a.T, b.T);
-  p.A = p.Af = make_float2(a.A, b.A);
-  p.Z = p.Zf = make_float2(a.Z, b.Z);
-#pragma unroll
-  for (int s = 0; s < kMaxSets; ++s) {
-    p.S[s] = make_float2(a.S[s], b.S[s]);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) p.gC[s][c] = make_float2(a.gC[s][c], b.gC[s][c]);
-  }
-  p.gA = make_float2(a.gA, b.gA);
-  p.gZ = make_float2(a.gZ, b.gZ);
-  p.gI = make_float2(a.gI, b.gI);
-  p.gMed = make_float2(a.gMed, b.gMed);
-  p.gD2 = make_float2(a.gD2, b.gD2);
-  p.gN0 = make_float2(a.gN0, b.gN0);
-  p.gN1 = make_float2(a.gN1, b.gN1);
-  p.gN2 = make_float2(a.gN2, b.gN2);
-  p.lastA = a.last;
-  p.lastB = b.last;
-  p.medA = a.med;
-  p.medB = b.med;
+// A pair that was not blended (or lies past the pixel's last blended
+// entry) is masked so that every term of bwd_pair is a finite zero and the
+// pixel's state passes through unchanged: alpha = G = 0 and the
+// screen-space branch, whose terms are finite for any offset.
+__device__ __forceinline__ void mask_pair(PixPair& q, bool live) {
+  const bool h = live && q.hit;
+  q.hit = h;
+  q.alpha = h ? q.alpha : 0.f;
+  q.G = h ? q.G : 0.f;
+  q.obj = h && q.obj;
 }
 
-__device__ __forceinline__ float hsum(float2 x) { return x.x + x.y; }
-__device__ __forceinline__ float dot2(float2 a, float2 b) { return fmaf(a.y, b.y, a.x * b.x); }
-
-// Gradients of the thread's two pairs at list position k, added up into v
-// (gradient-vector layout), and the pixels' replay state moved past the entry.
-// Branch-free.  A pair that was not blended (or lies past the pixel's last
-// blended entry) has hit false: with alpha 0 on the screen-space branch every
-// term is a finite zero and the pixel's state passes through.  The screen
-// branch is the object branch with (nu, nv) = 0 and rden = 1 (then u = v = 0,
-// z = p_z and only the depth's chain through e.d has to be masked) plus the
-// term sinv d of rho_scr.
+// Gradient of one pair at list position k, added into v (gradient-vector
+// layout), and the pixel's replay state moved past it.  Branch-free, so that
+// the two pixels of a thread interleave: both branches of the ray-splat are
+// formed and the one the forward took is selected.
 template <bool kLoss>
-__device__ __forceinline__ void bwd_pair(BwdPix& p, const Pair& q, bool hitA, bool hitB, float4 e0, float4 e1,
-                                         float4 e2, float4 e3, int k, int nsets, const SetDev& set, float* v) {
+__device__ __forceinline__ void bwd_pair(BwdPix& p, const PixPair& q, float4 e0, float4 e1, float4 e2,
+                                         float4 e3, int k, int nsets, const SetDev& set, float* v) {
   using LY = Layout<kLoss>;
-  const float2 one = bc(1.f), zero = bc(0.f);
-  const float2 al = sel2(hitA, hitB, q.alpha, zero);
-  const bool oA = hitA & q.objA, oB = hitB & q.objB;
-  const float2 rd = sel2(oA, oB, q.rden, one);
-  const float2 nu = sel2(oA, oB, q.nu, zero), nv = sel2(oA, oB, q.nv, zero);
-  const float2 rom = rcp2(fma2(neg2(al), one, one));
-  p.T = sel2(hitA, hitB, mul2(p.T, rom), p.T);  // transmittance before this pair
-  const float2 w = mul2(al, p.T);
-  const float2 z = mul2(bc(e2.x), rd);
-  const float2 rz = rcp2(z);
-  float2 dLdw = fma2(p.gC[0][0], bc(e2.z), mul2(p.gC[0][1], bc(e2.w)));
-  dLdw = fma2(p.gI, rz, fma2(p.gC[0][2], bc(e3.x), dLdw));
-  float2 dzv = mul2(mul2(mul2(neg2(w), p.gI), rz), rz);
+  const float rom = rcp_approx(1.f - q.alpha);
+  p.T = q.hit ? p.T * rom : p.T;  // transmittance before this pair
+  const float w = q.alpha * p.T;
+  const float pz = e2.x;
+  const float z = q.obj ? pz * q.rden : pz;
+  const float rz = rcp_approx(z);
+  float dLdw = p.gC[0][0] * e2.z + p.gC[0][1] * e2.w + p.gC[0][2] * e3.x + p.gI * rz;
+  float dzv = -w * p.gI * rz * rz;
   if constexpr (!kLoss) {
-    const float2 Ap = add2(p.A, neg2(w)), Zp = fma2(neg2(w), z, p.Z);  // in front of this pair
-    const float2 Ab = add2(p.Af, neg2(p.A)), Zb = add2(p.Zf, neg2(p.Z));  // behind it
-    const float2 dD = fma2(neg2(z), Ab, add2(fma2(z, Ap, neg2(Zp)), Zb));
-    dLdw = fma2(p.gZ, z, add2(dLdw, p.gA));
-    dLdw = fma2(p.gN2, bc(e3.w), fma2(p.gN1, bc(e3.z), fma2(p.gN0, bc(e3.y), dLdw)));
-    dLdw = fma2(p.gD2, dD, dLdw);
-    dzv = fma2(w, fma2(p.gD2, add2(Ap, neg2(Ab)), p.gZ), dzv);
-    dzv = add2(dzv, sel2(hitA & (k == p.medA), hitB & (k == p.medB), p.gMed, zero));
+    const float Ap = p.A - w, Zp = p.Z - w * z;
+    const float dDdw = 2.f * (z * Ap - Zp + (p.Zf - p.Z) - z * (p.Af - p.A));
+    dLdw += p.gA + p.gZ * z + p.gN0 * e3.y + p.gN1 * e3.z + p.gN2 * e3.w + p.gD * dDdw;
+    dzv += w * p.gZ + p.gD * 2.f * w * (Ap - (p.Af - p.A)) + (k == p.med ? p.gMed : 0.f);
     p.A = Ap;
     p.Z = Zp;
   }
-  // alpha -> rho (zero where alpha is clamped at alpha_max): d alpha / d rho =
-  // -alpha / 2; every derivative of rho below carries a factor 2, so
-  // nd = -2 dL / d rho = dL/dalpha alpha
-  const float2 am = make_float2(al.x < set.alpha_max ? al.x : 0.f, al.y < set.alpha_max ? al.y : 0.f);
-  float2 nd[kMaxSets];
-  nd[0] = mul2(fma2(p.T, dLdw, neg2(mul2(p.S[0], rom))), am);
-  p.S[0] = fma2(w, dLdw, p.S[0]);
+  float dLda[kMaxSets];
+  dLda[0] = p.T * dLdw - p.S[0] * rom;
+  p.S[0] += w * dLdw;
 #pragma unroll
   for (int s = 1; s < kMaxSets; ++s) {
     if (s < nsets) {
-      const float2 dw = fma2(p.gC[s][2], bc(e3.x), fma2(p.gC[s][0], bc(e2.z), mul2(p.gC[s][1], bc(e2.w))));
-      nd[s] = mul2(fma2(p.T, dw, neg2(mul2(p.S[s], rom))), am);
-      p.S[s] = fma2(w, dw, p.S[s]);
+      const float dw = p.gC[s][0] * e2.z + p.gC[s][1] * e2.w + p.gC[s][2] * e3.x;
+      dLda[s] = p.T * dw - p.S[s] * rom;
+      p.S[s] += w * dw;
     } else {
-      nd[s] = zero;
+      dLda[s] = 0.f;
     }
   }
-  // rho = u^2 + v^2 with (u, v) = (nu, nv) rden, z = p_z rden;
-  // rx, ry are half of d rho / d d
-  const float2 u = mul2(nu, rd), vv = mul2(nv, rd);
-  const float2 up = mul2(u, rd), vp = mul2(vv, rd);
-  const float2 c1 = fma2(u, up, mul2(vv, vp));
-  const float2 r2d = mul2(rd, rd), dzp = sel2(oA, oB, mul2(dzv, bc(e2.x)), zero);
-  const float2 zr2 = mul2(dzp, r2d);
-  const float2 dnu = mul2(up, neg2(nd[0])), dnv = mul2(vp, neg2(nd[0]));
-  // d L / d rden, then through rden = 1 / (1 + e.d)
-  const float2 dden = fma2(nd[0], c1, neg2(zr2));
-  const float2 ks = sel2(oA, oB, zero, bc(set.sinv));
-  const float2 rx = fma2(ks, bc(q.dx), fma2(c1, bc(-e0.z), fma2(up, bc(e1.x), mul2(vp, bc(e1.z)))));
-  const float2 ry = fma2(ks, q.dy, fma2(c1, bc(-e0.w), fma2(up, bc(e1.y), mul2(vp, bc(e1.w)))));
-  v[LY::nat(0)] = dot2(dnu, bc(q.dx));
-  v[LY::nat(1)] = dot2(dnu, q.dy);
-  v[LY::nat(2)] = dot2(dnv, bc(q.dx));
-  v[LY::nat(3)] = dot2(dnv, q.dy);
-  v[LY::nat(4)] = dot2(dden, bc(q.dx));
-  v[LY::nat(5)] = dot2(dden, q.dy);
-  v[LY::nat(6)] = dot2(nd[0], rx);
-  v[LY::nat(7)] = dot2(nd[0], ry);
-  v[LY::nat(8)] = hsum(zr2);
-  v[LY::nat(9)] = dot2(dzv, rd);
-  v[LY::nat(10)] = hsum(nd[0]);
-  v[LY::nat(11)] = dot2(w, p.gC[0][0]);
-  v[LY::nat(12)] = dot2(w, p.gC[0][1]);
-  v[LY::nat(13)] = dot2(w, p.gC[0][2]);
-  v[LY::nat(14)] = dot2(nd[1], rx);
-  v[LY::nat(15)] = dot2(nd[1], ry);
-  v[LY::nat(16)] = dot2(nd[2], rx);
-  v[LY::nat(17)] = dot2(nd[2], ry);
+  // alpha -> rho (zero where alpha is clamped at alpha_max).  Every
+  // derivative of rho below carries a factor 2; it is kept in
+  // dadrho2 = 2 d alpha / d rho and drho2 = 2 dL / d rho (exact scalings),
+  // and rx, ry are half of d rho / d d.
+  const bool unclamped = e2.y * q.G < set.alpha_max;
+  const float dadrho2 = unclamped ? -q.alpha : 0.f;
+  const float drho2 = dLda[0] * dadrho2;
+  // object-space branch: rho = u^2 + v^2 with (u, v) = (nu, nv) rden,
+  // z = p_z rden (its terms may be non-finite where it was not taken)
+  const float r2d = q.rden * q.rden;
+  const float tx = q.nu * e1.x + q.nv * e1.z, ty = q.nu * e1.y + q.nv * e1.w;
+  const float c1 = q.rho * q.rden;
+  const float u = q.nu * q.rden, vv = q.nv * q.rden;
+  const float dnu = u * q.rden * drho2, dnv = vv * q.rden * drho2;
+  const float zr2 = dzv * pz * r2d;
+  const float drden = drho2 * (u * q.nu + vv * q.nv) + dzv * pz;
+  const float dden = -drden * r2d;
+  const bool ob = q.obj;
+  const float rx = ob ? r2d * tx - c1 * e0.z : set.sinv * q.dx;
+  const float ry = ob ? r2d * ty - c1 * e0.w : set.sinv * q.dy;
+  const float gpz = ob ? dzv * q.rden : dzv;
+  // the object-space terms of Ji, e and the centre's depth term, zero (and
+  // finite) where the screen branch was taken
+  const float dnu_o = ob ? dnu : 0.f, dnv_o = ob ? dnv : 0.f, dden_o = ob ? dden : 0.f;
+  v[0] = fmaf(dnu_o, q.dx, v[0]);
+  v[1] = fmaf(dnu_o, q.dy, v[1]);
+  v[2] = fmaf(dnv_o, q.dx, v[2]);
+  v[3] = fmaf(dnv_o, q.dy, v[3]);
+  v[4] = fmaf(dden_o, q.dx, v[4]);
+  v[5] = fmaf(dden_o, q.dy, v[5]);
+  v[6] += ob ? zr2 : 0.f;
+  v[7] += gpz;
+  v[8] = fmaf(dLda[0], unclamped ? q.G : 0.f, v[8]);
+  v[9] += w * p.gC[0][0];
+  v[10] += w * p.gC[0][1];
+  v[11] += w * p.gC[0][2];
   if constexpr (!kLoss) {
-    v[LY::nat(18)] = dot2(w, p.gN0);
-    v[LY::nat(19)] = dot2(w, p.gN1);
-    v[LY::nat(20)] = dot2(w, p.gN2);
+    v[12] += w * p.gN0;
+    v[13] += w * p.gN1;
+    v[14] += w * p.gN2;
+  }
+#pragma unroll
+  for (int s = 0; s < kMaxSets; ++s) {
+    const float dr = dLda[s] * dadrho2;
+    v[LY::kRec + 2 * s] -= dr * rx;
+    v[LY::kRec + 2 * s + 1] -= dr * ry;
   }
 }
 
-constexpr float kMinNormal = 1.17549435e-38f;
+// Shared-memory staging of the backward (one batch of kBB entries).
+template <int kAcc, int kBB>
+struct BwdSmem {
+  float4 s0[kBB], s1[kBB], s2[kBB], s3[kBB], s4[kBB], s5[kBB];
+  uint16_t sm[kBB];
+  uint32_t sid[kBB];
+  float acc[kBB][kAcc];
+  uint32_t wbits[kThreads / 32][kBB / 32];
+  int smax;
+};
 
-// The double with the value of a normal, finite v (a conversion instruction
-// runs at one warp per 17 clocks of an SM here, measured; these are five
-// integer operations).
-__device__ __forceinline__ double widen(float v) {
-  const uint32_t b = __float_as_uint(v);
-  const uint32_t hi = ((uint32_t)((int)b >> 3) & 0x8fffffffu) + 0x38000000u;
-  return __hiloint2double((int)hi, (int)(b << 29));
+// Reverse replay of entry kk (list position k) for a thread's two pixels:
+// the pair's gradients, reduced over the warp into the entry's accumulator.
+template <bool kLoss, int kN, int kAcc, int kBB>
+__device__ __forceinline__ void bwd_entry(BwdSmem<kAcc, kBB>& sh, int kk, int k, float lx, float ly, BwdPix& a,
+                                          BwdPix& b, int nsets, const SetDev& set, int lane, int myslot,
+                                          unsigned& wentries, unsigned& wlanes) {
+  const float4 e0 = sh.s0[kk], jh = sh.s1[kk], e2 = sh.s2[kk];
+  const bool liveA = k < a.last, liveB = k < b.last;
+  const float4 jl = sh.s4[kk];
+  const Pair q = eval_pair(lx, bc(ly), make_float2(0.f, (float)kBwdRowStep), e0, jh, jl, sh.s5[kk], e2.y, set);
+  PixPair qa = pair_a(q), qb = pair_b(q);
+  mask_pair(qa, liveA);
+  mask_pair(qb, liveB);
+  const bool contrib = qa.hit || qb.hit;
+  const unsigned ballot = __ballot_sync(0xffffffffu, contrib);
+  if (ballot == 0u) return;
+  ++wentries;
+  wlanes += __popc(ballot);
+  float v[kN];
+#pragma unroll
+  for (int i = 0; i < kN; ++i) v[i] = 0.f;
+  const float4 e3 = sh.s3[kk];
+  // Ji = Jh + Jl (FP32) for the chain rule
+  const float4 e1 = make_float4(jh.x + jl.x, jh.y + jl.y, jh.z + jl.z, jh.w + jl.w);
+  // a pixel row with no hit in the whole warp needs no gradient pass (a
+  // masked pair leaves the pixel's state and the sums unchanged)
+  const bool anyA = __any_sync(0xffffffffu, qa.hit), anyB = __any_sync(0xffffffffu, qb.hit);
+  if (anyA && anyB) {
+    bwd_pair<kLoss>(a, qa, e0, e1, e2, e3, k, nsets, set, v);
+    bwd_pair<kLoss>(b, qb, e0, e1, e2, e3, k, nsets, set, v);
+  } else if (anyA) {
+    bwd_pair<kLoss>(a, qa, e0, e1, e2, e3, k, nsets, set, v);
+  } else {
+    bwd_pair<kLoss>(b, qb, e0, e1, e2, e3, k, nsets, set, v);
+  }
+  if (__popc(ballot) == 1) {
+    if (contrib) {
+#pragma unroll
+      for (int i = 0; i < kN; ++i)
+        if (v[i] != 0.f) atomicAdd(&sh.acc[kk][i], v[i]);
+    }
+  } else {
+    rs_level<16, kN>(v, lane);
+    if (myslot >= 0 && v[0] != 0.f) atomicAdd(&sh.acc[kk][myslot], v[0]);
+  }
 }
 
-// One CTA per tile, one warp per 8 x 8 block.  Each lane group adds its sums
-// of an entry straight to the surfel's gradient row in global memory.  That
-// leaves the warps without a barrier, an accumulator to clear or a
-// compare-and-swap loop (which is what a shared-memory float addition
-// compiles to).  The rows are double: there are three to eight times as many
-// additions to a row as with one per (surfel, tile), and in float they cost
-// accuracy (the scale gradient's error against 64 bits went from 2.3e-5 to
-// 4.8e-5 of its norm on a 300k-surfel view).  5.5 million additions of a whole
-// row, about what a 1M-surfel view has, take 0.21 ms when nothing else runs
-// (0.12 ms in float).
-// Rows [lo, lo + rows) of the surfels are present; the other surfels' sums
+// Records of the surfels [lo, lo + rows) are present; the other surfels' sums
 // are dropped (gs_backward makes several passes when it gets no memory for
-// all rows at once).
-// Four CTAs per SM (up to 128 registers): with five the code spills (720 ->
-// 767 us on the 1M-surfel view, 5.0 -> 5.7 ms for the four backwards of a 4M
-// training step).
-template <bool kLoss>
-__global__ void __launch_bounds__(kThreads, 4) blend_bwd_kernel(
+// all records at once).
+// kMinCtas: the CTAs per SM the register budget is sized for (5: 96
+// registers; 4: up to 128, for dense lists of small footprints).
+template <bool kLoss, int kMinCtas>
+__global__ void __launch_bounds__(kThreads, kMinCtas) blend_bwd_kernel(
     CamDev cam, SetDev set, const uint32_t* __restrict__ order, const float4* __restrict__ rec,
     const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, const int2* __restrict__ ranges,
     const float* __restrict__ out, const int32_t* __restrict__ last, const int32_t* __restrict__ med,
-    AdjDev adj, double* __restrict__ grow, uint32_t lo, uint32_t rows, unsigned long long* __restrict__ counters) {
+    AdjDev adj, float* __restrict__ grec, float* __restrict__ screen, int n, uint32_t lo, uint32_t rows,
+    unsigned long long* __restrict__ counters) {
   using LY = Layout<kLoss>;
   constexpr int kN = LY::kN;
-  __shared__ WarpSmem sh[kThreads / 32];
+  constexpr int kAcc = kN | 1;  // odd row stride: the flush's column reads are conflict-free
+  constexpr int kBatchB = batch_b(kMinCtas), kWordsB = kBatchB / 32;
+  __shared__ BwdSmem<kAcc, kBatchB> sh;
   const int tile = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
-  const int blk = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int lxi = local_x(threadIdx.x), lyi = local_y(threadIdx.x);
-  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
-  const float lx = (float)lxi + 0.5f;
-  const float2 ly = make_float2((float)lyi + 0.5f, (float)(lyi + kRowStep) + 0.5f);
+  const int lxi = bwd_x(threadIdx.x), lyi = bwd_y(threadIdx.x);
+  const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kBwdRowStep;
+  const int warp = threadIdx.x >> 5;
+  const float lx = (float)lxi + 0.5f, lyA = (float)lyi + 0.5f;
   const int2 rg = ranges[tile];
   const size_t HW = (size_t)cam.W * cam.H;
+  const int lane = threadIdx.x & 31;
   const int nsets = adj.n_sets;
+  const int myslot = rs_slot<kN>(lane);
   const bool inA = px < cam.W && pyA < cam.H, inB = px < cam.W && pyB < cam.H;
-  BwdPix p;
-  bwd_init(p, bwd_load<kLoss>(inA, inA ? (size_t)pyA * cam.W + px : 0, HW, out, last, med, adj, set),
-           bwd_load<kLoss>(inB, inB ? (size_t)pyB * cam.W + px : 0, HW, out, last, med, adj, set));
-  // the lane group's own last blended position: entries behind it are dead for
-  // all of its pixels and are not visited
-  int glast = max(p.lastA, p.lastB);
+  BwdPix a, b;
+  bwd_init<kLoss>(a, inA, inA ? (size_t)pyA * cam.W + px : 0, HW, out, last, med, adj, set);
+  bwd_init<kLoss>(b, inB, inB ? (size_t)pyB * cam.W + px : 0, HW, out, last, med, adj, set);
+  if (threadIdx.x == 0) sh.smax = 0;
+  __syncthreads();
+  atomicMax(&sh.smax, max(a.last, b.last));
+  __syncthreads();
+  const int maxlast = sh.smax;
+  // the warp's own last blended position: entries behind it are dead for all
+  // of its pixels and are not visited
+  int wlast = max(a.last, b.last);
 #pragma unroll
-  for (int o = kGroup / 2; o > 0; o >>= 1) glast = max(glast, __shfl_xor_sync(0xffffffffu, glast, o));
-  const int wlast = max(max(__shfl_sync(0xffffffffu, glast, 0), __shfl_sync(0xffffffffu, glast, 8)),
-                        max(__shfl_sync(0xffffffffu, glast, 16), __shfl_sync(0xffffffffu, glast, 24)));
-  // where the lane's sums go within a row
-  const int r = lane & (kGroup - 1);
-  double* const dst = grow + r;
-  int off1 = -1, off2 = -1;
-#pragma unroll
-  for (int x = 0; x < kGroup; ++x) {
-    if (x == r) {
-      off1 = LY::at(x, 1) - x;
-      off2 = LY::at(x, 2) - x;
-    }
-  }
-  const bool has1 = off1 + r >= 0, has2 = off2 + r >= 0;
+  for (int o = 16; o > 0; o >>= 1) wlast = max(wlast, __shfl_xor_sync(0xffffffffu, wlast, o));
   unsigned replayed = 0, wentries = 0, wlanes = 0;
-  WarpSmem& sm = sh[blk];
-  walk_list<true>(sm, rec, masks + rg.x, vals + rg.x, 0, wlast, glast, tx0, ty0, blk, 0,
-                  [&](int k, int&) {
-    const float4 e0 = at16(sm.s0, k), jh = at16(sm.s1, k), e2 = at16(sm.s2, k), jl = at16(sm.s4, k);
-    const uint2 meta = at16(sm.meta, k);
-    const Pair q = eval_pair(lx, ly, e0, jh, jl, at16(sm.s5, k), e2.y, set);
-    const int pos = (int)meta.x;
-    const bool liveA = pos < p.lastA, liveB = pos < p.lastB;
-    const bool hitA = liveA & q.hitA, hitB = liveB & q.hitB;
-    replayed += (liveA ? 1u : 0u) + (liveB ? 1u : 0u);  // performance counter, as wentries and wlanes
-    const unsigned ballot = __ballot_sync(0xffffffffu, hitA | hitB);
-    if (ballot == 0u) return;
-    ++wentries;
-    wlanes += __popc(ballot);
-    float v[kN];
-    // Ji = Jh + Jl (FP32) for the chain rule
-    const float4 e1 = make_float4(jh.x + jl.x, jh.y + jl.y, jh.z + jl.z, jh.w + jl.w);
-    bwd_pair<kLoss>(p, q, hitA, hitB, e0, e1, e2, at16(sm.s3, k), pos, nsets, set, v);
-    rs_level<kGroup / 2, kN>(v, lane);
-    const uint32_t row = meta.y - lo;
-    if (((ballot >> (lane & 24)) & 0xffu) && row < rows) {
-      double* const d = dst + (size_t)row * grad_row_stride(kLoss);
-      const float a0 = fabsf(v[0]), a1 = has1 ? fabsf(v[1]) : 0.f, a2 = has2 ? fabsf(v[2]) : 0.f;
-      if (a0 + a1 + a2 < INFINITY) {
-        // zeros (and what is below the normal range) add nothing
-        if (a0 >= kMinNormal) atomicAdd(d, widen(v[0]));
-        if (a1 >= kMinNormal) atomicAdd(d + off1, widen(v[1]));
-        if (a2 >= kMinNormal) atomicAdd(d + off2, widen(v[2]));
-      } else {  // infinities and NaN go through as they are
-        atomicAdd(d, (double)v[0]);
-        if (has1) atomicAdd(d + off1, (double)v[1]);
-        if (has2) atomicAdd(d + off2, (double)v[2]);
+
+  for (int bend = maxlast; bend > 0; bend -= kBatchB) {
+    const int b0 = bend > kBatchB ? bend - kBatchB : 0;
+    const int nb = bend - b0;
+    __syncthreads();
+    for (int t = threadIdx.x; t < nb; t += kThreads) {
+      const uint32_t s = vals[rg.x + b0 + t];
+      sh.sid[t] = s;
+      const Staged e = stage_entry(rec, s, tx0, ty0);
+      sh.s0[t] = e.s0;
+      sh.s1[t] = e.s1;
+      sh.s2[t] = e.s2;
+      sh.s3[t] = e.s3;
+      sh.s4[t] = e.s4;
+      sh.s5[t] = e.s5;
+      sh.sm[t] = masks[rg.x + b0 + t];
+    }
+    for (int i = threadIdx.x; i < nb * kAcc; i += kThreads) (&sh.acc[0][0])[i] = 0.f;
+    __syncthreads();
+    warp_entry_bits<kWordsB>(sh.sm, nb, warp, lane, sh.wbits[warp]);
+    if (lane == 0) {
+#pragma unroll
+      for (int j = 0; j < kWordsB; ++j) {
+        const int lw = wlast - b0 - 32 * j;
+        sh.wbits[warp][j] &= lw >= 32 ? 0xffffffffu : (lw > 0 ? (1u << lw) - 1u : 0u);
       }
     }
-  });
+    __syncwarp();
+    if (counters) {
+      // the batch's entries before each pixel's last blended one that the
+      // warp visits (performance counter)
+#pragma unroll
+      for (int j = 0; j < kWordsB; ++j) {
+        const uint32_t bits = sh.wbits[warp][j];
+        const int la = a.last - b0 - 32 * j, lb = b.last - b0 - 32 * j;
+        replayed += (unsigned)__popc(la >= 32 ? bits : (la > 0 ? bits & ((1u << la) - 1u) : 0u));
+        replayed += (unsigned)__popc(lb >= 32 ? bits : (lb > 0 ? bits & ((1u << lb) - 1u) : 0u));
+      }
+    }
+    for (int j = kWordsB - 1; j >= 0; --j) {
+      uint32_t bits = sh.wbits[warp][j];
+      while (bits != 0u) {  // back to front: highest set bit first
+        const int hb = 31 - __clz(bits);
+        bits &= ~(1u << hb);
+        bwd_entry<kLoss, kN, kAcc, kBatchB>(sh, 32 * j + hb, b0 + 32 * j + hb, lx, lyA, a, b, nsets, set, lane, myslot,
+                                   wentries, wlanes);
+      }
+    }
+    __syncthreads();
+    // flush this batch: one (surfel, tile) gradient record per entry, the
+    // centre gradient formed from set 0's screen gradient and Zc
+    for (int t = threadIdx.x; t < nb; t += kThreads) {
+      const uint32_t s = sh.sid[t];
+      if (s - lo >= rows) continue;
+      float* g = grec + (size_t)(s - lo) * kGradRec;
+      const float* x = sh.acc[t];
+      const float4 e0 = sh.s0[t];
+      float r[kGradRec];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) r[i] = x[i];
+      r[6] = fmaf(e0.z, x[6], x[LY::kRec]);
+      r[7] = fmaf(e0.w, x[6], x[LY::kRec + 1]);
+#pragma unroll
+      for (int i = 7; i < LY::kRec; ++i) r[i + 1] = x[i];
+#pragma unroll
+      for (int i = 0; i < LY::kRec + 1; ++i)
+        if (r[i] != 0.f) atomicAdd(&g[i], r[i]);
+      if (screen) {
+        for (int st = 0; st < nsets; ++st) {
+          const float x0 = sh.acc[t][LY::kRec + 2 * st];
+          const float x1 = sh.acc[t][LY::kRec + 2 * st + 1];
+          float* sg = screen + ((size_t)st * n + s) * 2;
+          if (x0 != 0.f) atomicAdd(&sg[0], x0);
+          if (x1 != 0.f) atomicAdd(&sg[1], x1);
+        }
+      }
+    }
+  }
   if (counters) {
     unsigned e = replayed;
 #pragma unroll
@@ -1229,7 +1318,8 @@ __global__ void __launch_bounds__(kThreads, 5) blend_contrib_kernel(
   const int px = tx0 + lxi, pyA = ty0 + lyi, pyB = pyA + kRowStep;
   const int blk = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float lx = (float)lxi + 0.5f;
-  const float2 ly = make_float2((float)lyi + 0.5f, (float)(lyi + kRowStep) + 0.5f);
+  const float2 off = bc((float)(lyi & 4));
+  const float2 lb = make_float2((float)(lyi & ~4) + 0.5f, (float)((lyi & ~4) + kRowStep) + 0.5f);
   const bool inA = px < cam.W && pyA < cam.H, inB = px < cam.W && pyB < cam.H;
   const int2 rg = ranges[tile];
   float TA = 1.f, TB = 1.f;
@@ -1237,7 +1327,7 @@ __global__ void __launch_bounds__(kThreads, 5) blend_contrib_kernel(
   WarpSmem& sm = sh[blk];
   walk_list<false>(sm, rec, masks + rg.x, vals + rg.x, 0, rg.y - rg.x, 0, tx0, ty0, blk, 0,
                    [&](int k, int&) {
-    const Pair q = eval_pair(lx, ly, at16(sm.s0, k), at16(sm.s1, k), at16(sm.s4, k), at16(sm.s5, k), at16(sm.s2, k).y,
+    const Pair q = eval_pair(lx, lb, off, at16(sm.s0, k), at16(sm.s1, k), at16(sm.s4, k), at16(sm.s5, k), at16(sm.s2, k).y,
                              set);
     const unsigned ba = __ballot_sync(0xffffffffu, inA & (q.rho.x <= set.rho_max));
     const unsigned bb = __ballot_sync(0xffffffffu, inB & (q.rho.y <= set.rho_max));
@@ -1248,7 +1338,7 @@ __global__ void __launch_bounds__(kThreads, 5) blend_contrib_kernel(
               contrib_step(TB, stB, q.hitB, q.alpha.y, set, gamma);
     if (__any_sync(0xffffffffu, c != 0.f)) {
 #pragma unroll
-      for (int o = kGroup / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     }
     if (cnt != 0u && (lane & 7) == 0) {
       const uint32_t sid = at16(sm.meta, k).y;
@@ -1313,17 +1403,26 @@ cudaError_t launch_blend_fwd_batched(const BlendBatch& batch, int grid, cudaStre
 
 cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
                              const uint16_t* masks, const uint32_t* vals, const int2* ranges, const float* out,
-                             const int32_t* last, const int32_t* med, const AdjDev& adj,
-                             bool loss_layout, double* grow, uint32_t lo, uint32_t rows,
-                             unsigned long long* counters, cudaStream_t st) {
+                             const int32_t* last, const int32_t* med, const AdjDev& adj, float* grec, uint32_t lo,
+                             uint32_t rows, float* screen, int n, int64_t K, unsigned long long* counters, cudaStream_t st) {
   const unsigned grid = (unsigned)cam.tiles_x * (unsigned)cam.tiles_y;
+  // the training loss drives set 0 through colour and inverse depth only and
+  // the other sets through colour: a leaner kernel for that layout
+  bool loss_layout = (adj.mask[0] & ~(GS_MASK_RGB | (1u << GS_PLANE_INVDEPTH))) == 0u;
+  for (int s = 1; s < adj.n_sets; ++s) loss_layout = loss_layout && (adj.mask[s] & ~GS_MASK_RGB) == 0u;
   ProfScope ps(kProfBlendBwd, st);
-  if (loss_layout)
-    blend_bwd_kernel<true><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, last, med, adj,
-                                                      grow, lo, rows, counters);
-  else
-    blend_bwd_kernel<false><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, last, med, adj,
-                                                       grow, lo, rows, counters);
+  const bool dense = K >= (int64_t)kDenseListLen * (int64_t)grid;
+#define GS_BWD(L, M)                                                                                           \
+  blend_bwd_kernel<L, M><<<grid, kThreads, 0, st>>>(cam, set, order, rec, masks, vals, ranges, out, last, med, \
+                                                    adj, grec, screen, n, lo, rows, counters)
+  if (loss_layout) {
+    if (dense) GS_BWD(true, 4);
+    else GS_BWD(true, 5);
+  } else {
+    if (dense) GS_BWD(false, 4);
+    else GS_BWD(false, 5);
+  }
+#undef GS_BWD
   count_launch();
   return cudaGetLastError();
 }

@@ -311,28 +311,15 @@ struct AdjDev {
   int n_sets;
 };
 
-// Per-surfel gradient row of the blend backward, in double (see
-// blend_bwd_kernel): [0..3] d Ji, [4..5] d e, [6..7] screen-space gradient of
-// set 0, [8] depth term of the centre gradient, [9] d p_z, [10] opacity times
-// d opacity, [11..13] d rgb, [14..15] and [16..17] screen-space gradients of
-// sets 1 and 2, [18..20] d normal.  The loss layout ends before the normal.
-constexpr int kRowLoss = 18, kRowAll = 21;
-// distance between rows, whole 32-byte sectors
-__host__ __device__ constexpr int grad_row_stride(bool loss_layout) { return loss_layout ? 20 : 24; }
-// The training loss drives set 0 through colour and inverse depth only and
-// the other sets through colour.
-inline bool grad_loss_layout(const AdjDev& adj) {
-  bool l = (adj.mask[0] & ~(GS_MASK_RGB | (1u << GS_PLANE_INVDEPTH))) == 0u;
-  for (int s = 1; s < adj.n_sets; ++s) l = l && (adj.mask[s] & ~GS_MASK_RGB) == 0u;
-  return l;
-}
+// Per-surfel intermediate gradient record of the blend backward.
+constexpr int kGradRec = 16;  // Ji(4) e(2) c(2) p_z(1) opacity(1) rgb(3) n(3)
 
-// Gradient rows of surfels [lo, lo + rows), added to (grow[0] is surfel lo's).
+// Gradient records of surfels [lo, lo + rows), added to (grec[0] is surfel
+// lo's), and their screen gradients added to screen ([n_sets][n][2]; may be null).
 cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_t* order, const float4* rec,
                              const uint16_t* masks, const uint32_t* vals, const int2* ranges, const float* out,
-                             const int32_t* last, const int32_t* med, const AdjDev& adj,
-                             bool loss_layout, double* grow, uint32_t lo, uint32_t rows,
-                             unsigned long long* counters, cudaStream_t st);
+                             const int32_t* last, const int32_t* med, const AdjDev& adj, float* grec, uint32_t lo,
+                             uint32_t rows, float* screen, int n, int64_t K, unsigned long long* counters, cudaStream_t st);
 
 // Trim contribution (Sec. 3.3, Eq. 3) of one view over the frame's tile
 // lists: per surfel the support count and the sum of alpha^gamma T^(1-gamma)
@@ -394,15 +381,13 @@ size_t select_tmp_words();
 cudaError_t launch_prune(int64_t n, const float* contrib, int64_t k, uint8_t* keep, float* bound,
                          uint32_t* tmp, cudaStream_t st);
 
-// Zeroes the candidates' gradient rows.
-cudaError_t launch_zero_rows(int64_t n, const uint32_t* cand, const uint32_t* ncand, bool loss_layout, double* grow,
-                             uint32_t lo, uint32_t rows, cudaStream_t st);
-// The candidates' parameter gradients from their rows, and the rows' screen
-// gradients added to screen ([n_sets][n][2]; may be null).
+// Zeroes the candidates' gradient records.
+cudaError_t launch_zero_records(int64_t n, const uint32_t* cand, const uint32_t* ncand, float* grec, uint32_t lo,
+                                uint32_t rows, cudaStream_t st);
+// The candidates' parameter gradients from their records.
 cudaError_t launch_preprocess_bwd(const ParamsDev& P, const CamDev& cam, const uint32_t* cand,
-                                  const uint32_t* ncand, const uint32_t* tcount, const float4* rec,
-                                  bool loss_layout, const double* grow, uint32_t lo, uint32_t rows, int n_sets,
-                                  float* screen, const gs_param_grads& G, cudaStream_t st);
+                                  const uint32_t* ncand, const uint32_t* tcount, const float* grec, uint32_t lo,
+                                  uint32_t rows, const gs_param_grads& G, cudaStream_t st);
 
 cudaError_t launch_loss(int W, int H, const float* out, const float* tgt, const float* tinv,
                         const gs_loss_weights& w, float* adj_total, float* adj_ssim,

@@ -512,17 +512,6 @@ cudaError_t launch_main(const ParamsDev& P, const CamDev& cam, const SetDev& set
 // ---------------------------------------------------------------------------
 // Backward.
 
-// The float nearest to d: integer operations for a normal result (a conversion
-// instruction runs at one warp per 17 clocks of an SM here, measured).
-__device__ __forceinline__ float narrow(double d) {
-  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
-  const uint32_t e = (hi >> 20) & 0x7ffu;
-  if (e < 897u || e > 1149u) return (hi & 0x7fffffffu) | lo ? __double2float_rn(d) : 0.f;
-  const uint32_t b = (hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-  const uint32_t rest = lo << 3;  // below the last bit kept; ties to even
-  return __uint_as_float(b + (rest > 0x80000000u || (rest == 0x80000000u && (b & 1u)) ? 1u : 0u));
-}
-
 // Gradient of one visible surfel n: chain the per-surfel record (d Ji, d e,
 // d c, d p_z, d opacity, d rgb, d normal) back to mu, q, s, o and SH,
 // accumulated into G.  kVec: SH rows and gradient rows are float4-aligned.
@@ -534,21 +523,14 @@ __device__ __forceinline__ float narrow(double d) {
 // another or the parameters.
 template <int DEG, bool kVec>
 __device__ __forceinline__ void bwd_one(const ParamsDev& P, const CamDev& cam, int n, uint32_t tc,
-                                        const float4* __restrict__ rec, const double* __restrict__ row, bool normals,
-                                        int n_sets, float* __restrict__ screen, const gs_param_grads& G) {
+                                        const float* __restrict__ row, const gs_param_grads& G) {
+  static_assert(kGradRec == 16, "gradient record of four float4");
   float* __restrict__ Gq = G.quat;
   float* __restrict__ Gm = G.mu;
   float* __restrict__ Gs = G.scale;
   float* __restrict__ Go = G.opacity;
-  double2 x[kRowAll / 2 + 1];
-#pragma unroll
-  for (int i = 0; i < kRowLoss / 2; ++i) x[i] = reinterpret_cast<const double2*>(row)[i];
-  x[9] = x[10] = make_double2(0.0, 0.0);
-  if (normals) {
-    x[9] = reinterpret_cast<const double2*>(row)[9];
-    x[10] = reinterpret_cast<const double2*>(row)[10];
-  }
-  const float4 rr = rec[(size_t)n * kRecF4 + 2];  // (e.x, e.y, p_z, opacity) of the render
+  const float4* g4 = reinterpret_cast<const float4*>(row);
+  const float4 ga4 = g4[0], gb4 = g4[1], gc4 = g4[2], gd4 = g4[3];
   float oq[4] = {0.f, 0.f, 0.f, 0.f}, om[3] = {0.f, 0.f, 0.f}, os[2] = {0.f, 0.f}, oo = 0.f;
   if (Gq) {
 #pragma unroll
@@ -563,16 +545,10 @@ __device__ __forceinline__ void bwd_one(const ParamsDev& P, const CamDev& cam, i
     os[1] = Gs[2 * n + 1];
   }
   if (Go) oo = Go[n];
-  float sg[3][2] = {{narrow(x[3].x), narrow(x[3].y)}, {narrow(x[7].x), narrow(x[7].y)},
-                    {narrow(x[8].x), narrow(x[8].y)}};
-  float gJi11 = narrow(x[0].x), gJi12 = narrow(x[0].y), gJi21 = narrow(x[1].x), gJi22 = narrow(x[1].y);
-  const float zc = narrow(x[4].x), gpz0 = narrow(x[4].y), gno = narrow(x[5].x);
-  const float ge1 = narrow(x[2].x), ge2 = narrow(x[2].y);
-  // d c from the screen gradient and the depth term; d opacity
-  const float gcx = fmaf(rr.x, zc, sg[0][0]), gcy = fmaf(rr.y, zc, sg[0][1]);
-  const float gop = gno != 0.f ? gno / rr.w : 0.f;
-  const float grgb[3] = {narrow(x[5].y), narrow(x[6].x), narrow(x[6].y)};
-  const V3<float> gnrm = {narrow(x[9].x), narrow(x[9].y), narrow(x[10].x)};
+  float gJi11 = ga4.x, gJi12 = ga4.y, gJi21 = ga4.z, gJi22 = ga4.w;
+  const float ge1 = gb4.x, ge2 = gb4.y, gcx = gb4.z, gcy = gb4.w, gpz0 = gc4.x, gop = gc4.y;
+  const float grgb[3] = {gc4.z, gc4.w, gd4.x};
+  const V3<float> gnrm = {gd4.y, gd4.z, gd4.w};
   // forward intermediates, FP32
   const float qw0 = P.quat[4 * n], qx0 = P.quat[4 * n + 1], qy0 = P.quat[4 * n + 2], qz0 = P.quat[4 * n + 3];
   const float qn = sqrtf(qw0 * qw0 + qx0 * qx0 + qy0 * qy0 + qz0 * qz0);
@@ -646,15 +622,6 @@ __device__ __forceinline__ void bwd_one(const ParamsDev& P, const CamDev& cam, i
     for (int i = 0; i < K * 3; ++i) fv[i] = f[i];
   }
   if (tc == 0u) return;  // no tile: nothing to add
-  if (screen) {
-#pragma unroll
-    for (int st = 0; st < 3; ++st) {
-      if (st >= n_sets) break;
-      float* s = screen + ((size_t)st * P.n + n) * 2;
-      s[0] += sg[st][0];
-      s[1] += sg[st][1];
-    }
-  }
   float acc[3] = {0.f, 0.f, 0.f};
 #pragma unroll
   for (int k = 0; k < K; ++k)
@@ -734,48 +701,43 @@ __global__ void __launch_bounds__(256, 2) preprocess_bwd_kernel(ParamsDev P, Cam
                                                              const uint32_t* __restrict__ cand,
                                                              const uint32_t* __restrict__ ncand,
                                                              const uint32_t* __restrict__ tcount,
-                                                             const float4* __restrict__ rec, int stride,
-                                                             const double* __restrict__ grow, uint32_t lo,
-                                                             uint32_t rows, int n_sets, float* __restrict__ screen,
+                                                             const float* __restrict__ grec, uint32_t lo, uint32_t rows,
                                                              gs_param_grads G) {
   const int nc = (int)*ncand;
   for (int ci = blockIdx.x * blockDim.x + threadIdx.x; ci < nc; ci += gridDim.x * blockDim.x) {
     const int n = (int)cand[ci];
     const uint32_t row = (uint32_t)n - lo;
     if (row >= rows) continue;
-    bwd_one<DEG, kVec>(P, cam, n, tcount[n], rec, grow + (size_t)row * stride, stride > kRowAll, n_sets, screen, G);
+    bwd_one<DEG, kVec>(P, cam, n, tcount[n], grec + (size_t)row * kGradRec, G);
   }
 }
 
-// Zeroes the candidates' gradient rows, 16 bytes per thread and step.
-__global__ void __launch_bounds__(256) zero_rows_kernel(const uint32_t* __restrict__ cand,
-                                                        const uint32_t* __restrict__ ncand, int stride,
-                                                        double* __restrict__ grow, uint32_t lo, uint32_t rows) {
-  const int half = stride / 2;
-  const int64_t total = (int64_t)*ncand * half;
+// Zeroes the candidates' gradient records, 16 bytes per thread and step.
+__global__ void __launch_bounds__(256) zero_records_kernel(const uint32_t* __restrict__ cand,
+                                                           const uint32_t* __restrict__ ncand,
+                                                           float* __restrict__ grec, uint32_t lo, uint32_t rows) {
+  constexpr int kPieces = kGradRec / 4;
+  const int64_t total = (int64_t)*ncand * kPieces;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = i / half;
-    const uint32_t row = cand[c] - lo;
-    if (row < rows) reinterpret_cast<double2*>(grow + (size_t)row * stride)[i - c * half] = make_double2(0.0, 0.0);
+    const uint32_t row = cand[i / kPieces] - lo;
+    if (row < rows)
+      reinterpret_cast<float4*>(grec)[(size_t)row * kPieces + (size_t)(i % kPieces)] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
 template <int DEG>
 void launch_bwd_deg(const ParamsDev& P, const CamDev& cam, const uint32_t* cand, const uint32_t* ncand,
-                    const uint32_t* tcount, const float4* rec, int stride, const double* grow, uint32_t lo,
-                    uint32_t rows, int n_sets, float* screen, const gs_param_grads& G, unsigned blocks,
-                    cudaStream_t st) {
+                    const uint32_t* tcount, const float* grec, uint32_t lo, uint32_t rows, const gs_param_grads& G,
+                    unsigned blocks, cudaStream_t st) {
   constexpr int K3 = (DEG + 1) * (DEG + 1) * 3;
   const bool vec = K3 % 4 == 0 && ((uintptr_t)P.sh % 16u) == 0 && ((uintptr_t)G.sh % 16u) == 0;
   if constexpr (K3 % 4 == 0) {
     if (vec) {
-      preprocess_bwd_kernel<DEG, true><<<blocks, 256, 0, st>>>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows,
-                                                               n_sets, screen, G);
+      preprocess_bwd_kernel<DEG, true><<<blocks, 256, 0, st>>>(P, cam, cand, ncand, tcount, grec, lo, rows, G);
       return;
     }
   }
-  preprocess_bwd_kernel<DEG, false><<<blocks, 256, 0, st>>>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows,
-                                                            n_sets, screen, G);
+  preprocess_bwd_kernel<DEG, false><<<blocks, 256, 0, st>>>(P, cam, cand, ncand, tcount, grec, lo, rows, G);
 }
 
 }  // namespace
@@ -830,32 +792,29 @@ cudaError_t launch_preprocess(const ParamsDev& P, const CamDev& cam, const SetDe
   return cudaGetLastError();
 }
 
-cudaError_t launch_zero_rows(int64_t n, const uint32_t* cand, const uint32_t* ncand, bool loss_layout, double* grow,
-                             uint32_t lo, uint32_t rows, cudaStream_t st) {
+cudaError_t launch_zero_records(int64_t n, const uint32_t* cand, const uint32_t* ncand, float* grec, uint32_t lo,
+                                uint32_t rows, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  ProfScope ps(kProfPreprocessBwd, st);  // beside the rows' reader: the blend's group is its launches alone
+  ProfScope ps(kProfPreprocessBwd, st);  // beside the records' reader: the blend's group is its launches alone
   count_launch();
-  const int64_t blocks = (n * (grad_row_stride(loss_layout) / 2) + 255) / 256;
-  zero_rows_kernel<<<(unsigned)(blocks < 2432 ? blocks : 2432), 256, 0, st>>>(cand, ncand, grad_row_stride(loss_layout),
-                                                                              grow, lo, rows);
+  const int64_t blocks = (n * (kGradRec / 4) + 255) / 256;
+  zero_records_kernel<<<(unsigned)(blocks < 2432 ? blocks : 2432), 256, 0, st>>>(cand, ncand, grec, lo, rows);
   return cudaGetLastError();
 }
 
 cudaError_t launch_preprocess_bwd(const ParamsDev& P, const CamDev& cam, const uint32_t* cand,
-                                  const uint32_t* ncand, const uint32_t* tcount, const float4* rec,
-                                  bool loss_layout, const double* grow, uint32_t lo, uint32_t rows, int n_sets,
-                                  float* screen, const gs_param_grads& G, cudaStream_t st) {
+                                  const uint32_t* ncand, const uint32_t* tcount, const float* grec, uint32_t lo,
+                                  uint32_t rows, const gs_param_grads& G, cudaStream_t st) {
   if (P.n == 0) return cudaSuccess;
   ProfScope ps(kProfPreprocessBwd, st);
   // candidates are a subset of the surfels: a grid-stride loop over the
   // device-side count, two CTAs per SM
   const unsigned blocks = div_up(P.n, 256) < 304u ? div_up(P.n, 256) : 304u;
-  const int stride = grad_row_stride(loss_layout);
   switch (P.sh_degree) {
-    case 0: launch_bwd_deg<0>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows, n_sets, screen, G, blocks, st); break;
-    case 1: launch_bwd_deg<1>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows, n_sets, screen, G, blocks, st); break;
-    case 2: launch_bwd_deg<2>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows, n_sets, screen, G, blocks, st); break;
-    default: launch_bwd_deg<3>(P, cam, cand, ncand, tcount, rec, stride, grow, lo, rows, n_sets, screen, G, blocks, st); break;
+    case 0: launch_bwd_deg<0>(P, cam, cand, ncand, tcount, grec, lo, rows, G, blocks, st); break;
+    case 1: launch_bwd_deg<1>(P, cam, cand, ncand, tcount, grec, lo, rows, G, blocks, st); break;
+    case 2: launch_bwd_deg<2>(P, cam, cand, ncand, tcount, grec, lo, rows, G, blocks, st); break;
+    default: launch_bwd_deg<3>(P, cam, cand, ncand, tcount, grec, lo, rows, G, blocks, st); break;
   }
   count_launch();
   return cudaGetLastError();
