@@ -254,7 +254,11 @@ typedef struct {
  *  screen_grads: device [n_sets][N][2] or NULL: ADDS, per set, the gradient
  *               of that set's loss with respect to a screen-space translation
  *               of each surfel's opacity footprint (pixels), the view-space
- *               position gradient used by densification (Sec. 3.1, Eq. 2). */
+ *               position gradient used by densification (Sec. 3.1, Eq. 2).
+ * Needs 64 bytes per surfel from the scene's allocator.  When that is refused
+ * it asks for a half, a quarter, ... down to a sixteenth and replays the view
+ * once for each part of the surfels; GS_ERR_OOM, with nothing done, when a
+ * sixteenth is refused too. */
 gs_status gs_backward(gs_scene* scene, gs_frame* frame, const float* const* adj_sets,
                       const uint32_t* plane_masks, int32_t n_sets, const gs_param_grads* grads,
                       float* screen_grads, void* stream);

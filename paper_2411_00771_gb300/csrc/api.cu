@@ -655,11 +655,14 @@ gs_status gs_backward(gs_scene* sc, gs_frame* f, const float* const* adj_sets,
   cudaStream_t st = (cudaStream_t)stream;
   const int n = f->n;
   constexpr size_t rec_bytes = sizeof(float) * kGradRec;
-  // gradient records of all surfels, or of as many as there is memory for: the
-  // replay then runs once for each part of them
+  // gradient records of all surfels, or of as many as there is memory for, a
+  // sixteenth at least: the whole replay runs once for each part of them
+  constexpr int kMaxParts = 16;
+  const int least = n > 0 ? (n + kMaxParts - 1) / kMaxParts : 1;
   int rows = n > 0 ? n : 1;
   float* grec = nullptr;
-  while (!(grec = static_cast<float*>(sc->al.get(rec_bytes * (size_t)rows, st))) && rows > 1) rows = (rows + 1) / 2;
+  while (!(grec = static_cast<float*>(sc->al.get(rec_bytes * (size_t)rows, st))) && rows > least)
+    rows = (rows + 1) / 2 > least ? (rows + 1) / 2 : least;
   if (!grec) return fail(GS_ERR_OOM, "gs_backward: scratch allocation failed");
   cudaError_t e = cudaMemsetAsync(f->counters + 2, 0, 3 * sizeof(unsigned long long), st);
   const SetDev set = to_dev(sc->settings);
