@@ -509,11 +509,11 @@ gs_status gs_contribution(gs_scene* sc, const gs_camera* c, float gamma, float w
   if (!f) return s;
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t n = f->n;
-  // per-view sums and support counts: the caller's arrays (overwritten, zero
-  // outside the candidates) or scratch (zeroed for the candidates only)
-  float* csum = view_sum ? view_sum : f->buf.get<float>(n > 0 ? n : 1, st);
+  // per-view sums in double (scratch, once the lists' is free again) and support
+  // counts (the caller's array or scratch), zeroed for the candidates; the
+  // caller's arrays are overwritten, zero outside the candidates
   uint32_t* ccnt = view_count ? view_count : f->buf.get<uint32_t>(n > 0 ? n : 1, st);
-  if (!csum || !ccnt) {
+  if (!ccnt) {
     gs_frame_release(f, stream);
     return fail(GS_ERR_OOM, "gs_contribution: device allocation failed");
   }
@@ -526,9 +526,13 @@ gs_status gs_contribution(gs_scene* sc, const gs_camera* c, float gamma, float w
   }
   s = build_lists(sc, f, "gs_contribution", st);
   if (s == GS_OK) {
-    const bool zero_cand = !view_sum || !view_count;
+    double* csum = f->buf.get<double>(n > 0 ? n : 1, st);
+    if (!csum) {
+      gs_frame_release(f, stream);
+      return fail(GS_ERR_OOM, "gs_contribution: device allocation failed");
+    }
     e = launch_contribution(f->cam, to_dev(sc->settings), gamma, weight, f->order, f->rec, f->masks, f->vals,
-                            f->ranges, f->cand, f->ncand, n, zero_cand, csum, ccnt, contrib, st);
+                            f->ranges, f->cand, f->ncand, n, csum, ccnt, view_sum, contrib, st);
     if (e != cudaSuccess) s = cuda_fail(e, "gs_contribution");
   }
   gs_frame_release(f, stream);

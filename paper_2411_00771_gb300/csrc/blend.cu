@@ -1290,7 +1290,9 @@ __global__ void __launch_bounds__(kThreads, kMinCtas) blend_bwd_kernel(
 // the pixel's stop.  A blended pair adds alpha^gamma T^(1 - gamma), T the
 // transmittance in front of it.  Per entry a lane group counts its support
 // pixels with ballots, sums its contributions with shuffles and adds both to
-// the surfel's totals.
+// the surfel's totals.  A wide, faint surfel gets an addition from every 4 x 4
+// block of the image, half a million at 4K: in FP32 each would round the same
+// way (an error of a percent there), so the sum is double.
 
 __device__ __forceinline__ float contrib_step(float& T, bool& stopped, bool hit, float alpha, const SetDev& set,
                                               float gamma) {
@@ -1310,7 +1312,7 @@ __device__ __forceinline__ float contrib_step(float& T, bool& stopped, bool hit,
 __global__ void __launch_bounds__(kThreads, 5) blend_contrib_kernel(
     CamDev cam, SetDev set, float gamma, const uint32_t* __restrict__ order,
     const float4* __restrict__ rec, const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals,
-    const int2* __restrict__ ranges, float* __restrict__ csum, uint32_t* __restrict__ ccnt) {
+    const int2* __restrict__ ranges, double* __restrict__ csum, uint32_t* __restrict__ ccnt) {
   __shared__ WarpSmem sh[kThreads / 32];
   const int tile = order ? (int)order[blockIdx.x] : (int)blockIdx.x;
   const int tx0 = (tile % cam.tiles_x) * kTile, ty0 = (tile / cam.tiles_x) * kTile;
@@ -1343,7 +1345,7 @@ __global__ void __launch_bounds__(kThreads, 5) blend_contrib_kernel(
     if (cnt != 0u && (lane & 7) == 0) {
       const uint32_t sid = at16(sm.meta, k).y;
       atomicAdd(&ccnt[sid], cnt);
-      if (c != 0.f) atomicAdd(&csum[sid], c);
+      if (c != 0.f) atomicAdd(&csum[sid], (double)c);
     }
   });
 }
@@ -1429,7 +1431,7 @@ cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_
 
 cudaError_t launch_blend_contrib(const CamDev& cam, const SetDev& set, float gamma, const uint32_t* order,
                                  const float4* rec, const uint16_t* masks, const uint32_t* vals,
-                                 const int2* ranges, float* csum, uint32_t* ccnt, cudaStream_t st) {
+                                 const int2* ranges, double* csum, uint32_t* ccnt, cudaStream_t st) {
   const unsigned grid = (unsigned)cam.tiles_x * (unsigned)cam.tiles_y;
   ProfScope ps(kProfContrib, st);
   blend_contrib_kernel<<<grid, kThreads, 0, st>>>(cam, set, gamma, order, rec, masks, vals, ranges, csum,

@@ -16,23 +16,28 @@ namespace {
 constexpr int kThreads = 256;
 
 __global__ void contrib_zero_kernel(const uint32_t* __restrict__ cand, const uint32_t* __restrict__ ncand,
-                                    float* __restrict__ csum, uint32_t* __restrict__ ccnt) {
+                                    double* __restrict__ csum, uint32_t* __restrict__ ccnt) {
   const uint32_t nc = *ncand;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
     const uint32_t n = cand[i];
-    csum[n] = 0.f;
+    csum[n] = 0.0;
     ccnt[n] = 0u;
   }
 }
 
+// The sums rounded to FP32 once: the view's own (view_sum, may be null) and
+// weight times their mean over the support added to contrib (may be null).
 __global__ void contrib_finalize_kernel(const uint32_t* __restrict__ cand, const uint32_t* __restrict__ ncand,
-                                        const float* __restrict__ csum, const uint32_t* __restrict__ ccnt,
-                                        float weight, float* __restrict__ contrib) {
+                                        const double* __restrict__ csum, const uint32_t* __restrict__ ccnt,
+                                        float weight, float* __restrict__ view_sum, float* __restrict__ contrib) {
   const uint32_t nc = *ncand;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
     const uint32_t n = cand[i];
     const uint32_t c = ccnt[n];
-    if (c != 0u) contrib[n] += weight * (csum[n] / (float)c);
+    if (c == 0u) continue;
+    const float s = (float)csum[n];
+    if (view_sum) view_sum[n] = s;
+    if (contrib) contrib[n] += weight * (s / (float)c);
   }
 }
 
@@ -128,21 +133,19 @@ unsigned grid_for(int64_t n) {
 cudaError_t launch_contribution(const CamDev& cam, const SetDev& set, float gamma, float weight,
                                 const uint32_t* order, const float4* rec, const uint16_t* masks,
                                 const uint32_t* vals, const int2* ranges, const uint32_t* cand,
-                                const uint32_t* ncand, int64_t n, bool zero_cand, float* csum, uint32_t* ccnt,
+                                const uint32_t* ncand, int64_t n, double* csum, uint32_t* ccnt, float* view_sum,
                                 float* contrib, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   {
     ProfScope ps(kProfContrib, st);
-    if (zero_cand) {
-      count_launch();
-      contrib_zero_kernel<<<grid_for(n), kThreads, 0, st>>>(cand, ncand, csum, ccnt);
-    }
+    count_launch();
+    contrib_zero_kernel<<<grid_for(n), kThreads, 0, st>>>(cand, ncand, csum, ccnt);
   }
   cudaError_t e = launch_blend_contrib(cam, set, gamma, order, rec, masks, vals, ranges, csum, ccnt, st);
-  if (e != cudaSuccess || !contrib) return e;
+  if (e != cudaSuccess || (!view_sum && !contrib)) return e;
   ProfScope ps(kProfContrib, st);
   count_launch();
-  contrib_finalize_kernel<<<grid_for(n), kThreads, 0, st>>>(cand, ncand, csum, ccnt, weight, contrib);
+  contrib_finalize_kernel<<<grid_for(n), kThreads, 0, st>>>(cand, ncand, csum, ccnt, weight, view_sum, contrib);
   return cudaGetLastError();
 }
 

@@ -326,14 +326,14 @@ cudaError_t launch_blend_bwd(const CamDev& cam, const SetDev& set, const uint32_
 // (csum, ccnt: [N], accumulated).
 cudaError_t launch_blend_contrib(const CamDev& cam, const SetDev& set, float gamma, const uint32_t* order,
                                  const float4* rec, const uint16_t* masks, const uint32_t* vals,
-                                 const int2* ranges, float* csum, uint32_t* ccnt, cudaStream_t st);
-// Zero the candidates' csum/ccnt (when zero_cand), run the contribution blend
-// and add weight * csum / ccnt to contrib[n] for the candidates (contrib may
-// be null).
+                                 const int2* ranges, double* csum, uint32_t* ccnt, cudaStream_t st);
+// Zero the candidates' csum/ccnt, run the contribution blend, and for the
+// candidates write the sums to view_sum[n] and add weight * csum / ccnt to
+// contrib[n] (either may be null).
 cudaError_t launch_contribution(const CamDev& cam, const SetDev& set, float gamma, float weight,
                                 const uint32_t* order, const float4* rec, const uint16_t* masks,
                                 const uint32_t* vals, const int2* ranges, const uint32_t* cand,
-                                const uint32_t* ncand, int64_t n, bool zero_cand, float* csum, uint32_t* ccnt,
+                                const uint32_t* ncand, int64_t n, double* csum, uint32_t* ccnt, float* view_sum,
                                 float* contrib, cudaStream_t st);
 // Visible frequency of points (Sec. 4 crop volume): a view as the count
 // kernel reads it (world-to-camera rotation row-major, translation,
