@@ -147,25 +147,22 @@ __device__ __forceinline__ Staged stage_entry(const float4* __restrict__ rec, ui
 // group's 4 x 4 pixel block, as a list of indices into the batch: the four
 // groups of a warp walk their own lists side by side, so an entry costs a
 // group nothing where it misses the group's block.
-// sm holds the entries' block masks (bit 4 w + g); entry e is listed for a
-// group only below the group's limit.  Returns the length of the caller's
-// group's list.
+// sm holds the entries' block masks (bit 4 w + g).  Returns the length of the
+// caller's group's list.
 template <int NB>
 constexpr int kListStride = NB + 4;  // padded: a walk reads one index past its list
 template <int NB>
 __device__ __forceinline__ int group_lists(const uint16_t* sm, int nb, int warp, int lane,
-                                           uint8_t (*list)[kListStride<NB>], int limit = NB) {
+                                           uint8_t (*list)[kListStride<NB>]) {
   const uint32_t lt = (1u << lane) - 1u;
-  int base[4] = {0, 0, 0, 0}, lim[4];
-#pragma unroll
-  for (int g = 0; g < 4; ++g) lim[g] = min(__shfl_sync(0xffffffffu, limit, 8 * g), nb);
+  int base[4] = {0, 0, 0, 0};
 #pragma unroll
   for (int j = 0; j < NB / 32; ++j) {
     const int e = 32 * j + lane;
     const uint32_t m = e < nb ? (uint32_t)sm[e] >> (4 * warp) : 0u;
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-      const bool in = ((m >> g) & 1u) && e < lim[g];
+      const bool in = (m >> g) & 1u;
       const uint32_t b = __ballot_sync(0xffffffffu, in);
       if (in) list[g][base[g] + __popc(b & lt)] = (uint8_t)e;
       base[g] += __popc(b);
@@ -176,93 +173,75 @@ __device__ __forceinline__ int group_lists(const uint16_t* sm, int nb, int warp,
   return g == 0 ? base[0] : (g == 1 ? base[1] : (g == 2 ? base[2] : base[3]));
 }
 
-// One warp's window on its tile's list: the entries that reach its 8 x 8
-// block, staged 32 at a time into the two halves of a ring, and for each of
-// the warp's four lane groups the ring slots of the entries that reach the
-// group's 4 x 4 block, in walking order.
+// One warp's window on its tile's list (the trim contribution): the entries
+// that reach its 8 x 8 block, staged 32 at a time into the two halves of a
+// ring, and for each of the warp's four lane groups the ring slots of the
+// entries that reach the group's 4 x 4 block, in list order.
 constexpr int kHalf = 32;
 constexpr int kRing = 2 * kHalf;
 constexpr int kQueue = kRing;
-constexpr int kNoMore = 1 << 30;
 struct WarpSmem {
   // slot kRing: an entry that no pixel is near, for the groups whose list is used up
-  float4 s0[kRing + 1], s1[kRing + 1], s2[kRing + 1], s3[kRing + 1], s4[kRing + 1], s5[kRing + 1];
-  uint2 meta[kRing + 1];   // list position, surfel
-  uint2 q[kQueue];         // entries found but not yet staged (a ring): position, surfel
-  uint8_t qm[kQueue];      // and their group masks
+  float4 s0[kRing + 1], s1[kRing + 1], s2[kRing + 1], s4[kRing + 1], s5[kRing + 1];
+  uint32_t sid[kRing + 1];  // surfel
+  uint32_t q[kQueue];       // surfels found but not yet staged (a ring)
+  uint8_t qm[kQueue];       // and their group masks
   uint16_t list[4][kRing];  // per group, byte offsets of ring slots (16 x slot; a ring of its own)
 };
+// Element of a staged array at a byte offset that is 16 times its slot.
+__device__ __forceinline__ float4 at16(const float4* a, int k) {
+  return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(a) + k);
+}
 
-// Walks list positions [p0, p1) of a tile (front to back, or back to front
-// when kBack) for one warp.  body(k, i) is called with every lane: k is the
-// offset (16 x ring slot) of the lane's group's next entry and i the number
-// of entries of its list walked so far, this one included; a group whose list
-// is used up for now gets an entry that misses every pixel.  A lane that needs
-// no more entries sets i to kNoMore (or starts with it).  kBack: the group
-// takes only entries below its limit.  Returns the lane's i.
+// Walks the len entries of a tile's list front to back for one warp (its block
+// blk).  body(k) is called with every lane: k is the offset (16 x ring slot) of
+// the lane's group's next entry; a group whose list is used up for now gets an
+// entry that misses every pixel.
 //
 // The warps of a CTA share no data and no barrier: with one staging per CTA
 // and batch, a quarter of the warps' time went to waiting for the slowest
 // warp and for the staging loads.  A group may run ahead of the others by
 // up to one half of the ring, which evens out most of the difference between
 // the groups' lists (the older half is refilled when all groups are past it).
-// Element of a staged array at a byte offset that is 16 times its slot.
-__device__ __forceinline__ float4 at16(const float4* a, int k) {
-  return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(a) + k);
-}
-__device__ __forceinline__ uint2 at16(const uint2* a, int k) {
-  return *reinterpret_cast<const uint2*>(reinterpret_cast<const char*>(a) + k / 2);
-}
-
-template <bool kBack, class Body>
-__device__ __forceinline__ int walk_list(WarpSmem& sm, const float4* __restrict__ rec,
-                                         const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals, int p0,
-                                         int p1, int limit, int tx0, int ty0, int blk, int i, Body body) {
+template <class Body>
+__device__ __forceinline__ void walk_list(WarpSmem& sm, const float4* __restrict__ rec,
+                                          const uint16_t* __restrict__ masks, const uint32_t* __restrict__ vals,
+                                          int len, int tx0, int ty0, int blk, Body body) {
   constexpr unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31, g = lane >> 3;
   const uint32_t lt = (1u << lane) - 1u;
-  int scan = kBack ? p1 : p0, qn = 0, q0 = 0;
+  int scan = 0, qn = 0, q0 = 0;
   uint32_t pm = 0u, pv = 0u;  // the next 32 entries' masks and surfels, loaded ahead
-  auto left = [&] { return kBack ? scan > p0 : scan < p1; };
-  auto at = [&] { return kBack ? scan - 1 - lane : scan + lane; };
   auto load = [&] {
-    const int e = at();
-    const bool in = kBack ? e >= p0 : e < p1;
-    pm = in ? masks[e] : 0u;
-    pv = in ? vals[e] : 0u;
+    const int e = scan + lane;
+    pm = e < len ? masks[e] : 0u;
+    pv = e < len ? vals[e] : 0u;
   };
   load();
   if (lane == 0) {
     sm.s0[kRing] = make_float4(1e15f, 1e15f, 0.f, 0.f);
-    sm.s1[kRing] = sm.s3[kRing] = sm.s4[kRing] = make_float4(0.f, 0.f, 0.f, 0.f);
+    sm.s1[kRing] = sm.s4[kRing] = make_float4(0.f, 0.f, 0.f, 0.f);
     sm.s2[kRing] = make_float4(1.f, 0.f, 0.f, 0.f);
     sm.s5[kRing] = make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, 0.f);
-    sm.meta[kRing] = make_uint2(0x7fffffffu, 0u);
+    sm.sid[kRing] = 0u;
   }
-  // entries staged so far for the lane's group, and for all four groups modulo
-  // the ring (one byte each); mid: those of the older half
-  int end = 0, h = 0;
+  // entries staged so far for the lane's group, those of them it has walked, and
+  // for all four groups the staged ones modulo the ring (one byte each)
+  int end = 0, i = 0, h = 0;
   uint32_t cnt = 0u;
   for (;;) {
-    int mid = end;
-    const bool fill = qn > 0 || left();
+    int mid = end;  // the older half's
+    const bool fill = qn > 0 || scan < len;
     if (fill) {
       __syncwarp();  // every lane is done with the older half
-      while (qn < kHalf && left()) {
-        const int e = at();
-        uint32_t m = (pm >> (4 * blk)) & 15u;
-        const uint32_t v = pv;
-        if constexpr (kBack) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (e >= __shfl_sync(kFull, limit, 8 * j)) m &= ~(1u << j);
-        }
-        scan += kBack ? -32 : 32;
-        if (left()) load();
+      while (qn < kHalf && scan < len) {
+        const uint32_t m = (pm >> (4 * blk)) & 15u, v = pv;
+        scan += 32;
+        if (scan < len) load();
         const uint32_t b = __ballot_sync(kFull, m != 0u);
         if (m != 0u) {
           const int slot = (q0 + qn + __popc(b & lt)) & (kQueue - 1);
-          sm.q[slot] = make_uint2((uint32_t)e, v);
+          sm.q[slot] = v;
           sm.qm[slot] = (uint8_t)m;
         }
         qn += __popc(b);
@@ -272,16 +251,15 @@ __device__ __forceinline__ int walk_list(WarpSmem& sm, const float4* __restrict_
       const int slot = h * kHalf + lane;
       uint32_t m = 0u;
       if (lane < nb) {
-        const uint2 x = sm.q[(q0 + lane) & (kQueue - 1)];
+        const uint32_t v = sm.q[(q0 + lane) & (kQueue - 1)];
         m = sm.qm[(q0 + lane) & (kQueue - 1)];
-        const Staged e = stage_entry(rec, x.y, tx0, ty0);
+        const Staged e = stage_entry(rec, v, tx0, ty0);
         sm.s0[slot] = e.s0;
         sm.s1[slot] = e.s1;
         sm.s2[slot] = e.s2;
-        sm.s3[slot] = e.s3;
         sm.s4[slot] = e.s4;
         sm.s5[slot] = e.s5;
-        sm.meta[slot] = make_uint2(x.x, x.y);
+        sm.sid[slot] = v;
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -305,11 +283,10 @@ __device__ __forceinline__ int walk_list(WarpSmem& sm, const float4* __restrict_
         k = sm.list[g][i & (kRing - 1)];
         ++i;
       }
-      body(k, i);
+      body(k);
     }
-    if (!__any_sync(kFull, i < (fill ? kNoMore : end))) break;
+    if (!fill) break;
   }
-  return i;
 }
 
 // One entry against a thread's two pixels A and B (one column, kRowStep rows
@@ -1327,8 +1304,7 @@ __global__ void __launch_bounds__(kThreads, 5) blend_contrib_kernel(
   float TA = 1.f, TB = 1.f;
   bool stA = !inA, stB = !inB;
   WarpSmem& sm = sh[blk];
-  walk_list<false>(sm, rec, masks + rg.x, vals + rg.x, 0, rg.y - rg.x, 0, tx0, ty0, blk, 0,
-                   [&](int k, int&) {
+  walk_list(sm, rec, masks + rg.x, vals + rg.x, rg.y - rg.x, tx0, ty0, blk, [&](int k) {
     const Pair q = eval_pair(lx, lb, off, at16(sm.s0, k), at16(sm.s1, k), at16(sm.s4, k), at16(sm.s5, k), at16(sm.s2, k).y,
                              set);
     const unsigned ba = __ballot_sync(0xffffffffu, inA & (q.rho.x <= set.rho_max));
@@ -1343,7 +1319,7 @@ __global__ void __launch_bounds__(kThreads, 5) blend_contrib_kernel(
       for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     }
     if (cnt != 0u && (lane & 7) == 0) {
-      const uint32_t sid = at16(sm.meta, k).y;
+      const uint32_t sid = sm.sid[k / 16];
       atomicAdd(&ccnt[sid], cnt);
       if (c != 0.f) atomicAdd(&csum[sid], (double)c);
     }
