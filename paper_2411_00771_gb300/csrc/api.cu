@@ -256,7 +256,7 @@ gs_frame* new_frame(gs_scene* sc, const gs_camera* c, const float* out, const ch
 // tile lists, ranges and the tiles' launch order, into frame f.  Reads the
 // 4-byte instance count back once.  On failure f keeps what it allocated
 // (the caller releases it).
-gs_status build_lists(gs_scene* sc, gs_frame* f, const char* who, cudaStream_t st) {
+gs_status build_lists(gs_scene* sc, gs_frame* f, const char* who, bool keep, cudaStream_t st) {
   const CamDev& cam = f->cam;
   const int ntiles = cam.tiles_x * cam.tiles_y;
   const int64_t n = f->n;
@@ -322,8 +322,16 @@ gs_status build_lists(gs_scene* sc, gs_frame* f, const char* who, cudaStream_t s
   GS_CKC(radix_sort_pairs(keys, vals, keys2, vals2, K, bits_for(ntiles), ktmp, &tk, &tv, st));
   f->vals = tv;
   f->buf.release(tv == vals ? vals2 : vals, st);
-  // the key buffer that the sort left free holds the block masks
-  f->masks = reinterpret_cast<uint16_t*>(tk == keys ? keys2 : keys);
+  // the key buffer that the sort left free holds the block masks; a frame that
+  // is kept has them in a buffer of their own size, half of a key each
+  uint32_t* const spare = tk == keys ? keys2 : keys;
+  if (keep) {
+    f->buf.release(spare, st);
+    f->masks = f->buf.get<uint16_t>(K > 0 ? K : 1, st);
+    if (!f->masks) return failed(fail(GS_ERR_OOM, std::string(who) + ": device allocation failed (tile lists)"));
+  } else {
+    f->masks = reinterpret_cast<uint16_t*>(spare);
+  }
   GS_CKC(launch_ranges(tk, tv, K, f->ranges, ntiles, f->geom, rf, cam, f->masks, st));
   f->buf.release(tk, st);
   if (tile_order_supported(ntiles)) GS_CKC(launch_tile_order(f->ranges, ntiles, f->order, st));
@@ -490,7 +498,7 @@ gs_status gs_render(gs_scene* sc, const gs_camera* c, float* out, int32_t* n_con
       return fail(GS_ERR_OOM, "gs_render: device allocation failed");
     }
   }
-  s = build_lists(sc, f, "gs_render", st);
+  s = build_lists(sc, f, "gs_render", saved != nullptr, st);
   if (s == GS_OK) s = blend_forward(sc, f, out, n_contrib, st);
   if (s != GS_OK || !saved) {
     gs_frame_release(f, stream);
@@ -524,7 +532,7 @@ gs_status gs_contribution(gs_scene* sc, const gs_camera* c, float gamma, float w
     gs_frame_release(f, stream);
     return cuda_fail(e, "gs_contribution");
   }
-  s = build_lists(sc, f, "gs_contribution", st);
+  s = build_lists(sc, f, "gs_contribution", false, st);
   if (s == GS_OK) {
     double* csum = f->buf.get<double>(n > 0 ? n : 1, st);
     if (!csum) {
