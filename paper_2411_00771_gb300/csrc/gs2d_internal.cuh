@@ -405,6 +405,17 @@ cudaError_t launch_elongation(int64_t n, const float* scale, float eta_thr, uint
 
 inline unsigned div_up(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
+// SMs of the device in use at the first call.
+inline unsigned sm_count() {
+  static const unsigned sms = [] {
+    int dev = 0, n = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return (unsigned)n;
+  }();
+  return sms;
+}
+
 // Launch accounting and optional per-kernel CUDA-event timing (diagnostics:
 // gs_kernel_launches, gs_profile_enable, gs_profile_read).
 enum ProfId {

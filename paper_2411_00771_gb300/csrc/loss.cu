@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kThr, 3) ssim_fwd_kernel(int W, int H, const f
     for (int i = 0; i < kHS; ++i) h3[r][c0 + i] = p[i];
   }
   __syncthreads();
-  // vertical pass: item = (column, 4-row segment), then the SSIM terms
+  // vertical pass: item = (column, kVS rows), then the SSIM terms
   const int col = t % kTW, r0 = (t / kTW) * kVS;
   float2 m1[kVS], m2[kVS];
   float m3[kVS];

@@ -757,12 +757,7 @@ cudaError_t launch_preprocess(const ParamsDev& P, const CamDev& cam, const SetDe
   compact_kernel<<<div_up(P.n, 256), 256, 0, st>>>(flags, dkey, P.n, cand);
   // candidates are a subset of the surfels; a grid-stride loop over the
   // device-side count, as many CTAs per SM as its registers allow
-  static const unsigned resident = [] {
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return (unsigned)kMainCtas * (unsigned)sms;
-  }();
+  const unsigned resident = (unsigned)kMainCtas * sm_count();
   const unsigned blocks = div_up(P.n, kMainThreads) < resident ? div_up(P.n, kMainThreads) : resident;
 #define GS_MAIN(D, HALF, PIECE) \
   launch_main<D, HALF, PIECE>(P, cam, set, cand, ncand, rec, rect, tcount, dkey, idx, geom, blocks, st)

@@ -848,12 +848,7 @@ cudaError_t launch_emit(const uint32_t* order, const uint32_t* offs, const uint3
   count_launch();
   // at most two waves (the count of candidates is on the device; the bound n
   // is usually several times larger)
-  static const unsigned resident = [] {
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return 8u * (unsigned)sms;
-  }();
+  const unsigned resident = 8u * sm_count();
   const unsigned blocks = div_up(n, 256) < resident ? div_up(n, 256) : resident;
   if (masks_in_keys(cam))
     emit_kernel<true><<<blocks, 256, 0, st>>>(order, offs, counts, rect, geom, rf, n, n_dev, cam.tiles_x, keys, vals);

@@ -787,7 +787,7 @@ cudaError_t launch_vq_accum(const VqBufs& b, int m, int C, const uint16_t* cb, i
     if (e != cudaSuccess) return e;
   }
   if (m == 0) return cudaSuccess;
-  const unsigned steps = div_up(m, kAccumRows), blocks = steps < 8u * 152u ? steps : 8u * 152u;
+  const unsigned steps = div_up(m, kAccumRows), most = 8u * sm_count(), blocks = steps < most ? steps : most;
   unsigned long long* const sums = with_sums ? b.sums : nullptr;
   unsigned int* const cnt = with_sums ? b.cnt : nullptr;
 #define GS_ACCUM(CC, E) \
