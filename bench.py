@@ -122,8 +122,8 @@ def measured_peak(key):
 # DRAM bytes (read + write) of one blend_bwd launch on this workload, from one
 # ncu capture (dram__bytes_read.sum + dram__bytes_write.sum, one pass, the
 # full-size view); valid only for the kernel sources it was taken on.
-BLEND_BWD_TRAFFIC = {"bytes": 242747904 + 48148992,
-                     "sources_sha256": "f79e75ab42e91d4da9d57bde8b192e2b0f367752923f11da84cb48181b82bc92"}
+BLEND_BWD_TRAFFIC = {"bytes": 151059456 + 8488960,
+                     "sources_sha256": "eb5dc449a025548f6666aff9196b41f2945a191441653301fe1ca6aa3f9ca31f"}
 
 
 def blend_sources_sha256():

@@ -28,8 +28,8 @@
 // gradient's root mean square (seen in a third of the training steps of 4M
 // surfels).  So the pairs' terms and the levels of the sum stay as they are,
 // although lane groups of eight that walk their own lists and add their sums
-// to the surfel's row in double took 768 instead of 1050 us (1M-surfel 1600 x
-// 900 view) and 4930 instead of 8420 (the four backwards of the training step).
+// to the surfel's row in double took 768 instead of 1117 us (1M-surfel 1600 x
+// 900 view) and 4930 instead of 8430 (the four backwards of the training step).
 //
 // All are bound by instruction issue, so the time is (group, entry) or (warp,
 // entry) steps times instructions per step.  With one list per warp (8 x 8
@@ -41,6 +41,7 @@
 //   one list per warp, scalar FP32          501  1148
 //   one list per group                      335   690
 //   packed FP32                             294   583
+//   low part in the rows' order             300   586
 #include <math.h>
 
 #include "gs2d_internal.cuh"

@@ -11,7 +11,7 @@
 // edge-on disks are accurate to FP32 rounding; the record the blends read is
 // FP32 with c split into two floats.
 //
-// Backward: chains the per-surfel gradient row of the blend backward (d Ji,
+// Backward: chains the per-surfel gradient record of the blend backward (d Ji,
 // d e, d c, d p_z, d opacity, d rgb, d normal) to the parameters, in FP32,
 // recomputing the forward intermediates.
 #include <math.h>
@@ -516,7 +516,7 @@ cudaError_t launch_main(const ParamsDev& P, const CamDev& cam, const SetDev& set
 // d c, d p_z, d opacity, d rgb, d normal) back to mu, q, s, o and SH,
 // accumulated into G.  kVec: SH rows and gradient rows are float4-aligned.
 // Every load that does not depend on the computation (the surfel's tile
-// count tc, its gradient row, parameters and the current values of the
+// count tc, its gradient record, parameters and the current values of the
 // small gradient arrays) is issued before the first use, so that a surfel
 // costs two memory round trips (these loads, then the SH gradient row) and
 // not one per dependent access.  The gradient arrays must not overlap one
